@@ -19,9 +19,9 @@
 //     loads per row (x-4 .. x-1 and x+4 .. x+7 cover any R <= 4).  Pairs of cells use Blackwell's packed FP32x2 FMA/ADD.
 //   * Stores are one 16-byte vector per row.  Periodic images (Eq. 2) cost one predicated
 //     vector store on the two x-face lanes (XVEC: nx a multiple of 4, the 4th element lands in
-//     the row padding) or per-cell scalar stores otherwise; y- and z-images are behind one
-//     test that is uniform per warp row and per plane.  Tiles that overhang the interior
-//     store element-wise through an out-of-line path.
+//     the row padding) or per-cell predicated stores otherwise; y- and z-images are behind one
+//     test that is uniform per warp row and per plane.  The lane that straddles the x face of an
+//     extent that 4 does not divide stores its cells under predicates.
 //   * Consecutive steps are launched with programmatic dependent launch: a step's CTAs set up
 //     their barriers while the previous step drains, then wait for it before the first load.
 //   * Waits are bounded (globaltimer); on expiry the CTA records ERR_TIMEOUT, drains its
@@ -68,15 +68,6 @@ __device__ __forceinline__ void queue_period(F &f, int m, std::integer_sequence<
 
 __device__ __forceinline__ float4 lds4(const float *p) { return *reinterpret_cast<const float4 *>(p); }
 __device__ __forceinline__ void stg4(float *p, const float4 v) { *reinterpret_cast<float4 *>(p) = v; }
-
-// Element-wise store of a (possibly overhanging) group of 4 cells with all periodic images.
-__device__ __noinline__ void store4_bounded(float *out, const Geom &g, int r, int images, int x, int y, int z,
-                                           float4 v) {
-    const float e[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-    for (int u = 0; u < 4; ++u)
-        if (x + u < g.n[0] && y < g.n[1]) store_with_images(out, g, r, images != 0, x + u, y, z, e[u]);
-}
 
 // One xy-tile of one z-chunk.  `map` may point at a __grid_constant__ parameter or at a
 // descriptor in global memory (batched launches).  Returns false if a bounded wait expired.
@@ -140,9 +131,14 @@ __device__ __forceinline__ bool heat32_tile(const CUtensorMap *map, float *__res
     if (!bad && threadIdx.x == 0)
         for (; issued < NSLOT + R && issued < nplanes; ++issued) issue(issued);
 
-    // Store targets.  x-images: lanes whose cells lie within 4 (XVEC) or R of an x face.
-    const bool full_tile = x + 4 <= nx && yb + RY <= ny;
-    int xs = 0, xmask = 0;
+    // Store targets.  nv of the thread's 4 cells lie in the interior: 4 everywhere when nx is a
+    // multiple of 4, fewer in the one lane per row that straddles the x face otherwise, 0 past it.
+    // That lane stores its cells one by one under predicates; nothing leaves the common path, so
+    // an extent that no tile divides costs what its tiles cost (301 x 187 x 250, 20 steps: 2.47 ms
+    // with an out-of-line element-wise path for every overhanging thread, 1.27 ms like this).
+    // x-images: lanes whose cells lie within 4 (XVEC) or R of an x face.
+    const int nv = min(max(nx - x, 0), 4);
+    int xs = 0, mlo = 0, mhi = 0;  // XVEC: shift of the vector image; else cells with an image at +nx / -nx
     int ys[RY];
 #pragma unroll
     for (int r = 0; r < RY; ++r) ys[r] = 0;
@@ -152,26 +148,31 @@ __device__ __forceinline__ bool heat32_tile(const CUtensorMap *map, float *__res
         } else {
 #pragma unroll
             for (int u = 0; u < 4; ++u) {
-                if (x + u < R) { xmask |= 1 << u; xs = nx; }
-                else if (x + u >= nx - R && x + u < nx) { xmask |= 1 << u; xs = -nx; }
+                if (x + u < R) mlo |= 1 << u;
+                else if (x + u >= nx - R && x + u < nx) mhi |= 1 << u;
             }
         }
 #pragma unroll
         for (int r = 0; r < RY; ++r) ys[r] = (yb + r < R) ? ny : (yb + r >= ny - R ? -ny : 0);
     }
-    const bool xi = XVEC ? xs != 0 : xmask != 0;
     const int pitch_y = (int)g.pad[0];
     const int64_t pitch_z = g.pad[0] * g.pad[1];
     float *optr = out + g.idx(x, yb, zc0);
+    auto put_masked = [](float *p, const float4 v, int mask) {
+        if (mask & 1) p[0] = v.x;
+        if (mask & 2) p[1] = v.y;
+        if (mask & 4) p[2] = v.z;
+        if (mask & 8) p[3] = v.w;
+    };
     auto put = [&](float *p, const float4 v) {  // one row of 4 cells and its x-image
-        stg4(p, v);
         if (XVEC) {
-            if (xi) stg4(p + xs, v);
-        } else if (xi) {
-            if (xmask & 1) p[xs] = v.x;
-            if (xmask & 2) p[1 + xs] = v.y;
-            if (xmask & 4) p[2 + xs] = v.z;
-            if (xmask & 8) p[3 + xs] = v.w;
+            stg4(p, v);
+            if (xs) stg4(p + xs, v);
+        } else {
+            if (nv == 4) stg4(p, v);
+            else put_masked(p, v, (1 << nv) - 1);
+            if (mlo) put_masked(p + nx, v, mlo);
+            if (mhi) put_masked(p - nx, v, mhi);
         }
     };
 
@@ -248,9 +249,10 @@ __device__ __forceinline__ bool heat32_tile(const CUtensorMap *map, float *__res
                     const int z = zc0 + m + b;
                     const int zs = images ? (z < R ? nz : (z >= nz - R ? -nz : 0)) : 0;
                     float *op = optr + b * pitch_z;
-                    if (full_tile) {
+                    if (nv) {
 #pragma unroll
                         for (int r = 0; r < RY; ++r) {
+                            if (yb + r >= ny) break;  // uniform per warp row
                             float *p = op + r * pitch_y;
                             put(p, res[r]);
                             if (ys[r] | zs) {  // y- and z-images: uniform per warp row / per plane
@@ -260,9 +262,6 @@ __device__ __forceinline__ bool heat32_tile(const CUtensorMap *map, float *__res
                                 if (ys[r] && zs) put(p + dy + dz, res[r]);
                             }
                         }
-                    } else {
-#pragma unroll
-                        for (int r = 0; r < RY; ++r) store4_bounded(out, g, R, images, x, yb + r, z, res[r]);
                     }
                 }
             }
