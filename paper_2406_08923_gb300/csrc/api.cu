@@ -470,6 +470,7 @@ stencil_status stencil_create(int ndim, const int64_t dims[3], int radius, const
                 for (int i = 0; i < radius; ++i) p->dcoef.ga[a][i] = s * c2[i + 1] / (h[a] * h[a]);
             }
             p->dcoef.g0 = g0;
+            p->dcoef.fx = ndim == 3 && storage == STENCIL_F64 && diffusion_fx_fits(p->dcoef);
             if (ndim == 1) {  // 1D: the folded step is the cross-correlation of Eq. 3 with these weights
                 for (int j = -radius; j <= radius; ++j) {
                     const double w = j == 0 ? g0 : p->dcoef.ga[0][std::abs(j) - 1];
@@ -634,7 +635,7 @@ static stencil_status run_pass(stencil_t p, void *const *src, void *const *dst, 
     if (p->kind == STENCIL_DIFFUSION) {
         int box[3];
         if (p->ndim == 2) diffusion2d_box(storage_code(p->storage), p->radius, box);
-        else diffusion_box(storage_code(p->storage), p->radius, p->variant, box);
+        else diffusion_box(storage_code(p->storage), p->radius, p->variant, p->dcoef.fx, box);
         CUtensorMap m;
         stencil_status st = tma_map(p, src[0], box, &m);
         if (st != STENCIL_OK) return st;
@@ -642,7 +643,7 @@ static stencil_status run_pass(stencil_t p, void *const *src, void *const *dst, 
             CK(p, launch_diffusion2d(storage_code(p->storage), &m, dst[0], g, p->dcoef, periodic, p->err, s),
                "diffusion (2D) launch");
         else
-            CK(p, launch_diffusion(storage_code(p->storage), &m, dst[0], g, p->dcoef, p->bc != STENCIL_BC_CALLER,
+            CK(p, launch_diffusion(storage_code(p->storage), &m, src[0], dst[0], g, p->dcoef, p->bc != STENCIL_BC_CALLER,
                                    p->err, s, p->variant, p->zmode),
                "diffusion launch");
         return STENCIL_OK;
@@ -691,7 +692,7 @@ static stencil_status step_persistent(stencil_t p, void *const *fin, void *const
         CK(p, launch_halo_fill(p->geom, p->radius, p->esize, ptrs(fin, 1), 1, s, p->bc == STENCIL_BC_PERIODIC),
            "halo_fill launch");
     int box[3];
-    diffusion_box(dt, p->radius, p->variant, box);
+    diffusion_box(dt, p->radius, p->variant, p->dcoef.fx, box);
     CUtensorMap maps[3];
     const void *bufs[3] = {fin[0], p->tmp[0], fout[0]};
     for (int i = 0; i < 3; ++i) {

@@ -446,19 +446,14 @@ static cudaError_t run(const CUtensorMap *map, void *out, const Geom &g, const D
                       err);
 }
 
-// Variant table: (VP pairs per row, BY warps, RY rows, ZB planes, NSLOT, packed FP32x2).  The
-// autotuner times each on the problem and keeps the fastest.  Radius 3 (the 6th-order step)
-// carries the tuned set; the other radii of the sweep use its first shape.
-#define DIFF_VARIANTS_F64(X) \
-    X(1, 8, 1, 2, 8, false)  \
-    X(1, 4, 1, 2, 8, false)  \
-    X(1, 8, 1, 1, 8, false)  \
-    X(1, 4, 2, 2, 8, false)
-#define DIFF_VARIANTS_F64_OTHER(X) X(1, 8, 1, 2, 8, false)
-static const char *F64_NAMES[] = {"vx2_by8_ry1_zb2_s8", "vx2_by4_ry1_zb2_s8", "vx2_by8_ry1_zb1_s8",
-                                  "vx2_by4_ry2_zb2_s8"};
-static const char *F64_NAMES_OTHER[] = {"?", "f64_r1_vx2_by8_ry1_zb2_s8", "f64_r2_vx2_by8_ry1_zb2_s8", "?",
-                                        "f64_r4_vx2_by8_ry1_zb2_s8"};
+// The shape of the FP64-pipe kernel: (VP pairs per row, BY warps, RY rows, ZB planes, NSLOT, packed
+// FP32x2).  It serves plans whose weights do not fit the fixed-point kernel of diffusion_fx.cu
+// (not finite, or the signs of a backward or far from stable step); every other FP64 plan runs that one, whose launch
+// shapes the variants of radius 3 name.
+#define DIFF_VARIANT_F64(X) X(1, 8, 1, 2, 8, false)
+static const char *F64_NAMES[] = {"fx64x16_zb1_s16", "fx64x16_zb2_s16", "fx64x16_zb4_s16", "fx64x16_zb3_s16"};
+static const char *F64_NAMES_OTHER[] = {"?", "f64_r1_fx64x16_zb1_s16", "f64_r2_fx64x16_zb1_s16", "?",
+                                        "f64_r4_fx64x16_zb1_s16"};
 
 int diffusion_num_variants(int dtype, int r) {
     if (dtype != 1) return diffusion_f32_num_variants(r);
@@ -471,47 +466,34 @@ const char *diffusion_variant_name(int dtype, int r, int v) {
     return r == 3 ? F64_NAMES[v] : F64_NAMES_OTHER[r];
 }
 
-void diffusion_box(int dtype, int r, int v, int box[3]) {
+void diffusion_box(int dtype, int r, int v, bool fx, int box[3]) {
     if (dtype != 1) return diffusion_f32_box(r, v, box);
-    int i = 0;
-    auto put = [&](int vp, int by, int ry) {
-        if (i++ == v) { box[0] = 64 * vp + 8; box[1] = by * ry + 2 * r; box[2] = 1; }
-    };
-#define X(VP, BY, RY, ZB, NS, PK) put(VP, BY, RY);
-    if (r == 3) {
-        DIFF_VARIANTS_F64(X)
-    } else {
-        DIFF_VARIANTS_F64_OTHER(X)
-    }
+    if (fx) return diffusion_fx_box(r, box);
+#define X(VP, BY, RY, ZB, NS, PK) box[0] = 64 * VP + 8, box[1] = BY * RY + 2 * r, box[2] = 1;
+    DIFF_VARIANT_F64(X)
 #undef X
 }
 
 template <int R>
-static cudaError_t dispatch_f64(int variant, const CUtensorMap *map, void *out, const Geom &g, const DiffCoef &c,
-                                bool images, unsigned *err, cudaStream_t s, int zmode) {
-    using T = double;
-    int i = 0;
-    cudaError_t res = cudaErrorInvalidValue;
-#define X(VP, BY, RY, ZB, NS, PK) \
-    if (i++ == variant) res = run<T, VP, BY, RY, ZB, NS, PK, R>(map, out, g, c, images, err, s, zmode);
-    if constexpr (R == 3) {
-        DIFF_VARIANTS_F64(X)
-    } else {
-        DIFF_VARIANTS_F64_OTHER(X)
-    }
+static cudaError_t dispatch_f64(const CUtensorMap *map, void *out, const Geom &g, const DiffCoef &c, bool images,
+                                unsigned *err, cudaStream_t s, int zmode) {
+#define X(VP, BY, RY, ZB, NS, PK) return run<double, VP, BY, RY, ZB, NS, PK, R>(map, out, g, c, images, err, s, zmode);
+    DIFF_VARIANT_F64(X)
 #undef X
-    return res;
 }
 
-cudaError_t launch_diffusion(int dtype, const CUtensorMap *map, void *out, const Geom &g, const DiffCoef &c,
-                             bool images, unsigned *err, cudaStream_t s, int variant, int zmode) {
+cudaError_t launch_diffusion(int dtype, const CUtensorMap *map, const void *in, void *out, const Geom &g,
+                             const DiffCoef &c, bool images, unsigned *err, cudaStream_t s, int variant, int zmode) {
     if (dtype == 2) return launch_diffusion_f32(map, static_cast<float *>(out), g, c, images, err, s, variant, zmode);
-    if (dtype != 1) return cudaErrorInvalidValue;
+    if (dtype != 1 || variant < 0 || variant >= diffusion_num_variants(1, c.r)) return cudaErrorInvalidValue;
+    if (c.fx)
+        return launch_diffusion_fx(map, static_cast<const double *>(in), static_cast<double *>(out), g, c, images, err,
+                                   s, variant, zmode);
     switch (c.r) {
-    case 1: return dispatch_f64<1>(variant, map, out, g, c, images, err, s, zmode);
-    case 2: return dispatch_f64<2>(variant, map, out, g, c, images, err, s, zmode);
-    case 3: return dispatch_f64<3>(variant, map, out, g, c, images, err, s, zmode);
-    case 4: return dispatch_f64<4>(variant, map, out, g, c, images, err, s, zmode);
+    case 1: return dispatch_f64<1>(map, out, g, c, images, err, s, zmode);
+    case 2: return dispatch_f64<2>(map, out, g, c, images, err, s, zmode);
+    case 3: return dispatch_f64<3>(map, out, g, c, images, err, s, zmode);
+    case 4: return dispatch_f64<4>(map, out, g, c, images, err, s, zmode);
     default: return cudaErrorInvalidValue;
     }
 }

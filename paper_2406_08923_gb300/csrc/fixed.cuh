@@ -1,0 +1,129 @@
+// fixed.cuh -- sums of products of doubles in 64-bit fixed point.
+//
+// GB300's FP64 pipe retires 2 multiply-adds per clock and SM, its integer pipe 64
+// 32 x 32 + 64-bit multiply-adds (mad.wide, measured 63.5 lanes per clock).  Four of those make
+// a 64 x 64-bit product, so a linear stencil of doubles runs up to eight times faster as integers
+// when the values of a neighbourhood share one binary scale.
+//
+// A set of values whose largest magnitude has the (biased) exponent E is held as
+// q = trunc(v 2^(1082 - E)): |q| < 2^60, and 7 bits below a double's last place at the largest
+// value.  Values are stored biased by 2^60, so that they and sums of up to 8 of them are
+// unsigned and split into 32-bit limbs for free.  A weight is an unsigned 57-bit integer
+// 2^28 wh + wl with a sign of its own.  Sums of products are exact in four 64-bit accumulators
+// and are rounded once, to the nearest double, at the end.
+//
+// Accuracy: truncating the values and rounding the sum costs less than 2^-58 of the scale, so an
+// output whose stencil holds a value of at least 2^-6 of the scale is no further from the exact
+// result than a chain of FP64 multiply-adds (2^-53 of its largest term).  Callers check that
+// per output and evaluate the rest in FP64; infinities, NaN and exponents near the ends of the
+// range go the same way.
+#pragma once
+
+#include <cmath>
+
+#include "common.cuh"
+
+namespace stn {
+
+typedef unsigned long long u64;
+typedef unsigned int u32;
+
+constexpr u64 FX_BIAS = 1ull << 60;
+constexpr u32 FX_BIAS_HI = 1u << 28;
+constexpr u32 FX_FLAG_HI = 1u << 22;  // high word of 2^54 = 2^-6 of the scale
+// scales (biased exponents) that convert without meeting denormals or overflow
+constexpr int FX_EMIN = 192, FX_EMAX = 1856;
+// scales a sum uses: what lies below FX_EMIN is more than 63 bits below them
+constexpr int FX_SMIN = FX_EMIN + 64;
+
+// Exponent code of a set of values from the largest high word (sign cleared): 0 only for all
+// zeros, 1 for denormals alone, 2047 for infinities and NaN.
+__device__ __forceinline__ int fx_code(u32 hmax, bool any) { return hmax >> 20 ? (int)(hmax >> 20) : (any ? 1 : 0); }
+
+// v as a biased integer at scale E >= its own exponent.  A zero shifts past the last bit, as
+// E >= FX_EMIN.
+__device__ __forceinline__ u64 fx_from_double(double v, int E) {
+    const u32 hi = (u32)__double2hiint(v), lo = (u32)__double2loint(v);
+    const int d = min(E - (int)((hi >> 20) & 0x7ffu), 63);
+    const u64 m = (((u64)((hi & 0xfffffu) | 0x100000u) << 32) | lo) << 7 >> d;
+    const int s = (int)hi >> 31;
+    const u64 q = ((u64)((u32)(m >> 32) ^ (u32)s) << 32) | ((u32)m ^ (u32)s);
+    return q + (FX_BIAS + (u64)(u32)(-s));
+}
+
+// A biased value (bias a multiple of 2^60) moved to a scale d >= 0 bits coarser, rounded down.
+// shr.u64 takes any shift (0 from 64 on).
+__device__ __forceinline__ u64 fx_shift(u64 v, u64 bias, int d) {
+    u64 a, b;
+    asm("shr.u64 %0, %1, %2;" : "=l"(a) : "l"(v), "r"(d));
+    asm("shr.u64 %0, %1, %2;" : "=l"(b) : "l"(bias), "r"(d));
+    return a + (bias - b);
+}
+
+// Nearest double (ties to even) of the integer v times 2^(ex - 1082), for |v| >= 2^32.
+__device__ __forceinline__ double fx_to_double(long long v, int ex) {
+    const u32 s = (u32)(v >> 63);
+    const u64 a = (u64)((v ^ (v >> 63)) - (v >> 63));
+    const int n = __clz((int)(u32)(a >> 32)) - 1;  // top bit to bit 62
+    const u64 t = a << n;
+    // round to 53 bits: bit 10 is the last place kept
+    const u64 m = (t + (u64)(0x1ffu + (((u32)t >> 10) & 1u))) >> 10;  // the leading one at bit 52, or 53 after a carry
+    // value = m 2^(10 - n) 2^(ex - 1082); the leading one of m adds 1 to the exponent field
+    const u32 f = (u32)(ex - n + 2) << 20;
+    return __hiloint2double((int)(((u32)(m >> 32) + f) | (s & 0x80000000u)), (int)(u32)m);
+}
+// Whether fx_to_double may take v (the rest, at most 2^-28 of the scale, is left to FP64).
+__device__ __forceinline__ bool fx_big(long long v) { return (u64)(v + (1ll << 32)) >= (2ull << 32); }
+
+// Accumulators of sum W s with W = 2^28 wh + wl, s = 2^32 sh + sl (all unsigned).
+struct FxAcc {
+    u64 hh = 0, m1 = 0, m2 = 1ull << 24, ll = 0;  // m2 starts at half of the last place kept
+    __device__ __forceinline__ void mac(u32 wh, u32 wl, u64 s) {
+        const u32 sh = (u32)(s >> 32), sl = (u32)s;
+        hh += (u64)wh * sh;
+        m1 += (u64)wh * sl;
+        m2 += (u64)wl * sh;
+        ll += (u64)wl * sl;
+    }
+    // sum W s / 2^57, rounded, modulo 2^64, less the bias the caller folded into `corr`
+    __device__ __forceinline__ long long result(u64 corr) const {
+        return (long long)((hh << 3) + ((m2 + (m1 >> 4) + (ll >> 32)) >> 25) + corr);
+    }
+};
+
+// One launch's weights: value i times 2^-ew is (2^28 wh + wl) 2^-57; `corr` takes the bias of
+// every sum off the result.  The kernels know the signs: a sum with a negative weight enters as
+// 2^61 mult - s, the biased negative.
+template <int N> struct FxWeights {
+    u32 wh[N], wl[N];
+    int ew;
+    u64 corr;
+};
+
+// mult[i]: how many values sum i adds.  False where fixed point does not apply (a weight is not
+// finite, all are zero, or the exponent is out of range).
+template <int N> inline bool fx_weights(const double *w, const int *mult, FxWeights<N> &o) {
+    double top = 0.0, sum = 0.0;
+    for (int i = 0; i < N; ++i) {
+        if (!std::isfinite(w[i])) return false;
+        top = std::fmax(top, std::fabs(w[i]));
+        sum += mult[i] * std::fabs(w[i]);
+    }
+    if (!(top > 0.0) || !std::isfinite(sum)) return false;
+    int ew = 0;
+    (void)std::frexp(top, &ew);  // top < 2^ew
+    while (std::ldexp(sum, -ew) >= 4.0) ++ew;  // |result| < 2^62
+    if (ew < -100 || ew > 100) return false;
+    o.ew = ew;
+    u64 corr = 0;
+    for (int i = 0; i < N; ++i) {
+        const u64 W = (u64)std::llrint(std::ldexp(std::fabs(w[i]), 57 - ew));
+        o.wh[i] = (u32)(W >> 28);
+        o.wl[i] = (u32)(W & 0xfffffffu);
+        corr += W * (u64)mult[i];
+    }
+    o.corr = 0ull - 8ull * corr;  // 2^60 / 2^57 per unit
+    return true;
+}
+
+}  // namespace stn

@@ -67,14 +67,21 @@ struct DiffCoef {
     double g0;        // centre weight 1 + dt*alpha*sum_axes c0/h^2
     double ga[3][4];  // [axis][a-1] weight of the pair at offset +-a along axis (0 beyond r)
     int r;            // radius 1..4
+    bool fx;          // 3D FP64: the weights fit the fixed-point kernel (diffusion_fx_fits)
 };
 // 3D
-cudaError_t launch_diffusion(int dtype, const CUtensorMap *map_in, void *out, const Geom &g,
+cudaError_t launch_diffusion(int dtype, const CUtensorMap *map_in, const void *in, void *out, const Geom &g,
                              const DiffCoef &c, bool images, unsigned *err, cudaStream_t s,
                              int variant, int zmode = 0);
 int diffusion_num_variants(int dtype, int r);
 const char *diffusion_variant_name(int dtype, int r, int variant);
-void diffusion_box(int dtype, int r, int variant, int box[3]);  // TMA box (x, y, z) of a variant
+// TMA box (x, y, z) of a variant; fx: the plan's weights fit the fixed-point kernel
+void diffusion_box(int dtype, int r, int variant, bool fx, int box[3]);
+// The FP64 kernel in 64-bit fixed point (diffusion_fx.cu).
+bool diffusion_fx_fits(const DiffCoef &c);
+void diffusion_fx_box(int r, int box[3]);
+cudaError_t launch_diffusion_fx(const CUtensorMap *map_in, const double *in, double *out, const Geom &g,
+                                const DiffCoef &c, bool images, unsigned *err, cudaStream_t s, int variant, int zmode);
 // Persistent variants run all nsteps steps of a call in one cooperative launch (persist.cuh):
 // step s reads the field written by step s-1 (maps[0], the input, for s = 0) and writes `out`
 // when nsteps - 1 - s is even, `tmp` otherwise; maps = {in, tmp, out}.  `sync` is a zeroed

@@ -1,0 +1,102 @@
+"""The FP64 3D heat step in 64-bit fixed point (csrc/diffusion_fx.cu, csrc/fixed.cuh): every output,
+also where a field spans hundreds of binary orders, is as close to the exact step as a chain of
+FP64 multiply-adds is, infinities and NaN spread as they do in FP64, and the launch shapes agree
+bit for bit."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2406_08923_gb300 import _lib as L
+
+pytestmark = pytest.mark.gpu
+
+C = {1: (-2.0, 1.0), 2: (-5 / 2, 4 / 3, -1 / 12), 3: (-49 / 18, 3 / 2, -3 / 20, 1 / 90),
+     4: (-205 / 72, 8 / 5, -1 / 5, 8 / 315, -1 / 560)}
+
+
+def _plan(shape, r, h, dt=0.02):
+    par = L.heat_params(shape)
+    par.dx[0], par.dx[1], par.dx[2] = h
+    par.dt, par.alpha = dt, 1.0
+    return L.Plan(3, shape[::-1], r, 1, L.STENCIL_BC_PERIODIC, L.STENCIL_DIFFUSION, L.STENCIL_F64, L.STENCIL_F64,
+                  params=par)
+
+
+def _step(p, f, variant=0):
+    p.set_variant(variant)
+    a, b = p.alloc(), p.alloc()
+    p.upload(a, [f])
+    p.step(a, b, 1)
+    p.sync()
+    return p.download(b)[0], b[0].cpu().numpy()
+
+
+def _reference(f, r, h, dt=0.02):
+    """The folded step and sum |w| |f| per cell, in extended precision."""
+    q = f.astype(np.longdouble)
+    g0 = np.longdouble(1.0 + sum(dt * C[r][0] / (x * x) for x in h))
+    out, mag = g0 * q, abs(g0) * abs(q)
+    for a in range(3):
+        for k in range(1, r + 1):
+            w = np.longdouble(dt * C[r][k] / (h[a] * h[a]))
+            s, t = np.roll(q, k, 2 - a), np.roll(q, -k, 2 - a)
+            out = out + w * (s + t)
+            mag = mag + abs(w) * (abs(s) + abs(t))
+    return out, mag
+
+
+def _fields(shape, seed):
+    rng = np.random.default_rng(seed)
+    z, y, x = np.meshgrid(*[np.arange(n) for n in shape], indexing="ij")
+    smooth = np.sin(0.3 * x + 0.2 * y + 0.25 * z)
+    yield "random", rng.standard_normal(shape)
+    yield "smooth", smooth
+    yield "decay", np.exp(-2.0 * (x + y + z)) * (1 + 0.1 * rng.standard_normal(shape))
+    yield "orders", rng.standard_normal(shape) * 2.0 ** rng.integers(-300, 300, shape)
+    yield "blocks", np.where((x // 5 + y // 4 + z // 3) % 2, 0.0, smooth * 1e-30)
+    yield "edges of the range", smooth * 2.0 ** np.where(z % 7 < 3, -1015.0, 900.0)
+
+
+@pytest.mark.parametrize("r,h", [(1, (0.5, 0.5, 0.5)), (2, (0.4, 0.5, 0.6)), (3, (0.5, 0.5, 0.5)), (3, (0.5, 0.4, 0.7)),
+                                 (4, (0.5, 0.5, 0.5)), (4, (0.45, 0.5, 0.6))])
+@pytest.mark.parametrize("shape", [(9, 17, 65), (21, 33, 130), (40, 16, 64)])
+def test_every_output_is_as_close_as_fp64(cuda_lib, r, h, shape):
+    p = _plan(shape, r, h)
+    for name, f in _fields(shape, 5):
+        got, _ = _step(p, f)
+        ref, mag = _reference(f, r, h)
+        # the weights' own roundings and one rounding per multiply-add of the 1 + 6 r terms
+        bound = (1 + 6 * r + 2) * 2.0 ** -53 * mag + 2.0 ** -1074
+        worst = float(np.max(np.abs(got - ref) / bound))
+        assert worst <= 1.0, (name, worst)
+
+
+def test_infinities_and_nan_spread_as_in_fp64(cuda_lib):
+    shape, r, h = (20, 20, 70), 3, (0.5, 0.5, 0.5)
+    f = np.random.default_rng(3).standard_normal(shape)
+    f[4, 5, 6], f[15, 3, 66], f[10, 12, 30] = np.inf, -np.inf, np.nan
+    p = _plan(shape, r, h)
+    got, _ = _step(p, f)
+    ref, mag = _reference(f, r, h)
+    fine = np.isfinite(ref)
+    assert np.array_equal(np.isnan(got), np.isnan(ref)) and np.array_equal(np.isfinite(got), fine)
+    inf = np.isinf(ref.astype(np.float64))
+    assert np.array_equal(got[inf], ref[inf].astype(np.float64))
+    assert np.all(np.abs(got - ref)[fine] <= 21 * 2.0 ** -53 * mag[fine])
+
+
+@pytest.mark.parametrize("shape", [(7, 7, 7), (37, 40, 66), (50, 33, 131)])
+def test_launch_shapes_agree_bit_for_bit(cuda_lib, shape):
+    p = _plan(shape, 3, (0.5, 0.5, 0.5))
+    f = np.random.default_rng(7).standard_normal(shape) * 2.0 ** np.random.default_rng(8).integers(-6, 3, (shape[0], 1, 1))
+    first = _step(p, f)[0]
+    for v in range(1, p.variant()[1]):
+        assert np.array_equal(_step(p, f, v)[0], first), v
+
+
+def test_weights_of_a_backward_step_run_on_the_fp64_pipe(cuda_lib):
+    shape, r, h = (12, 18, 40), 3, (0.5, 0.5, 0.5)  # dt < 0: the signs the fixed-point kernel has not compiled in
+    p = _plan(shape, r, h, dt=-0.01)
+    f = np.random.default_rng(9).standard_normal(shape)
+    ref, mag = _reference(f, r, h, dt=-0.01)
+    assert np.all(np.abs(_step(p, f)[0] - ref) <= 21 * 2.0 ** -53 * mag)
