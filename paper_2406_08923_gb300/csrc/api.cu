@@ -88,6 +88,8 @@ struct stencil_plan {
     double *red_out = nullptr;
     unsigned *err = nullptr;
     void *wdev = nullptr;  // XCORR of radius > 4: the 2r+1 weights on the device (storage type)
+    void *wfx = nullptr;   // FP64 XCORR of radius > 4: their fixed-point limbs (scale wfx_ew), if they fit
+    int wfx_ew = 0;
     unsigned long long *psync = nullptr;  // sync words of the persistent heat schedule (persist.cuh)
     int64_t psync_words = 0;
     int variant = 0;
@@ -147,6 +149,8 @@ static void free_scratch(stencil_t p) {
     if (p->red_out) cudaFree(p->red_out);
     if (p->err) cudaFree(p->err);
     if (p->wdev) cudaFree(p->wdev);
+    if (p->wfx) cudaFree(p->wfx);
+    p->wfx = nullptr;
     if (p->psync) cudaFree(p->psync);
     p->psync = nullptr;
     p->psync_words = 0;
@@ -540,6 +544,14 @@ stencil_status stencil_create(int ndim, const int64_t dims[3], int radius, const
             e = cudaMemcpy(p->wdev, src, wide_w.size() * p->esize, cudaMemcpyHostToDevice);
             if (e != cudaSuccess) { cuda_fail(nullptr, e, "cudaMemcpy(weights)"); okay = false; }
         }
+        std::vector<int32_t> limbs;
+        if (okay && storage == STENCIL_F64 && fx_wide_weights(wide_w.data(), ncoeffs, limbs, &p->wfx_ew)) {
+            okay = alloc(&p->wfx, limbs.size() * sizeof(int32_t), "cudaMalloc(weight limbs)");
+            if (okay) {
+                e = cudaMemcpy(p->wfx, limbs.data(), limbs.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
+                if (e != cudaSuccess) { cuda_fail(nullptr, e, "cudaMemcpy(weight limbs)"); okay = false; }
+            }
+        }
     }
     if (okay) {
         e = cudaMemset(p->err, 0, sizeof(unsigned));
@@ -605,6 +617,12 @@ static stencil_status run_pass(stencil_t p, void *const *src, void *const *dst, 
     if (p->kind == STENCIL_MAXFILTER) {
         CK(p, launch_maxfilter(storage_code(p->storage), p->radius, src[0], dst[0], g, periodic, periodic, p->err, s),
            "maxfilter launch");
+        return STENCIL_OK;
+    }
+    if (p->kind == STENCIL_XCORR && p->wfx) {
+        CK(p, launch_xcorr_wide_fx(p->radius, static_cast<const double *>(src[0]), static_cast<double *>(dst[0]), g,
+                                   static_cast<const double *>(p->wdev), p->wfx, p->wfx_ew, periodic, periodic, s),
+           "xcorr (wide, fixed point) launch");
         return STENCIL_OK;
     }
     if (p->kind == STENCIL_XCORR && !xcorr_blocked(p)) {

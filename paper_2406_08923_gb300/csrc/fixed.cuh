@@ -72,8 +72,12 @@ __device__ __forceinline__ double fx_to_double(long long v, int ex) {
     const u32 f = (u32)(ex - n + 2) << 20;
     return __hiloint2double((int)(((u32)(m >> 32) + f) | (s & 0x80000000u)), (int)(u32)m);
 }
-// Whether fx_to_double may take v (the rest, at most 2^-28 of the scale, is left to FP64).
+// Whether fx_to_double may take v.
 __device__ __forceinline__ bool fx_big(long long v) { return (u64)(v + (1ll << 32)) >= (2ull << 32); }
+// The same for |v| <= 2^32 (exact), ex from FX_SMIN - 102 on.
+__device__ __forceinline__ double fx_small_to_double(long long v, int ex) {
+    return (double)v * __hiloint2double((ex - 59) << 20, 0);  // 2^(ex - 1082)
+}
 
 // Accumulators of sum W s with W = 2^28 wh + wl, s = 2^32 sh + sl (all unsigned).
 struct FxAcc {

@@ -1,6 +1,8 @@
 // internal.h -- declarations shared between the C-ABI layer (api.cu) and the kernel files.
 #pragma once
 
+#include <vector>
+
 #include "common.cuh"
 #include "persist.cuh"
 
@@ -47,6 +49,12 @@ cudaError_t launch_xcorr(int dtype, int r, const void *in, void *out, const Geom
 int xcorr_wide_max_radius();
 cudaError_t launch_xcorr_wide(int dtype, int r, const void *in, void *out, const Geom &g, const void *wdev,
                               bool periodic, bool images, unsigned *err, cudaStream_t s);
+// FP64 cross-correlation of radius 5..1024 in fixed point (xcorr_fx.cu): `limbs` receives the
+// weights' limb pairs (a device copy is `wfx`) and `ew` their scale; false where fixed point does
+// not apply (a weight is not finite, all are zero, exponents out of range).
+bool fx_wide_weights(const double *w, int count, std::vector<int32_t> &limbs, int *ew);
+cudaError_t launch_xcorr_wide_fx(int r, const double *in, double *out, const Geom &g, const double *wdev,
+                                 const void *wfx, int ew, bool periodic, bool images, cudaStream_t s);
 cudaError_t launch_maxfilter(int dtype, int r, const void *in, void *out, const Geom &g, bool periodic, bool images,
                              unsigned *err, cudaStream_t s);
 

@@ -1,0 +1,90 @@
+"""The FP64 cross-correlation in fixed point (csrc/xcorr_fx.cu): every output, also
+where the data span hundreds of binary orders or cancel, is as close to the exact sum as a chain
+of FP64 multiply-adds is, and infinities and NaN spread as they do in FP64."""
+import numpy as np
+import pytest
+import torch
+
+from paper_2406_08923_gb300 import _lib as L
+
+pytestmark = pytest.mark.gpu
+
+
+def _run(data, g, bc=L.STENCIL_BC_PERIODIC, halo=None):
+    n, r = data.size, g.size // 2
+    p = L.Plan(1, (n,), r, 1, bc, L.STENCIL_XCORR, L.STENCIL_F64, L.STENCIL_F64, coeffs=g)
+    a, b = p.alloc(), p.alloc()
+    p.upload(a, [data])
+    if halo is not None:
+        o = p.origin[0]
+        v = p.view3(a[0])[0, 0]
+        v[o - r:o], v[o + n:o + n + r] = torch.from_numpy(halo[0]).cuda(), torch.from_numpy(halo[1]).cuda()
+    p.step(a, b, 1)
+    p.sync()
+    whole = p.view3(b[0])[0, 0].cpu().numpy()
+    o = p.origin[0]
+    return whole[o:o + n], (whole[o - r:o], whole[o + n:o + n + r])
+
+
+def _reference(fhat, g):
+    """sum_j g_j f_{i+j} and sum_j |g_j f_{i+j}| of the augmented array, in extended precision."""
+    q, w = fhat.astype(np.longdouble), g.astype(np.longdouble)
+    n = q.size - g.size + 1
+    out, mag = np.zeros(n, np.longdouble), np.zeros(n, np.longdouble)
+    for j in range(g.size):
+        t = w[j] * q[j:j + n]
+        out += t
+        mag += np.abs(t)
+    return out, mag
+
+
+def _data(n, seed):
+    rng = np.random.default_rng(seed)
+    i = np.arange(n)
+    yield "random", rng.standard_normal(n)
+    yield "positive", rng.random(n)
+    yield "decay", np.exp(-i / 3.0)
+    yield "orders", rng.standard_normal(n) * 2.0 ** rng.integers(-200, 200, n)
+    yield "cancel", np.where(i % 2, 1.0, -1.0) + 1e-13 * rng.standard_normal(n)
+    yield "spikes", np.where(i % 97 == 5, 1e200, rng.standard_normal(n) * 1e-100) * (i % 1000 < 700)
+    yield "tiny", rng.standard_normal(n) * 2.0 ** -1030
+
+
+def _weights(r, kind):
+    rng = np.random.default_rng(1000 + r)
+    j = np.arange(-r, r + 1)
+    return {"average": lambda: np.full(2 * r + 1, 1.0 / (2 * r + 1)), "signed": lambda: rng.uniform(-1.0, 1.0, 2 * r + 1),
+            "gauss": lambda: np.exp(-12.0 * (j / r) ** 2), "orders": lambda: rng.standard_normal(2 * r + 1) *
+            2.0 ** rng.integers(-70, 5, 2 * r + 1)}[kind]()
+
+
+# radii around whole register blocks of 5, 7 and 9 weights, and the ends of the range
+@pytest.mark.parametrize("r,n", [(5, 11), (5, 3001), (6, 2305), (7, 2304), (8, 1793), (13, 5001), (22, 4999), (100, 4096),
+                                 (333, 2777), (1024, 2049), (1024, 7001)])
+@pytest.mark.parametrize("kind", ["average", "signed", "gauss", "orders"])
+def test_every_output_is_as_close_as_fp64(cuda_lib, r, n, kind):
+    g = _weights(r, kind)
+    for name, f in _data(n, r):
+        got, (lo, hi) = _run(f, g)
+        ref, mag = _reference(np.pad(f, r, mode="wrap"), g)
+        bound = (2 * r + 1) * 2.0 ** -53 * mag + (2 * r + 1) * 2.0 ** -1074  # one rounding per multiply-add
+        worst = float(np.max(np.abs(got - ref) / bound))
+        assert worst <= 1.0, (name, worst)
+        assert np.array_equal(lo, got[-r:]) and np.array_equal(hi, got[:r])
+
+
+def test_caller_halo_and_special_values(cuda_lib):
+    r, n = 9, 5000
+    rng = np.random.default_rng(4)
+    g = rng.uniform(-1.0, 1.0, 2 * r + 1)
+    f, halo = rng.standard_normal(n), (rng.standard_normal(r) * 1e3, rng.standard_normal(r) * 1e-3)
+    got, _ = _run(f, g, L.STENCIL_BC_CALLER, halo)
+    ref, mag = _reference(np.concatenate([halo[0], f, halo[1]]), g)
+    assert np.all(np.abs(got - ref) <= (2 * r + 1) * 2.0 ** -53 * mag)
+    f[100], f[3000], f[4990] = np.inf, np.nan, -np.inf
+    got, _ = _run(f, g)
+    with np.errstate(invalid="ignore"):
+        ref, mag = _reference(np.pad(f, r, mode="wrap"), g)
+        fine = np.isfinite(ref)
+        assert np.array_equal(np.isnan(got), np.isnan(ref)) and np.array_equal(np.isfinite(got), fine)
+        assert np.all(np.abs(got - ref)[fine] <= (2 * r + 1) * 2.0 ** -53 * mag[fine])
