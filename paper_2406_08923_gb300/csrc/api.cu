@@ -88,8 +88,11 @@ struct stencil_plan {
     double *red_out = nullptr;
     unsigned *err = nullptr;
     void *wdev = nullptr;  // XCORR of radius > 4: the 2r+1 weights on the device (storage type)
-    void *wfx = nullptr;   // FP64 XCORR of radius > 4: their fixed-point limbs (scale wfx_ew), if they fit
-    int wfx_ew = 0;
+    // Fixed-point weights of FP64 XCORR (and 1D DIFFUSION), if they fit: entry k - 1 runs k sweeps in
+    // one launch (radius > 4: k = 1 only), its tables in fxmem
+    std::vector<FxSweep> fx;
+    void *fxmem = nullptr;
+    std::vector<I32Weights> i32;  // int32 XCORR: entry k - 1, the weights of k sweeps
     unsigned long long *psync = nullptr;  // sync words of the persistent heat schedule (persist.cuh)
     int64_t psync_words = 0;
     int variant = 0;
@@ -149,8 +152,9 @@ static void free_scratch(stencil_t p) {
     if (p->red_out) cudaFree(p->red_out);
     if (p->err) cudaFree(p->err);
     if (p->wdev) cudaFree(p->wdev);
-    if (p->wfx) cudaFree(p->wfx);
-    p->wfx = nullptr;
+    if (p->fxmem) cudaFree(p->fxmem);
+    p->fxmem = nullptr;
+    p->fx.clear();
     if (p->psync) cudaFree(p->psync);
     p->psync = nullptr;
     p->psync_words = 0;
@@ -317,6 +321,45 @@ const char *stencil_strerror(stencil_status s) {
 
 const char *stencil_last_error_detail(stencil_t p) {
     return p ? p->detail.c_str() : g_create_detail.c_str();
+}
+
+// The fixed-point tables of a plan's 2r+1 weights w1 for 1 .. kmax sweeps per launch, in one
+// allocation: per k the composed weights (doubles), then the limb pairs.  Leaves p->fx empty where
+// some k's weights do not fit.  False after a CUDA error (reported in the creation detail).
+static bool make_fx(stencil_t p, const double *w1, int kmax) {
+    std::vector<unsigned char> host;
+    std::vector<FxSweep> fx;
+    std::vector<std::pair<size_t, size_t>> at;
+    std::vector<double> hi(w1, w1 + 2 * p->radius + 1), lo(hi.size(), 0.0);
+    std::vector<int32_t> limbs;
+    for (int k = 1; k <= kmax; ++k) {
+        FxSweep f{};
+        if (k > 1) fx_convolve(w1, p->radius, hi, lo);
+        if (!fx_wide_weights(hi.data(), lo.data(), (int)hi.size(), limbs, &f.ew)) return true;
+        f.r = k * p->radius;
+        f.r1 = p->radius;
+        f.sweeps = k;
+        const size_t a = host.size(), b = a + hi.size() * sizeof(double);
+        host.resize(b + limbs.size() * sizeof(int32_t));
+        std::memcpy(host.data() + a, hi.data(), hi.size() * sizeof(double));
+        std::memcpy(host.data() + b, limbs.data(), limbs.size() * sizeof(int32_t));
+        at.emplace_back(a, b);
+        fx.push_back(f);
+    }
+    cudaError_t e = cudaMalloc(&p->fxmem, host.size());
+    if (e == cudaSuccess) e = cudaMemcpy(p->fxmem, host.data(), host.size(), cudaMemcpyHostToDevice);
+    if (e != cudaSuccess) {
+        cuda_fail(nullptr, e, "fixed-point weight tables");
+        return false;
+    }
+    unsigned char *base = static_cast<unsigned char *>(p->fxmem);
+    for (size_t i = 0; i < fx.size(); ++i) {
+        fx[i].w = reinterpret_cast<const double *>(base + at[i].first);
+        fx[i].limbs = base + at[i].second;
+        fx[i].w1 = reinterpret_cast<const double *>(base);
+    }
+    p->fx = std::move(fx);
+    return true;
 }
 
 // Centred 2nd-derivative weights of order 2r on points -r..r (unit spacing): c[0] for the centre,
@@ -544,15 +587,14 @@ stencil_status stencil_create(int ndim, const int64_t dims[3], int radius, const
             e = cudaMemcpy(p->wdev, src, wide_w.size() * p->esize, cudaMemcpyHostToDevice);
             if (e != cudaSuccess) { cuda_fail(nullptr, e, "cudaMemcpy(weights)"); okay = false; }
         }
-        std::vector<int32_t> limbs;
-        if (okay && storage == STENCIL_F64 && fx_wide_weights(wide_w.data(), ncoeffs, limbs, &p->wfx_ew)) {
-            okay = alloc(&p->wfx, limbs.size() * sizeof(int32_t), "cudaMalloc(weight limbs)");
-            if (okay) {
-                e = cudaMemcpy(p->wfx, limbs.data(), limbs.size() * sizeof(int32_t), cudaMemcpyHostToDevice);
-                if (e != cudaSuccess) { cuda_fail(nullptr, e, "cudaMemcpy(weight limbs)"); okay = false; }
-            }
-        }
     }
+    if (okay && storage == STENCIL_F64 && radius > 0 &&
+        (kind == STENCIL_XCORR || (kind == STENCIL_DIFFUSION && ndim == 1))) {
+        const double *w1 = kind == STENCIL_XCORR && radius > 4 ? wide_w.data() : p->gd;
+        okay = make_fx(p, w1, bc == STENCIL_BC_PERIODIC && radius <= 4 ? xcorr_max_sweeps_per_launch(radius) : 1);
+    }
+    if (storage == STENCIL_I32 && kind == STENCIL_XCORR && radius > 0 && bc == STENCIL_BC_PERIODIC)
+        i32_compose(p->gi, radius, xcorr_max_sweeps_per_launch(radius), p->i32);
     if (okay) {
         e = cudaMemset(p->err, 0, sizeof(unsigned));
         if (e != cudaSuccess) { cuda_fail(nullptr, e, "cudaMemset(error word)"); okay = false; }
@@ -619,10 +661,17 @@ static stencil_status run_pass(stencil_t p, void *const *src, void *const *dst, 
            "maxfilter launch");
         return STENCIL_OK;
     }
-    if (p->kind == STENCIL_XCORR && p->wfx) {
-        CK(p, launch_xcorr_wide_fx(p->radius, static_cast<const double *>(src[0]), static_cast<double *>(dst[0]), g,
-                                   static_cast<const double *>(p->wdev), p->wfx, p->wfx_ew, periodic, periodic, s),
-           "xcorr (wide, fixed point) launch");
+    // a single sweep of 3 or 5 weights stays on the FP64 pipe (2^24 cells, r = 1: 112 us against 142)
+    if (sweeps >= 1 && sweeps <= (int)p->fx.size() && (sweeps > 1 || p->radius > 2)) {
+        CK(p, launch_xcorr_fx(static_cast<const double *>(src[0]), static_cast<double *>(dst[0]), g, p->fx[sweeps - 1],
+                              periodic, periodic, s),
+           "xcorr (fixed point) launch");
+        return STENCIL_OK;
+    }
+    if (sweeps >= 2 && sweeps <= (int)p->i32.size()) {
+        CK(p, launch_xcorr_i32(static_cast<const int32_t *>(src[0]), static_cast<int32_t *>(dst[0]), g,
+                               p->i32[sweeps - 1], sweeps * p->radius, p->radius, periodic, s),
+           "xcorr (composed sweeps) launch");
         return STENCIL_OK;
     }
     if (p->kind == STENCIL_XCORR && !xcorr_blocked(p)) {

@@ -1,9 +1,9 @@
 // fixed.cuh -- sums of products of doubles in 64-bit fixed point.
 //
-// GB300's FP64 pipe retires 2 multiply-adds per clock and SM, its integer pipe 64
-// 32 x 32 + 64-bit multiply-adds (mad.wide, measured 63.5 lanes per clock).  Four of those make
-// a 64 x 64-bit product, so a linear stencil of doubles runs up to eight times faster as integers
-// when the values of a neighbourhood share one binary scale.
+// GB300's FP64 pipe retires 2 multiply-adds per clock and SM, its integer pipe 32 multiply-adds of
+// 32 x 32 + 64 bits (mad.wide; measured 28 to 30 with distinct operands).  Four of those make a
+// 64 x 64-bit product, so a linear stencil of doubles runs up to four times faster as integers
+// when the values of a neighbourhood share one binary scale, and more where sums share products.
 //
 // A set of values whose largest magnitude has the (biased) exponent E is held as
 // q = trunc(v 2^(1082 - E)): |q| < 2^60, and 7 bits below a double's last place at the largest

@@ -49,12 +49,31 @@ cudaError_t launch_xcorr(int dtype, int r, const void *in, void *out, const Geom
 int xcorr_wide_max_radius();
 cudaError_t launch_xcorr_wide(int dtype, int r, const void *in, void *out, const Geom &g, const void *wdev,
                               bool periodic, bool images, unsigned *err, cudaStream_t s);
-// FP64 cross-correlation of radius 5..1024 in fixed point (xcorr_fx.cu): `limbs` receives the
-// weights' limb pairs (a device copy is `wfx`) and `ew` their scale; false where fixed point does
-// not apply (a weight is not finite, all are zero, exponents out of range).
-bool fx_wide_weights(const double *w, int count, std::vector<int32_t> &limbs, int *ew);
-cudaError_t launch_xcorr_wide_fx(int r, const double *in, double *out, const Geom &g, const double *wdev,
-                                 const void *wfx, int ew, bool periodic, bool images, cudaStream_t s);
+// FP64 cross-correlation in fixed point, and sweeps composed into one (xcorr_fx.cu).
+// `limbs` receives the limb pairs of weights hi + lo (lo may be null) and `ew` their scale; false
+// where fixed point does not apply (a weight is not finite, all are zero, exponents out of range).
+bool fx_wide_weights(const double *hi, const double *lo, int count, std::vector<int32_t> &limbs, int *ew);
+// hi + lo convolved with the 2r+1 weights g, in place (one more sweep).
+void fx_convolve(const double *g, int r, std::vector<double> &hi, std::vector<double> &lo);
+// One launch: `sweeps` sweeps of radius r1 (weights w1) as one of radius r = sweeps r1 with
+// the composed weights w and their limbs, all in device memory.
+struct FxSweep {
+    const double *w;
+    const void *limbs;
+    int ew, r;
+    const double *w1;
+    int r1, sweeps;
+};
+cudaError_t launch_xcorr_fx(const double *in, double *out, const Geom &g, const FxSweep &w, bool periodic, bool images,
+                            cudaStream_t s);
+// int32: the composed weights modulo 2^32, zero-padded; 2r+1 <= 129 of them.
+struct I32Weights {
+    static constexpr int N = 135;
+    uint32_t w[N];
+};
+void i32_compose(const int32_t *g, int r, int kmax, std::vector<I32Weights> &o);  // o[k - 1]: k sweeps
+cudaError_t launch_xcorr_i32(const int32_t *in, int32_t *out, const Geom &g, const I32Weights &w, int r, int r1,
+                             bool images, cudaStream_t s);
 cudaError_t launch_maxfilter(int dtype, int r, const void *in, void *out, const Geom &g, bool periodic, bool images,
                              unsigned *err, cudaStream_t s);
 

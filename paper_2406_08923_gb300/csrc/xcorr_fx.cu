@@ -1,23 +1,32 @@
-// xcorr_fx.cu -- FP64 1D cross-correlation (Sec. 3.1, Eq. 3) of radius 5..1024 in fixed point.
+// xcorr_fx.cu -- 1D cross-correlation (Sec. 3.1, Eq. 3) in integers: FP64 in fixed point for
+// radius 1..1024, and int32 sweeps of radius 1..4 composed into one.
 //
-// 2r+1 FP64 multiply-adds per output ran at 99 % of the FP64 pipe (2 per clock and SM).  Here a
-// CTA converts its chunk of cells, halo included, to signed 59-bit integers of one binary scale,
-// split into two 30-bit limbs, and the weights come as limbs too.  A product is then three
+// Composition.  k sweeps of a radius-r correlation are one correlation of radius k r whose weights
+// are the k-fold convolution of g with itself: 2 k r + 1 multiply-adds per output instead of
+// k (2 r + 1), with no halo to shrink, no exchange and no barrier between sweeps.  Modulo 2^32 the
+// two are equal bit for bit.  In FP64 the composed sum has fewer roundings than the sweeps; its
+// weights are convolved in double-double arithmetic, so that the fixed-point weights are
+// as exact as those of a single sweep.  2^20 cells, 10 sweeps, r = 3: int32 12.6 -> 10.4 us on the
+// device, FP64 129 -> 35 us.
+//
+// FP64.  2r+1 FP64 multiply-adds per output ran at 99 % of the FP64 pipe (2 per clock and SM).
+// Here a CTA converts its chunk of cells, halo included, to signed 59-bit integers of one binary
+// scale, split into two 30-bit limbs, and the weights come as limbs too.  A product is then three
 // 32 x 32 + 64-bit multiply-adds (the product of the two low limbs, below 2^-60 of the scale, is
-// left out), at 64 per clock and SM: 10 times the FP64 rate.
+// left out), at 32 per clock and SM: 5.3 times the FP64 rate.  3 M cells, r = 100: 1063 -> 238 us.
 //
 //   * As in xcorr_wide.cu each thread computes V consecutive outputs (V odd: conflict-free shared
 //     loads) and keeps V weights and 2V-1 cells in registers per block of V weights.
 //   * An output keeps two 64-bit sums: the high products HH and the cross products M, whose
-//     upper part moves to HH every one to three blocks, before 20 terms could overflow it.
+//     upper part moves to HH every one to four blocks, before 20 terms could overflow it.
 //   * Accuracy (fx_wide_weights): the result is off by at most 2 (2r+1) + 4 units of 2^-62 of
 //     the largest result the scale admits, which is no more than a chain of FP64 multiply-adds may
 //     be off, 2^-53 (2r+1) sum |w f|, wherever sum |w f| is at least 2^-7 of that result.  An output
 //     of that size itself shows it; the others are listed, their sum |w f| is accumulated from
 //     the high limbs until it passes the bound (a few terms for most), and what stays below is
 //     evaluated by FP64 multiply-adds in the order j = -r .. r.
-//   * A chunk with infinities, NaN or exponents near the ends of the range runs FP64
-//     multiply-adds throughout.
+//   * A chunk with infinities, NaN or exponents near the ends of the range is swept in FP64, one
+//     sweep after the other, in shared memory.
 #include <algorithm>
 #include <vector>
 
@@ -51,10 +60,11 @@ __device__ __forceinline__ int2 fx_limbs(double v, int E) {
     return make_int2((int)(u32)q - (int)((u32)qh << 30), qh);  // x: low limb, y: high limb
 }
 
-template <int V>
-__global__ void __launch_bounds__(FT, 2)
+template <int V, int MINB>
+__global__ void __launch_bounds__(FT, MINB)
 xcorr_wide_fx_kernel(const double *__restrict__ in, double *__restrict__ out, Geom geo, const double *__restrict__ wg,
-                     const int2 *__restrict__ wfx, int ew, int r, int periodic, int images) {
+                     const int2 *__restrict__ wfx, int ew, int r, const double *__restrict__ w1, int r1, int sweeps,
+                     int periodic, int images) {
     using B = FxWide<V>;
     constexpr int CH = B::CH;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -62,7 +72,7 @@ xcorr_wide_fx_kernel(const double *__restrict__ in, double *__restrict__ out, Ge
     __shared__ u32 listed;
     const int tid = threadIdx.x, nw = 2 * r + 1, nwp = B::nwp(r), cells = B::cells(r), len = CH + 2 * r;
     int2 *s = reinterpret_cast<int2 *>(smem_raw);
-    double *sd = reinterpret_cast<double *>(smem_raw);  // the cells before conversion, and the results
+    double *sd = reinterpret_cast<double *>(smem_raw);  // the results
     int2 *ws = s + cells;
     uint16_t *list = reinterpret_cast<uint16_t *>(ws + nwp);
     const int64_t n = geo.n[0], c0 = (int64_t)blockIdx.x * CH;
@@ -81,15 +91,21 @@ xcorr_wide_fx_kernel(const double *__restrict__ in, double *__restrict__ out, Ge
     pdl_launch_dependents();
     pdl_wait();
 
-    // stage the cells and find the largest exponent.  Cells past the last output's window count as 0.
+    // The cells and their largest exponent; those past the last output's window count as 0.  A
+    // thread's first KR cells stay in registers until the scale is known (radius 128 and less:
+    // all of them), the rest are read again.
+    constexpr int KR = V + 1;
+    double kept[KR];
     u32 hm = 0u;
     const bool inside = c0 - r >= 0 && c0 + CH + r <= n;
     const int used = (int)min((int64_t)len, n - c0 + 2 * r);
-    for (int e = tid; e < cells; e += FT) {
-        const double v = e < used ? (inside ? inx[c0 - r + e] : cell(c0 - r + e)) : 0.0;
-        sd[e] = v;
-        hm = max(hm, (u32)__double2hiint(v) & 0x7fffffffu);
-    }
+    const double *src = inx + (c0 - r);
+    auto load = [&](int e) -> double { return e < used ? (inside ? src[e] : cell(c0 - r + e)) : 0.0; };
+#pragma unroll
+    for (int k = 0; k < KR; ++k) kept[k] = load(tid + k * FT);
+#pragma unroll
+    for (int k = 0; k < KR; ++k) hm = max(hm, (u32)__double2hiint(kept[k]) & 0x7fffffffu);
+    for (int e = tid + KR * FT; e < cells; e += FT) hm = max(hm, (u32)__double2hiint(load(e)) & 0x7fffffffu);
     for (int j = tid; j < nwp; j += FT) ws[j] = j < nw ? wfx[j] : make_int2(0, 0);
     hm = __reduce_max_sync(0xffffffffu, hm);
     if ((tid & 31) == 0) red[tid >> 5] = hm;
@@ -102,14 +118,17 @@ xcorr_wide_fx_kernel(const double *__restrict__ in, double *__restrict__ out, Ge
     // FP64 multiply-adds of output p from global memory
     auto by_fp64 = [&](int p) -> double {
         double acc = 0.0;
-        for (int j = 0; j < nw; ++j) acc = fma(wg[j], inside ? inx[c0 - r + p + j] : cell(c0 - r + p + j), acc);
+        for (int j = 0; j < nw; ++j) acc = fma(wg[j], load(p + j), acc);
         return acc;
     };
 
     const int base = tid * V;
     double res[V];
     if (fixed) {
-        for (int e = tid; e < cells; e += FT) s[e] = fx_limbs(sd[e], E);  // in place: own elements
+#pragma unroll
+        for (int k = 0; k < KR; ++k)
+            if (tid + k * FT < cells) s[tid + k * FT] = fx_limbs(kept[k], E);
+        for (int e = tid + KR * FT; e < cells; e += FT) s[e] = fx_limbs(load(e), E);
         __syncthreads();
         long long hh[V], m[V];
 #pragma unroll
@@ -157,19 +176,25 @@ xcorr_wide_fx_kernel(const double *__restrict__ in, double *__restrict__ out, Ge
             }
             __syncthreads();
         }
+        // results through shared memory, then coalesced stores
+#pragma unroll
+        for (int v = 0; v < V; ++v) sd[base + v] = res[v];
     } else {
+        // every sweep leaves cell e of the sum at e: it reads e .. e + 2 r1, ascending in waves of FT
+        for (int e = tid; e < cells; e += FT) sd[e] = load(e);
         __syncthreads();
-#pragma unroll
-        for (int v = 0; v < V; ++v) {
-            double acc = 0.0;
-            for (int j = 0; j < nw; ++j) acc = fma(wg[j], sd[base + v + j], acc);
-            res[v] = acc;
+        for (int k = 1; k <= sweeps; ++k) {
+            const int span = len - 2 * r1 * k;
+            for (int e0 = 0; e0 < span; e0 += FT) {
+                double acc = 0.0;
+                if (e0 + tid < span)
+                    for (int j = 0; j < 2 * r1 + 1; ++j) acc = fma(w1[j], sd[e0 + tid + j], acc);
+                __syncthreads();  // in place: cells below e0 + FT are read by this wave only ...
+                if (e0 + tid < span) sd[e0 + tid] = acc;
+                __syncthreads();  // ... and the next wave starts at e0 + FT
+            }
         }
-        __syncthreads();
     }
-    // results through shared memory, then coalesced stores
-#pragma unroll
-    for (int v = 0; v < V; ++v) sd[base + v] = res[v];
     __syncthreads();
     if (fixed && listed) {
         for (u32 i = tid; i < listed; i += FT)
@@ -183,53 +208,118 @@ xcorr_wide_fx_kernel(const double *__restrict__ in, double *__restrict__ out, Ge
     } else {
         for (int q = tid; q < valid; q += FT) outx[c0 + q] = sd[q];
     }
-    if (images && (c0 < r || c0 + CH > n - r))
+    if (images && (c0 < r1 || c0 + CH > n - r1))
         for (int q = tid; q < valid; q += FT) {
             const int64_t p = c0 + q;
-            if (p < r) outx[p + n] = sd[q];
-            if (p >= n - r) outx[p - n] = sd[q];
+            if (p < r1) outx[p + n] = sd[q];
+            if (p >= n - r1) outx[p - n] = sd[q];
         }
 }
 
-// Block size V for radius r: the one with the fewest cycles per output, counting padded
-// multiply-adds (3 V^2 per block at 64 per clock and SM, in warp cycles 1.5 V^2) and half of the
-// shared loads' (2 (2V - 1) + V wavefronts per block), which overlap them in part.
-int fx_block(int r) {
+// int32 sweeps composed into one correlation of radius r <= 64 modulo 2^32.  Shared loads as above;
+// bound by the 64 multiply-adds per clock and SM, and at 2^20 cells by the latency of one load,
+// compute and store after another.
+template <int V>
+__global__ void __launch_bounds__(FT)
+xcorr_i32_kernel(const uint32_t *__restrict__ in, uint32_t *__restrict__ out, Geom geo,
+                 const __grid_constant__ I32Weights wp, int r, int r1, int images) {
+    constexpr int CH = FT * V;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    uint32_t *s = reinterpret_cast<uint32_t *>(smem_raw);
+    const int tid = threadIdx.x, nwp = (2 * r + 1 + V - 1) / V * V, cells = CH + nwp + V;
+    const int64_t n = geo.n[0], c0 = (int64_t)blockIdx.x * CH;
+    const uint32_t *inx = in + geo.off[0];
+    uint32_t *outx = out + geo.off[0];
+    pdl_launch_dependents();
+    pdl_wait();
+    const bool inside = c0 - r >= 0 && c0 - r + cells <= n;
+    for (int e = tid; e < cells; e += FT) {
+        int64_t gi = c0 - r + e;
+        if (!inside) {
+            gi %= n;
+            if (gi < 0) gi += n;
+        }
+        s[e] = inx[gi];
+    }
+    __syncthreads();
+    const int base = tid * V;
+    uint32_t acc[V];
+#pragma unroll
+    for (int v = 0; v < V; ++v) acc[v] = 0u;
+    for (int j0 = 0; j0 < nwp; j0 += V) {
+        uint32_t x[2 * V - 1];
+#pragma unroll
+        for (int q = 0; q < 2 * V - 1; ++q) x[q] = s[base + j0 + q];
+#pragma unroll
+        for (int u = 0; u < V; ++u)
+#pragma unroll
+            for (int v = 0; v < V; ++v) acc[v] += wp.w[j0 + u] * x[v + u];
+    }
+    __syncthreads();
+#pragma unroll
+    for (int v = 0; v < V; ++v) s[base + v] = acc[v];
+    __syncthreads();
+    const int valid = (int)min((int64_t)CH, n - c0);
+    if (valid == CH) {
+        for (int q = tid; q < CH / 4; q += FT) reinterpret_cast<uint4 *>(outx + c0)[q] = reinterpret_cast<const uint4 *>(s)[q];
+    } else {
+        for (int q = tid; q < valid; q += FT) outx[c0 + q] = s[q];
+    }
+    if (images && (c0 < r1 || c0 + CH > n - r1))
+        for (int q = tid; q < valid; q += FT) {
+            const int64_t p = c0 + q;
+            if (p < r1) outx[p + n] = s[q];
+            if (p >= n - r1) outx[p - n] = s[q];
+        }
+}
+
+// Block size V for n cells at radius r: the one with the least estimated time of the busiest SM.
+// A CTA costs, in cycles of its SM, its padded multiply-adds (3 V^2 per block for each of 8 warps,
+// at 32 lanes per clock), half of the shared loads' wavefronts, which overlap them in part, and
+// the conversion and output of its cells (about 300 V).  The estimate is within 20 % of the times
+// measured from 11 to 2001 weights and 30 000 to 2^24 cells, and picks the measured best, e.g.
+// V = 3 for 30 000 cells and 97 weights (12.4 us; V = 7: 20.6, V = 9: 24.7), V = 9 for 300 001
+// cells and 2001 weights (256 us; V = 3: 297, V = 7: 386).
+int fx_block(int r, int64_t n) {
     int best = 9;
     double least = 0.0;
-    for (int v : {5, 7, 9}) {
+    for (int v : {3, 7, 9}) {
         const int nb = (2 * r + 1 + v - 1) / v;
-        const double c = nb * (1.5 * v * v + 0.5 * (5 * v - 2)) / v;
+        const double cta = 8.0 * nb * (3.0 * v * v + 0.5 * (5 * v - 2)) + 300.0 * v;
+        const int64_t ctas = (n + FT * v - 1) / (FT * v), sms = device_sms();
+        const double c = cta * (double)((ctas + sms - 1) / sms);
         if (least == 0.0 || c < least) { least = c; best = v; }
     }
     return best;
 }
 
-template <int V>
-cudaError_t run(int r, const double *in, double *out, const Geom &g, const double *wdev, const int2 *wfx, int ew,
-                bool periodic, bool images, cudaStream_t s) {
-    auto k = xcorr_wide_fx_kernel<V>;
-    const size_t smem = FxWide<V>::smem(r);
+template <int V, int MINB>
+cudaError_t run(const double *in, double *out, const Geom &g, const FxSweep &w, bool periodic, bool images,
+                cudaStream_t s) {
+    auto k = xcorr_wide_fx_kernel<V, MINB>;
+    const size_t smem = FxWide<V>::smem(w.r);
     if (smem > 48 * 1024) {
         cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
         if (e != cudaSuccess) return e;
     }
     const unsigned blocks = (unsigned)((g.n[0] + FxWide<V>::CH - 1) / FxWide<V>::CH);
-    return launch_pdl(k, dim3(blocks), dim3(FT), smem, s, in, out, g, wdev, wfx, ew, r, periodic ? 1 : 0, images ? 1 : 0);
+    return launch_pdl(k, dim3(blocks), dim3(FT), smem, s, in, out, g, w.w, static_cast<const int2 *>(w.limbs), w.ew, w.r,
+                      w.w1, w.r1, w.sweeps, periodic ? 1 : 0, images ? 1 : 0);
 }
 
 }  // namespace
 
-// The weights as balanced limbs W = 2^30 wh + wl (stored {wl, wh}), w = W 2^(ew - 57): |W| <= 2^57
-// and sum |W| < 2^61, so that with |q| <= 2^59 the result sum W q / 2^58 stays below 2^62 and the
-// cross products of 20 terms below 2^63.  Rounding the weights and leaving out the low limbs'
-// products costs at most one unit per term each, rounding the cells 4 in all.
-bool fx_wide_weights(const double *w, int count, std::vector<int32_t> &limbs, int *ew) {
+// The weights hi + lo (lo may be null) as balanced limbs W = 2^30 wh + wl (stored {wl, wh}),
+// w = W 2^(ew - 57): |W| <= 2^57 and sum |W| < 2^61, so that with |q| <= 2^59 the result
+// sum W q / 2^58 stays below 2^62 and the cross products of 20 terms below 2^63.  Rounding the
+// weights and leaving out the low limbs' products costs at most one unit per term each, rounding
+// the cells 4 in all.
+bool fx_wide_weights(const double *hi, const double *lo, int count, std::vector<int32_t> &limbs, int *ew) {
     double top = 0.0, sum = 0.0;
     for (int i = 0; i < count; ++i) {
-        if (!std::isfinite(w[i])) return false;
-        top = std::fmax(top, std::fabs(w[i]));
-        sum += std::fabs(w[i]);
+        if (!std::isfinite(hi[i])) return false;
+        top = std::fmax(top, std::fabs(hi[i]));
+        sum += std::fabs(hi[i]);
     }
     if (!(top > 0.0) || !std::isfinite(sum)) return false;
     int e = 0;
@@ -238,7 +328,9 @@ bool fx_wide_weights(const double *w, int count, std::vector<int32_t> &limbs, in
     if (e < -100 || e > 100) return false;
     limbs.resize(2 * (size_t)count);
     for (int i = 0; i < count; ++i) {
-        const long long W = std::llrint(std::ldexp(w[i], 57 - e));
+        const double a = std::ldexp(hi[i], 57 - e), whole = std::nearbyint(a);
+        const double rest = (a - whole) + (lo ? std::ldexp(lo[i], 57 - e) : 0.0);
+        const long long W = (long long)whole + std::llrint(rest);
         const long long h = (W + (1ll << 29)) >> 30;
         limbs[2 * i] = (int32_t)(W - h * (1ll << 30));
         limbs[2 * i + 1] = (int32_t)h;
@@ -247,14 +339,53 @@ bool fx_wide_weights(const double *w, int count, std::vector<int32_t> &limbs, in
     return true;
 }
 
-cudaError_t launch_xcorr_wide_fx(int r, const double *in, double *out, const Geom &g, const double *wdev,
-                                 const void *wfx, int ew, bool periodic, bool images, cudaStream_t s) {
-    const int2 *w = static_cast<const int2 *>(wfx);
-    switch (fx_block(r)) {
-    case 5: return run<5>(r, in, out, g, wdev, w, ew, periodic, images, s);
-    case 7: return run<7>(r, in, out, g, wdev, w, ew, periodic, images, s);
-    default: return run<9>(r, in, out, g, wdev, w, ew, periodic, images, s);
+// (hi + lo) convolved with the 2r+1 weights g, in place, as unevaluated sums.
+void fx_convolve(const double *g, int r, std::vector<double> &hi, std::vector<double> &lo) {
+    std::vector<double> h(hi.size() + 2 * r, 0.0), l(hi.size() + 2 * r, 0.0);
+    for (size_t i = 0; i < hi.size(); ++i)
+        for (int j = 0; j < 2 * r + 1; ++j) {
+            // h + l += (hi + lo) g: exact product of the leading parts, Knuth's two-sum
+            const double p = hi[i] * g[j], e = std::fma(hi[i], g[j], -p) + lo[i] * g[j];
+            double &H = h[i + j], &Lo = l[i + j];
+            const double t = H + p, z = t - H;
+            Lo += ((H - (t - z)) + (p - z)) + e;
+            H = t + Lo;
+            Lo -= H - t;
+        }
+    hi.swap(h);
+    lo.swap(l);
+}
+
+void i32_compose(const int32_t *g, int r, int kmax, std::vector<I32Weights> &o) {
+    o.assign(kmax, I32Weights{});
+    std::copy(g, g + 2 * r + 1, o[0].w);
+    for (int k = 2; k <= kmax; ++k)
+        for (int i = 0; i < 2 * r * (k - 1) + 1; ++i)
+            for (int j = 0; j < 2 * r + 1; ++j) o[k - 1].w[i + j] += o[k - 2].w[i] * (uint32_t)g[j];
+}
+
+cudaError_t launch_xcorr_fx(const double *in, double *out, const Geom &g, const FxSweep &w, bool periodic, bool images,
+                            cudaStream_t s) {
+    switch (fx_block(w.r, g.n[0])) {
+    case 3: return run<3, 5>(in, out, g, w, periodic, images, s);
+    case 7:
+        // few weights: more CTAs to overlap loads, conversion and output (11 weights, 2^24 cells: 152
+        // against 176 us); many: the register budget of two (61 weights, 2^20 cells: 35 against 37 us)
+        if (w.r <= 16) return run<7, 4>(in, out, g, w, periodic, images, s);
+        return run<7, 2>(in, out, g, w, periodic, images, s);
+    default: return run<9, 3>(in, out, g, w, periodic, images, s);
     }
+}
+
+cudaError_t launch_xcorr_i32(const int32_t *in, int32_t *out, const Geom &g, const I32Weights &w, int r, int r1,
+                             bool images, cudaStream_t s) {
+    constexpr int V = 9, CH = FT * V;
+    const int nwp = (2 * r + 1 + V - 1) / V * V;
+    if (nwp > I32Weights::N) return cudaErrorInvalidValue;
+    const unsigned blocks = (unsigned)((g.n[0] + CH - 1) / CH);
+    return launch_pdl(xcorr_i32_kernel<V>, dim3(blocks), dim3(FT), sizeof(uint32_t) * (size_t)(CH + nwp + V), s,
+                      reinterpret_cast<const uint32_t *>(in), reinterpret_cast<uint32_t *>(out), g, w, r, r1,
+                      images ? 1 : 0);
 }
 
 }  // namespace stn

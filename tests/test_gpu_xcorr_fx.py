@@ -1,6 +1,7 @@
-"""The FP64 cross-correlation in fixed point (csrc/xcorr_fx.cu): every output, also
-where the data span hundreds of binary orders or cancel, is as close to the exact sum as a chain
-of FP64 multiply-adds is, and infinities and NaN spread as they do in FP64."""
+"""The FP64 cross-correlation in fixed point and the sweeps composed into one launch
+(csrc/xcorr_fx.cu): every output, also where the data span hundreds of binary orders or cancel, is
+as close to the exact sum as a chain of FP64 multiply-adds is, and infinities and NaN spread as
+they do in FP64."""
 import numpy as np
 import pytest
 import torch
@@ -10,7 +11,7 @@ from paper_2406_08923_gb300 import _lib as L
 pytestmark = pytest.mark.gpu
 
 
-def _run(data, g, bc=L.STENCIL_BC_PERIODIC, halo=None):
+def _run(data, g, bc=L.STENCIL_BC_PERIODIC, halo=None, sweeps=1):
     n, r = data.size, g.size // 2
     p = L.Plan(1, (n,), r, 1, bc, L.STENCIL_XCORR, L.STENCIL_F64, L.STENCIL_F64, coeffs=g)
     a, b = p.alloc(), p.alloc()
@@ -19,7 +20,7 @@ def _run(data, g, bc=L.STENCIL_BC_PERIODIC, halo=None):
         o = p.origin[0]
         v = p.view3(a[0])[0, 0]
         v[o - r:o], v[o + n:o + n + r] = torch.from_numpy(halo[0]).cuda(), torch.from_numpy(halo[1]).cuda()
-    p.step(a, b, 1)
+    p.step(a, b, sweeps)
     p.sync()
     whole = p.view3(b[0])[0, 0].cpu().numpy()
     o = p.origin[0]
@@ -58,9 +59,10 @@ def _weights(r, kind):
             2.0 ** rng.integers(-70, 5, 2 * r + 1)}[kind]()
 
 
-# radii around whole register blocks of 5, 7 and 9 weights, and the ends of the range
+# radii around whole register blocks of 3, 7 and 9 weights, and the ends of the range
 @pytest.mark.parametrize("r,n", [(5, 11), (5, 3001), (6, 2305), (7, 2304), (8, 1793), (13, 5001), (22, 4999), (100, 4096),
-                                 (333, 2777), (1024, 2049), (1024, 7001)])
+                                 (333, 2777), (1024, 2049), (1024, 7001),
+                                 (10, 400001), (40, 300001)])
 @pytest.mark.parametrize("kind", ["average", "signed", "gauss", "orders"])
 def test_every_output_is_as_close_as_fp64(cuda_lib, r, n, kind):
     g = _weights(r, kind)
@@ -88,3 +90,58 @@ def test_caller_halo_and_special_values(cuda_lib):
         fine = np.isfinite(ref)
         assert np.array_equal(np.isnan(got), np.isnan(ref)) and np.array_equal(np.isfinite(got), fine)
         assert np.all(np.abs(got - ref)[fine] <= (2 * r + 1) * 2.0 ** -53 * mag[fine])
+
+
+# one launch, one launch and a remainder, and radii that fill register blocks or not; n below the
+# composed halo wraps more than once
+@pytest.mark.parametrize("r,n,sweeps", [(1, 3, 1), (1, 2305, 16), (2, 5, 16), (2, 4000, 7), (3, 4099, 10), (3, 2304, 17),
+                                        (4, 9, 16), (4, 1793, 5)])
+@pytest.mark.parametrize("kind", ["average", "signed", "orders"])
+def test_composed_sweeps_are_as_close_as_fp64(cuda_lib, r, n, sweeps, kind):
+    g = _weights(r, kind)
+    for name, f in _data(n, 50 + r):
+        got, (lo, hi) = _run(f, g, sweeps=sweeps)
+        ref, mag = f.astype(np.longdouble), np.abs(f).astype(np.longdouble)
+        for _ in range(sweeps):
+            ref, mag = _reference(np.pad(ref, r, mode="wrap"), g)[0], _reference(np.pad(mag, r, mode="wrap"), np.abs(g))[0]
+        # one rounding per multiply-add of every sweep, each worth a denormal at least
+        tiny = sweeps * (2 * r + 1) * max(1.0, float(np.abs(g).sum())) ** sweeps * 2.0 ** -1074
+        worst = float(np.max(np.abs(got - ref) / (sweeps * (2 * r + 1) * 2.0 ** -53 * mag + tiny)))
+        assert worst <= 1.0, (name, worst)
+        assert np.array_equal(lo, got[-r:]) and np.array_equal(hi, got[:r])
+
+
+def test_composed_sweeps_spread_special_values_as_sweeps_do(cuda_lib):
+    r, n, sweeps = 3, 9001, 6
+    g = np.array([0.1, -0.2, 0.0, 0.5, 0.3, -0.1, 0.2])
+    f = np.random.default_rng(6).standard_normal(n)
+    f[100], f[3000], f[n - 2] = np.inf, np.nan, -np.inf
+    got, _ = _run(f, g, sweeps=sweeps)
+    ref = f.copy()
+    with np.errstate(invalid="ignore"):
+        for _ in range(sweeps):
+            q = np.pad(ref, r, mode="wrap")
+            ref = sum(g[j] * q[j:j + n] for j in range(7))
+    assert np.array_equal(np.isnan(got), np.isnan(ref)) and np.array_equal(np.isinf(got), np.isinf(ref))
+    fine = np.isfinite(ref)
+    np.testing.assert_allclose(got[fine], ref[fine], rtol=0, atol=1e-14)
+
+
+@pytest.mark.parametrize("r,n,sweeps", [(1, 3, 16), (2, 2305, 2), (3, 4099, 10), (3, 7, 33), (4, 9, 16), (4, 2304, 17),
+                                        (4, 70001, 16)])
+def test_composed_int32_sweeps_are_exact(cuda_lib, r, n, sweeps):
+    rng = np.random.default_rng(r + n)
+    f = rng.integers(-2 ** 31, 2 ** 31, n).astype(np.int32)
+    g = rng.integers(-2 ** 31, 2 ** 31, 2 * r + 1).astype(np.int32)
+    p = L.Plan(1, (n,), r, 1, L.STENCIL_BC_PERIODIC, L.STENCIL_XCORR, L.STENCIL_I32, L.STENCIL_I32, coeffs=g)
+    a, b = p.alloc(), p.alloc()
+    p.upload(a, [f])
+    p.step(a, b, sweeps)
+    p.sync()
+    ref = f.astype(np.uint32)
+    for _ in range(sweeps):
+        q = np.pad(ref, r, mode="wrap")
+        ref = sum(g.astype(np.uint32)[j] * q[j:j + n] for j in range(2 * r + 1))
+    whole = p.view3(b[0])[0, 0].cpu().numpy().astype(np.uint32)
+    o = p.origin[0]
+    assert np.array_equal(whole[o - r:o + n + r], np.pad(ref, r, mode="wrap"))
