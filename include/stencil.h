@@ -286,7 +286,8 @@ stencil_status stencil_sync(stencil_t plan, void *stream);
 
 /*
  * Kernel variants and runtime autotuning.  Each kind has a small table of kernel variants
- * (tile shape, pipeline depth, z-chunk length).  2D FP32 DIFFUSION also has temporally
+ * (tile shape, pipeline depth, z-chunk length); a new plan starts with the one its kind, radius
+ * and extents call for.  2D FP32 DIFFUSION also has temporally
  * blocked variants (1: two, 2: four Euler steps per pass over the field, the remainder one
  * step at a time); they apply with periodic boundaries and nx a multiple of 4 and otherwise
  * run the one-step kernel, with the same results.  As in the paper's automated tuning of the
@@ -297,7 +298,7 @@ stencil_status stencil_sync(stencil_t plan, void *stream);
  * length each CTA streams: the kernel's own choice, half of it, or twice it.  It overwrites
  * fields_out and synchronises `stream`.
  *
- * 3D FP32 DIFFUSION has each tile shape in two schedules: one launch per Euler step, and a
+ * 3D FP32 DIFFUSION has each 128-cell-wide tile shape in two schedules: one launch per Euler step, and a
  * persistent schedule (variant names ending in "_persist") that runs all nsteps steps of a
  * stencil_step call in one cooperative launch, each tile waiting only for the tiles whose
  * cells it reads to finish the previous step (bounded waits; an expired wait ends the call

@@ -605,6 +605,10 @@ stencil_status stencil_create(int ndim, const int64_t dims[3], int radius, const
         delete p;
         return st;
     }
+    // the launch shape for this size; all shapes give the same bits (stencil_set_variant, stencil_autotune)
+    if (kind == STENCIL_MHD8) mhd_default(storage_code(storage), g, &p->variant, &p->zmode);
+    else if (kind == STENCIL_DIFFUSION && storage == STENCIL_F32 && ndim == 3) p->variant = diffusion_f32_default(radius, g);
+    else if (kind == STENCIL_DIFFUSION && storage == STENCIL_F32 && ndim == 2) p->variant = diffusion2d_default(radius, g);
     *out = p;
     return STENCIL_OK;
 }

@@ -287,6 +287,17 @@ cudaError_t run_tb_r(const void *in, void *out, const Geom &g, const DiffCoef &c
 
 }  // namespace
 
+// The schedule a 2D FP32 plan starts with: 0 one step per pass, 1 two, 2 four.  A strip is one warp,
+// so small grids leave the chip idle: 16 steps in us, one step per pass first: r = 1 2896^2 196 ->
+// 142 (four), 2048^2 125 (124); r = 2 4096^2 488 -> 392 (two), 3000 x 4000 332 -> 290, 2896^2 212
+// (266); r = 3 4096^2 537 -> 499, 3000 x 4000 374 (426); r = 4 4096^2 658 (755).
+int diffusion2d_default(int r, const Geom &g) {
+    const int64_t cells = g.n[0] * g.n[1];
+    if (r == 1) return cells >= 5000000 ? 2 : 0;
+    if (r == 2) return cells >= 11000000 ? 1 : 0;
+    return r == 3 && cells >= 16000000 ? 1 : 0;
+}
+
 bool diffusion2d_tb_ok(int dtype, const Geom &g) { return dtype == 2 && g.n[0] % 4 == 0; }
 
 cudaError_t launch_diffusion2d_tb(int dtype, int steps, const void *in, void *out, const Geom &g, const DiffCoef &c,

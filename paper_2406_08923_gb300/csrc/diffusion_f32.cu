@@ -43,10 +43,20 @@ struct Coef32 {
     float ga[3][4];  // [axis][a-1]
 };
 
-template <int BY, int RY, int ZB, int NSLOT, int R>
+// Tile widths: a warp covers one row group of 128 cells, or two of 64.
+template <int W> struct H32Width;
+template <> struct H32Width<128> {
+    static constexpr int TX = 128, HX = 4;
+};
+template <> struct H32Width<64> {
+    static constexpr int TX = 64, HX = 4;
+};
+
+template <int BY, int RY, int ZB, int NSLOT, int R, int W = 128>
 struct H32 {
-    static constexpr int TX = 128, HX = 4, TXP = TX + 2 * HX;
-    static constexpr int TY = BY * RY, ROWS = TY + 2 * R;
+    static constexpr int TX = H32Width<W>::TX, HX = H32Width<W>::HX, TXP = TX + 2 * HX;
+    static constexpr int LX = TX / 4, GROUPS = 32 / LX;  // lanes per row group, row groups per warp
+    static constexpr int TY = BY * RY * GROUPS, ROWS = TY + 2 * R;
     static constexpr int SLOT = ((TXP * ROWS * 4 + 127) / 128) * 128 / 4;  // floats, 128 B aligned
     static constexpr uint32_t BOX_BYTES = TXP * ROWS * 4;
     static constexpr size_t SMEM = (size_t)NSLOT * SLOT * 4 + 128;
@@ -71,18 +81,18 @@ __device__ __forceinline__ void stg4(float *p, const float4 v) { *reinterpret_ca
 
 // One xy-tile of one z-chunk.  `map` may point at a __grid_constant__ parameter or at a
 // descriptor in global memory (batched launches).  Returns false if a bounded wait expired.
-template <int BY, int RY, int ZB, int NSLOT, int R, bool XVEC, bool PDL>
+template <int BY, int RY, int ZB, int NSLOT, int R, bool XVEC, bool PDL, int W = 128>
 __device__ __forceinline__ bool heat32_tile(const CUtensorMap *map, float *__restrict__ out, const Geom &g,
                                             const Coef32 &c, int tile_x, int tile_y, int tile_z, int zc, int images,
                                             unsigned *err, float *ring, uint64_t *full) {
-    using Cfg = H32<BY, RY, ZB, NSLOT, R>;
+    using Cfg = H32<BY, RY, ZB, NSLOT, R, W>;
     constexpr int TXP = Cfg::TXP, S = Cfg::S;
-    const int lane = threadIdx.x & 31, wy = threadIdx.x >> 5;
+    const int lx = threadIdx.x % Cfg::LX, row0 = threadIdx.x / Cfg::LX * RY;  // lane in its row group, first row
     const int x0 = tile_x * Cfg::TX, y0 = tile_y * Cfg::TY, zc0 = tile_z * zc;
     const int nx = (int)g.n[0], ny = (int)g.n[1], nz = (int)g.n[2];
     const int count = min(nz, zc0 + zc) - zc0;
     const int nplanes = count + 2 * R;  // planes zc0-R .. zc0+count+R-1
-    const int x = x0 + 4 * lane, yb = y0 + wy * RY;
+    const int x = x0 + 4 * lx, yb = y0 + row0;
 
     if (threadIdx.x == 0) {
         tma_prefetch_desc(map);
@@ -107,7 +117,7 @@ __device__ __forceinline__ bool heat32_tile(const CUtensorMap *map, float *__res
         for (; issued < NSLOT && issued < nplanes; ++issued) issue(issued);
 
     // float offset of (row 0 of this thread, first cell) inside a slot
-    const int own = (wy * RY + R) * TXP + Cfg::HX + 4 * lane;
+    const int own = (row0 + R) * TXP + Cfg::HX + 4 * lx;
     const float2 G0 = make_float2(c.g0, c.g0);
     float2 GA[3][R];
 #pragma unroll
@@ -252,10 +262,10 @@ __device__ __forceinline__ bool heat32_tile(const CUtensorMap *map, float *__res
                     if (nv) {
 #pragma unroll
                         for (int r = 0; r < RY; ++r) {
-                            if (yb + r >= ny) break;  // uniform per warp row
+                            if (yb + r >= ny) break;  // uniform per row group
                             float *p = op + r * pitch_y;
                             put(p, res[r]);
-                            if (ys[r] | zs) {  // y- and z-images: uniform per warp row / per plane
+                            if (ys[r] | zs) {  // y- and z-images: uniform per row group / per plane
                                 const int64_t dy = (int64_t)ys[r] * pitch_y, dz = (int64_t)zs * pitch_z;
                                 if (ys[r]) put(p + dy, res[r]);
                                 if (zs) put(p + dz, res[r]);
@@ -285,14 +295,14 @@ __device__ __forceinline__ bool heat32_tile(const CUtensorMap *map, float *__res
     return !bad;
 }
 
-template <int BY, int RY, int ZB, int NSLOT, int R, int MINB, bool XVEC>
+template <int BY, int RY, int ZB, int NSLOT, int R, int MINB, bool XVEC, int W>
 __global__ void __launch_bounds__(32 * BY, MINB)
 heat32_kernel(const __grid_constant__ CUtensorMap map_in, float *__restrict__ out, Geom g, Coef32 c, int zc,
               int images, unsigned *err) {
     extern __shared__ __align__(128) unsigned char smem_raw[];
     float *ring = reinterpret_cast<float *>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
     __shared__ __align__(8) uint64_t full[NSLOT];
-    heat32_tile<BY, RY, ZB, NSLOT, R, XVEC, true>(&map_in, out, g, c, blockIdx.x, blockIdx.y, blockIdx.z, zc,
+    heat32_tile<BY, RY, ZB, NSLOT, R, XVEC, true, W>(&map_in, out, g, c, blockIdx.x, blockIdx.y, blockIdx.z, zc,
                                                   images, err, ring, full);
 }
 
@@ -373,9 +383,9 @@ template <typename K> cudaError_t occupancy(K k, int threads, size_t smem, int c
 
 // Unit decomposition shared by both schedules: 128 x TY tiles of the xy-plane, z split into
 // chunks so that the units fill the resident CTA slots (choose_zchunks), then zmode.
-template <int BY, int RY, int ZB, int NSLOT, int R>
+template <int BY, int RY, int ZB, int NSLOT, int R, int W = 128>
 PersistGrid units_of(const Geom &g, int slots, int zmode) {
-    using Cfg = H32<BY, RY, ZB, NSLOT, R>;
+    using Cfg = H32<BY, RY, ZB, NSLOT, R, W>;
     const int tx = (int)((g.n[0] + Cfg::TX - 1) / Cfg::TX), ty = (int)((g.n[1] + Cfg::TY - 1) / Cfg::TY);
     const int nz = (int)g.n[2];
     const int chunks = choose_zchunks(tx * ty, nz, slots, 0.5);
@@ -383,16 +393,16 @@ PersistGrid units_of(const Geom &g, int slots, int zmode) {
     return PersistGrid{{tx, ty, (nz + zc - 1) / zc}, {Cfg::TX, Cfg::TY, zc}};
 }
 
-template <int BY, int RY, int ZB, int NSLOT, int R, int MINB, bool XVEC>
+template <int BY, int RY, int ZB, int NSLOT, int R, int MINB, bool XVEC, int W = 128>
 cudaError_t run(const CUtensorMap *map, float *out, const Geom &g, const Coef32 &c, bool images, unsigned *err,
                 cudaStream_t s, int zmode) {
-    using Cfg = H32<BY, RY, ZB, NSLOT, R>;
-    auto k = heat32_kernel<BY, RY, ZB, NSLOT, R, MINB, XVEC>;
+    using Cfg = H32<BY, RY, ZB, NSLOT, R, W>;
+    auto k = heat32_kernel<BY, RY, ZB, NSLOT, R, MINB, XVEC, W>;
     static int occ_cache[64] = {};
     int occ = 0;
     cudaError_t e = occupancy(k, 32 * BY, Cfg::SMEM, occ_cache, &occ);
     if (e != cudaSuccess) return e;
-    const PersistGrid pg = units_of<BY, RY, ZB, NSLOT, R>(g, occ * device_sms(), zmode);
+    const PersistGrid pg = units_of<BY, RY, ZB, NSLOT, R, W>(g, occ * device_sms(), zmode);
     dim3 grid(pg.nt[0], pg.nt[1], pg.nt[2]);
     return launch_pdl(k, grid, dim3(32 * BY), Cfg::SMEM, s, *map, out, g, c, pg.tl[2], images ? 1 : 0, err);
 }
@@ -438,20 +448,29 @@ cudaError_t run_persist(const CUtensorMap *maps, float *tmp, float *out, const G
     X(4, 1, 2, 8, 3)          \
     X(8, 2, 2, 8, 2)
 #define HEAT32_VARIANTS_OTHER(X) X(4, 2, 2, 8, 3)
+// Shapes with 64-cell rows, per-step schedule only: nx = 257 fills 5 tiles of 64 to 80 % and 3 of
+// 128 to 67 %.  (BY, RY, ZB, NSLOT, MINB, W)
+#define HEAT32_NARROW(X) X(4, 2, 2, 8, 3, 64) X(4, 1, 2, 8, 3, 64)
 
-// Each tile shape comes in both schedules: variants 0 .. n-1 launch once per step (PDL),
-// variants n .. 2n-1 run all steps of a call in one persistent launch (suffix "_persist").
-constexpr int N_R3 = 5, N_OTHER = 1;
+// Each 128-wide tile shape comes in both schedules: variants 0 .. n-1 launch once per step (PDL),
+// variants n .. 2n-1 run all steps of a call in one persistent launch (suffix "_persist").  The
+// narrow shapes follow.
+constexpr int N_R3 = 5, N_OTHER = 1, N_NARROW = 2;
 const char *const NAMES_R3[] = {"f32_by4_ry2_zb2_s8_m3",         "f32_by4_ry1_zb2_s8_m4",
                                 "f32_by8_ry1_zb2_s8_m2",         "f32_by4_ry1_zb2_s8_m3",
                                 "f32_by8_ry2_zb2_s8_m2",         "f32_by4_ry2_zb2_s8_m3_persist",
                                 "f32_by4_ry1_zb2_s8_m4_persist", "f32_by8_ry1_zb2_s8_m2_persist",
-                                "f32_by4_ry1_zb2_s8_m3_persist", "f32_by8_ry2_zb2_s8_m2_persist"};
-const char *const NAMES_OTHER[][2] = {{"?", "?"},
-                                      {"f32_r1_by4_ry2_zb2_s8_m3", "f32_r1_by4_ry2_zb2_s8_m3_persist"},
-                                      {"f32_r2_by4_ry2_zb2_s8_m3", "f32_r2_by4_ry2_zb2_s8_m3_persist"},
-                                      {"?", "?"},
-                                      {"f32_r4_by4_ry2_zb2_s8_m3", "f32_r4_by4_ry2_zb2_s8_m3_persist"}};
+                                "f32_by4_ry1_zb2_s8_m3_persist", "f32_by8_ry2_zb2_s8_m2_persist",
+                                "f32_w64_by4_ry2_zb2_s8_m3",     "f32_w64_by4_ry1_zb2_s8_m3"};
+const char *const NAMES_OTHER[][4] = {
+    {"?", "?", "?", "?"},
+    {"f32_r1_by4_ry2_zb2_s8_m3", "f32_r1_by4_ry2_zb2_s8_m3_persist", "f32_r1_w64_by4_ry2_zb2_s8_m3",
+     "f32_r1_w64_by4_ry1_zb2_s8_m3"},
+    {"f32_r2_by4_ry2_zb2_s8_m3", "f32_r2_by4_ry2_zb2_s8_m3_persist", "f32_r2_w64_by4_ry2_zb2_s8_m3",
+     "f32_r2_w64_by4_ry1_zb2_s8_m3"},
+    {"?", "?", "?", "?"},
+    {"f32_r4_by4_ry2_zb2_s8_m3", "f32_r4_by4_ry2_zb2_s8_m3_persist", "f32_r4_w64_by4_ry2_zb2_s8_m3",
+     "f32_r4_w64_by4_ry1_zb2_s8_m3"}};
 
 constexpr int n_shapes(int r) { return r == 3 ? N_R3 : N_OTHER; }
 
@@ -470,6 +489,13 @@ cudaError_t dispatch(int variant, const CUtensorMap *map, float *out, const Geom
     } else {
         HEAT32_VARIANTS_OTHER(X)
     }
+#undef X
+    i = 2 * n_shapes(R);
+#define X(BY, RY, ZB, NS, MB, W)                                                          \
+    if (i++ == variant)                                                                   \
+        res = xv ? run<BY, RY, ZB, NS, R, MB, true, W>(map, out, g, c, images, err, s, zmode) \
+                 : run<BY, RY, ZB, NS, R, MB, false, W>(map, out, g, c, images, err, s, zmode);
+    HEAT32_NARROW(X)
 #undef X
     return res;
 }
@@ -498,9 +524,23 @@ cudaError_t dispatch_persist(int shape, const CUtensorMap *maps, float *tmp, flo
 
 }  // namespace
 
-int diffusion_f32_num_variants(int r) { return r >= 1 && r <= 4 ? 2 * n_shapes(r) : 0; }
+int diffusion_f32_num_variants(int r) { return r >= 1 && r <= 4 ? 2 * n_shapes(r) + N_NARROW : 0; }
 
-bool diffusion_f32_persistent(int r, int v) { return v >= n_shapes(r) && v < diffusion_f32_num_variants(r); }
+// The shape a plan starts with.  The narrow 64 x 4 tile (a row per thread, three CTAs per SM) is the
+// fastest or within 3 % of it wherever 128-wide tiles leave lanes idle or the grid is small, 10
+// steps in us, first 128 x 8: 301 x 187 x 250 650 -> 444, 190^3 336 -> 231, 257 x 256^2 677 -> 524,
+// 64^3 49.5 -> 40.3, 40 x 56 x 72 58 -> 40, 350^3 1265 -> 1064, 128^3 90.6 -> 89.9; at radius 4 with
+// two rows per thread (301 x 187 x 250: 740 -> 552, one row 569).  Grids of whole 128-cell rows and
+// at least 2^23 cells, which the wide tiles fill, keep them: 256^3 365 (narrow 381), and from 2^25
+// cells on 128 x 16, which halves the y-halo re-reads: 384^3 1036 -> 1000, 512^3 2237 -> 2113.
+int diffusion_f32_default(int r, const Geom &g) {
+    const int64_t cells = g.n[0] * g.n[1] * g.n[2];
+    if (g.n[0] % 4 == 0 && (g.n[0] + 127) / 128 * 2 == (g.n[0] + 63) / 64 && cells >= ((int64_t)1 << 23))
+        return r == 3 && cells >= ((int64_t)1 << 25) ? 4 : 0;
+    return 2 * n_shapes(r) + (r == 4 ? 0 : 1);
+}
+
+bool diffusion_f32_persistent(int r, int v) { return v >= n_shapes(r) && v < 2 * n_shapes(r); }
 
 const char *diffusion_f32_variant_name(int r, int v) {
     if (v < 0 || v >= diffusion_f32_num_variants(r)) return "?";
@@ -508,10 +548,19 @@ const char *diffusion_f32_variant_name(int r, int v) {
 }
 
 void diffusion_f32_box(int r, int v, int box[3]) {
-    v %= n_shapes(r);  // both schedules of a shape load the same box
-    int i = 0;
-    box[0] = H32<1, 1, 2, 8, 1>::TXP;
+    int i = 2 * n_shapes(r);
     box[2] = 1;
+#define X(BY, RY, ZB, NS, MB, W) \
+    if (i++ == v) {              \
+        box[0] = H32<BY, RY, ZB, NS, 1, W>::TXP;                 \
+        box[1] = H32<BY, RY, ZB, NS, 1, W>::TY + 2 * r;          \
+        return;                  \
+    }
+    HEAT32_NARROW(X)
+#undef X
+    v %= n_shapes(r);  // both schedules of a shape load the same box
+    i = 0;
+    box[0] = H32<1, 1, 2, 8, 1>::TXP;
 #define X(BY, RY, ZB, NS, MB) \
     if (i++ == v) box[1] = BY * RY + 2 * r;
     if (r == 3) {

@@ -123,6 +123,7 @@ cudaError_t launch_diffusion_persist(int dtype, const CUtensorMap *maps, void *t
 int diffusion_f32_num_variants(int r);
 const char *diffusion_f32_variant_name(int r, int variant);
 void diffusion_f32_box(int r, int variant, int box[3]);
+int diffusion_f32_default(int r, const Geom &g);  // variant a 3D FP32 plan starts with
 cudaError_t launch_diffusion_f32(const CUtensorMap *map_in, float *out, const Geom &g, const DiffCoef &c,
                                  bool images, unsigned *err, cudaStream_t s, int variant, int zmode = 0);
 bool diffusion_f32_persistent(int r, int variant);
@@ -137,6 +138,7 @@ void diffusion2d_box(int dtype, int r, int box[3]);
 // 2D, temporally blocked (diffusion2d_tb.cu): `steps` = 2 or 4 Euler steps per pass, FP32,
 // periodic, nx a multiple of 4 (diffusion2d_tb_ok); reads `in` with periodic wrap (no halo).
 bool diffusion2d_tb_ok(int dtype, const Geom &g);
+int diffusion2d_default(int r, const Geom &g);  // variant a 2D FP32 plan starts with
 cudaError_t launch_diffusion2d_tb(int dtype, int steps, const void *in, void *out, const Geom &g, const DiffCoef &c,
                                   cudaStream_t s);
 
@@ -161,6 +163,7 @@ cudaError_t launch_mhd(int storage, int mode, int sub, const MhdMaps &maps, cons
                        const MhdConst &k, bool images, unsigned *err, cudaStream_t s,
                        int variant, int zmode = 0);
 void mhd_box(int storage, int variant, int box[3]);
+void mhd_default(int storage, const Geom &g, int *variant, int *zmode);  // what a plan starts with
 int mhd_num_variants(int storage);
 const char *mhd_variant_name(int storage, int variant);
 

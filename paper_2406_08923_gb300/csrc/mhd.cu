@@ -325,6 +325,26 @@ const char *mhd_variant_name(int storage, int v) {
     return storage == 1 ? MHD_F64_NAMES[v] : storage == 2 ? MHD_F32_NAMES[v] : MHD_BF16_NAMES[v];
 }
 
+// The tile and z-chunk mode a plan starts with (one RK3 step in us, 32 x 8 with one CTA per SM
+// first).  FP32: 32 x 16 up to 5 M cells (64^3 139 -> 121, 160^3 1280 -> 1070, 200 x 230 x 70 1084 ->
+// 884), 32 x 12 beyond (256^3 4210 -> 3437, 384^3 12816 -> 10486).  BF16: 32 x 8 with two CTAs per SM
+// (64^3 153 -> 121, 200 x 150 x 171 1843 -> 1307, 256^3 4899 -> 3258).  FP64: 16 x 8 (100 x 80 x 120
+// 5028 -> 4309, 256^3 61 173 -> 60 787), except rows of up to 32 cells (32^3 178, with 16 x 8 181).
+// Half-length chunks pay from about 2.5 M cells on (384^3 FP32 10 668 -> 10 486, 192^3 BF16 1773 ->
+// 1737; 128^3 FP32 657, with half chunks 673), in FP64 from the smallest.
+void mhd_default(int storage, const Geom &g, int *variant, int *zmode) {
+    const int64_t cells = g.n[0] * g.n[1] * g.n[2];
+    *zmode = cells >= 2500000 ? 1 : 0;
+    if (storage == 1) {
+        *variant = g.n[0] > 32 ? 1 : 0;
+        *zmode = *variant;
+    } else if (storage == 2) {
+        *variant = cells < 5000000 ? 3 : 4;
+    } else {
+        *variant = 1;
+    }
+}
+
 void mhd_box(int storage, int v, int box[3]) {
     int i = 0;
     auto put = [&](int tx, int ty, int hx) {
