@@ -6,7 +6,7 @@
 // k (2 r + 1), with no halo to shrink, no exchange and no barrier between sweeps.  Modulo 2^32 the
 // two are equal bit for bit.  In FP64 the composed sum has fewer roundings than the sweeps; its
 // weights are convolved in double-double arithmetic, so that the fixed-point weights are
-// as exact as those of a single sweep.  2^20 cells, 10 sweeps, r = 3: int32 12.6 -> 10.4 us on the
+// as exact as those of a single sweep.  2^20 cells, 10 sweeps, r = 3: int32 12.6 -> 6.6 us on the
 // device, FP64 129 -> 35 us.
 //
 // FP64.  2r+1 FP64 multiply-adds per output ran at 99 % of the FP64 pipe (2 per clock and SM).
@@ -88,7 +88,6 @@ xcorr_wide_fx_kernel(const double *__restrict__ in, double *__restrict__ out, Ge
         return (gi >= -r && gi < n + r) ? inx[gi] : 0.0;
     };
     if (tid == 0) listed = 0u;
-    pdl_launch_dependents();
     pdl_wait();
 
     // The cells and their largest exponent; those past the last output's window count as 0.  A
@@ -201,6 +200,7 @@ xcorr_wide_fx_kernel(const double *__restrict__ in, double *__restrict__ out, Ge
             if (list[i] != 0xffffu) sd[list[i]] = by_fp64(list[i]);
         __syncthreads();
     }
+    pdl_launch_dependents();  // not earlier: the next launch's CTAs would wait on the SMs
     const int valid = (int)min((int64_t)CH, n - c0);
     if (valid == CH) {
         for (int q = tid; q < CH / 2; q += FT)
@@ -216,6 +216,11 @@ xcorr_wide_fx_kernel(const double *__restrict__ in, double *__restrict__ out, Ge
         }
 }
 
+__device__ __forceinline__ void cp_async4(void *dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
+__device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
+
 // int32 sweeps composed into one correlation of radius r <= 64 modulo 2^32.  Shared loads as above;
 // bound by the 64 multiply-adds per clock and SM, and at 2^20 cells by the latency of one load,
 // compute and store after another.
@@ -230,17 +235,19 @@ xcorr_i32_kernel(const uint32_t *__restrict__ in, uint32_t *__restrict__ out, Ge
     const int64_t n = geo.n[0], c0 = (int64_t)blockIdx.x * CH;
     const uint32_t *inx = in + geo.off[0];
     uint32_t *outx = out + geo.off[0];
-    pdl_launch_dependents();
     pdl_wait();
-    const bool inside = c0 - r >= 0 && c0 - r + cells <= n;
-    for (int e = tid; e < cells; e += FT) {
-        int64_t gi = c0 - r + e;
-        if (!inside) {
-            gi %= n;
-            if (gi < 0) gi += n;
+    // asynchronous 4-byte copies, all in flight at once: a load and a shared store per cell left
+    // the block waiting for one round trip after another
+    if (c0 - r >= 0 && c0 - r + cells <= n) {
+        const uint32_t *src = inx + (c0 - r);
+        for (int e = tid; e < cells; e += FT) cp_async4(s + e, src + e);
+    } else {
+        for (int e = tid; e < cells; e += FT) {
+            int64_t gi = (c0 - r + e) % n;
+            cp_async4(s + e, inx + (gi < 0 ? gi + n : gi));
         }
-        s[e] = inx[gi];
     }
+    cp_async_wait_all();
     __syncthreads();
     const int base = tid * V;
     uint32_t acc[V];
@@ -259,6 +266,9 @@ xcorr_i32_kernel(const uint32_t *__restrict__ in, uint32_t *__restrict__ out, Ge
 #pragma unroll
     for (int v = 0; v < V; ++v) s[base + v] = acc[v];
     __syncthreads();
+    // the next launch's CTAs enter here and not earlier: waiting on the SMs from the start, they took
+    // 9.7 us per 2^20-cell call against 6.6
+    pdl_launch_dependents();
     const int valid = (int)min((int64_t)CH, n - c0);
     if (valid == CH) {
         for (int q = tid; q < CH / 4; q += FT) reinterpret_cast<uint4 *>(outx + c0)[q] = reinterpret_cast<const uint4 *>(s)[q];
