@@ -678,6 +678,12 @@ static stencil_status run_pass(stencil_t p, void *const *src, void *const *dst, 
            "xcorr (composed sweeps) launch");
         return STENCIL_OK;
     }
+    if (p->kind == STENCIL_XCORR && !xcorr_blocked(p) && p->storage == STENCIL_F32 && periodic) {
+        CK(p, launch_xcorr_pair(static_cast<const float *>(src[0]), static_cast<float *>(dst[0]), g,
+                                static_cast<const float *>(p->wdev), p->radius, true, s),
+           "xcorr (packed) launch");
+        return STENCIL_OK;
+    }
     if (p->kind == STENCIL_XCORR && !xcorr_blocked(p)) {
         CK(p, launch_xcorr_wide(storage_code(p->storage), p->radius, src[0], dst[0], g, p->wdev, periodic, periodic,
                                 p->err, s),

@@ -74,6 +74,9 @@ struct I32Weights {
 void i32_compose(const int32_t *g, int r, int kmax, std::vector<I32Weights> &o);  // o[k - 1]: k sweeps
 cudaError_t launch_xcorr_i32(const int32_t *in, int32_t *out, const Geom &g, const I32Weights &w, int r, int r1,
                              bool images, cudaStream_t s);
+// FP32, radius 33..1024, periodic: packed multiply-adds (xcorr_pair.cu).
+cudaError_t launch_xcorr_pair(const float *in, float *out, const Geom &g, const float *wdev, int r, bool images,
+                              cudaStream_t s);
 cudaError_t launch_maxfilter(int dtype, int r, const void *in, void *out, const Geom &g, bool periodic, bool images,
                              unsigned *err, cudaStream_t s);
 
