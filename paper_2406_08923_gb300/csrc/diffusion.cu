@@ -451,9 +451,8 @@ static cudaError_t run(const CUtensorMap *map, void *out, const Geom &g, const D
 // (not finite, or the signs of a backward or far from stable step); every other FP64 plan runs that one, whose launch
 // shapes the variants of radius 3 name.
 #define DIFF_VARIANT_F64(X) X(1, 8, 1, 2, 8, false)
-static const char *F64_NAMES[] = {"fx64x16_zb1_s16", "fx64x16_zb2_s16", "fx64x16_zb4_s16", "fx64x16_zb3_s16"};
-static const char *F64_NAMES_OTHER[] = {"?", "f64_r1_fx64x16_zb1_s16", "f64_r2_fx64x16_zb1_s16", "?",
-                                        "f64_r4_fx64x16_zb1_s16"};
+static const char *F64_NAMES[] = {"fx64x16", "fx64x16_more_chunks", "fx64x16_fewer_chunks", "fx64x16_even_waves"};
+static const char *F64_NAMES_OTHER[] = {"?", "f64_r1_fx64x16", "f64_r2_fx64x16", "?", "f64_r4_fx64x16"};
 
 int diffusion_num_variants(int dtype, int r) {
     if (dtype != 1) return diffusion_f32_num_variants(r);

@@ -8,14 +8,15 @@
 //
 //   * 2.5D z-streaming as in diffusion.cu: a CTA owns a 64 x 16 tile of the xy-plane and marches
 //     along z; padded plane tiles (72 x (16 + 2R)) arrive by TMA in a ring of 16 slots.
-//   * ZB new planes per iteration: every thread takes its share of their tiles into registers,
-//     the block reduces the largest exponent of each, and the values go back in place as biased
-//     60-bit integers at that plane's scale.
-//   * A thread owns 2 x-cells and loads their z column (ZB + 2R planes) once per iteration.  An
-//     output uses the largest scale of the 2R+1 planes its z column spans (S), and values of
-//     planes with a smaller one are shifted right, behind branches that are uniform per block.
-//     S depends on nothing but those plane tiles, so results do not depend on how z is split
-//     into iterations, chunks or slabs.
+//   * Between two block barriers a CTA works on three planes at once: it converts plane t in place
+//     (a thread's share, held in registers since the last interval) to biased 60-bit integers at
+//     the plane's scale, loads its share of plane t + 1 and reduces the largest exponent, and
+//     computes the outputs of plane t - R - 1.  One barrier per plane, and the warps overlap the
+//     three (two barriers with the phases one after another took 264 us per 256^3 step, this 235).
+//   * A thread owns 2 x-cells.  An output uses the largest scale of the 2R+1 planes its z column
+//     spans (S), and values of planes with a smaller one are shifted right, behind branches that
+//     are uniform per block.  S depends on nothing but those plane tiles, so results do not
+//     depend on how z is split into chunks or slabs.
 //   * With one grid spacing on all axes (ISO) the six values at distance a are summed first: four
 //     64 x 64-bit products per cell instead of ten.
 //   * Outputs whose stencil is small against S (fixed.cuh), or that meet infinities or NaN, are
@@ -35,18 +36,17 @@ template <int R, bool ISO> struct FxCoef {
     double g0, ga[3][R];  // for the outputs evaluated in FP64
 };
 
-template <int ZB_, int NSLOT_, int R> struct FxCfg {
-    static constexpr int BY = 16, NT = 32 * BY, ZB = ZB_, NSLOT = NSLOT_;
+template <int R> struct FxCfg {
+    static constexpr int BY = 16, NT = 32 * BY, NSLOT = 16;
     static constexpr int TX = 64, TY = BY, HX = 4, TXP = TX + 2 * HX, ROWS = TY + 2 * R;
     static constexpr int PAIRS = TXP / 2 * ROWS;  // 16-byte pairs per plane tile
     static constexpr int KP = (PAIRS + NT - 1) / NT;
     static constexpr int SLOT = ((TXP * ROWS * 8 + 127) / 128) * 128 / 8;
     static constexpr uint32_t BOX_BYTES = TXP * ROWS * 8;
     static constexpr size_t SMEM = (size_t)NSLOT * SLOT * 8 + 128;
-    static constexpr int S = ZB + 2 * R;  // planes of an iteration's z column
     static constexpr int LIST = 1024;
     static_assert((NSLOT & (NSLOT - 1)) == 0, "ring depth is a power of two (slot = j & (NSLOT-1))");
-    static_assert(NSLOT >= 2 * ZB + 2 * R, "ring: an iteration's planes and the next ZB");
+    static_assert(NSLOT >= 2 * R + 4, "ring: an output's planes, the two being converted and loaded, one refill");
     static_assert(R >= 1 && R <= 4, "");
 };
 
@@ -67,9 +67,10 @@ __device__ __noinline__ double heat_fp64_cell(const double *__restrict__ in, con
 }
 
 // Two neighbouring outputs: `cp` points at the first in its centre plane (scale sc - dc), z(k, u)
-// gives the value of cell u at plane offset k, at scale sc.  Returns bit u set where output u is
-// left to FP64: the centre and its four neighbours in the plane are below 2^-6 of the scale.
-template <int R, bool ISO, int TXP, typename W, typename Z>
+// gives the value of cell u at plane offset k != 0, at scale sc; SAME: dc is 0.  Returns bit u set
+// where output u is left to FP64: the centre and its four neighbours in the plane are below 2^-6
+// of the scale.
+template <int R, bool ISO, bool SAME, int TXP, typename W, typename Z>
 __device__ __forceinline__ int fx_pair(const u64 *cp, const Z &z, int dc, int sc, const W &w, double (&res)[2]) {
     u64 X[10];  // x window: cells -4 .. 5
 #pragma unroll
@@ -86,7 +87,7 @@ __device__ __forceinline__ int fx_pair(const u64 *cp, const Z &z, int dc, int sc
         const u32 a = (u32)(X[3 + u] >> 32), d = (u32)(X[5 + u] >> 32), e = (u32)(X[4 + u] >> 32);
         hmx[u] = max(max(a, d), e);
         hmn[u] = min(min(a, d), e);
-        acc[u].mac(w.wh[0], w.wl[0], z(0, u));
+        acc[u].mac(w.wh[0], w.wl[0], SAME ? X[4 + u] : fx_shift(X[4 + u], FX_BIAS, dc));
     }
     // the in-plane pairs of every distance, moved to the common scale together
     u64 sxy[2][R], sy[2][R];
@@ -106,7 +107,7 @@ __device__ __forceinline__ int fx_pair(const u64 *cp, const Z &z, int dc, int sc
             if (ISO) sxy[u][a - 1] += sy[u][a - 1];
         }
     }
-    if (dc) {
+    if (!SAME) {
 #pragma unroll
         for (int a = 0; a < R; ++a)
 #pragma unroll
@@ -137,7 +138,7 @@ __device__ __forceinline__ int fx_pair(const u64 *cp, const Z &z, int dc, int sc
             }
         }
     }
-    const u32 flag = dc < 6 ? FX_FLAG_HI << dc : FX_BIAS_HI;
+    const u32 flag = SAME ? FX_FLAG_HI : (dc < 6 ? FX_FLAG_HI << dc : FX_BIAS_HI);
     int left = 0;
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
@@ -148,36 +149,19 @@ __device__ __forceinline__ int fx_pair(const u64 *cp, const Z &z, int dc, int sc
     return left;
 }
 
-// The same where the output's scale is finer than the one the iteration's z column is held at:
-// plane j (its centre) and the others are read again.  Out of line: a tenth of the outputs or fewer.
-template <int R, bool ISO, int TXP, int SLOT, int NSLOT, typename W>
-__device__ __noinline__ int fx_pair_reread(const u64 *ring, const int *scale, int j, int own, int sc, const W &w,
-                                           double *out) {
-    double res[2];
-    const int left = fx_pair<R, ISO, TXP>(
-        ring + (j & (NSLOT - 1)) * SLOT + own,
-        [&](int k, int u) {
-            const int s = (j + k) & (NSLOT - 1);
-            return fx_shift(ring[s * SLOT + own + u], FX_BIAS, sc - scale[s]);
-        },
-        sc - scale[j & (NSLOT - 1)], sc, w, res);
-    out[0] = res[0];
-    out[1] = res[1];
-    return left;
-}
-
-template <int ZB, int NSLOT, int R, bool ISO>
-__global__ void __launch_bounds__(FxCfg<ZB, NSLOT, R>::NT, 1)
+template <int R, bool ISO>
+__global__ void __launch_bounds__(FxCfg<R>::NT, 1)
 heat_fx_kernel(const __grid_constant__ CUtensorMap map, const double *__restrict__ in, double *__restrict__ out,
                const __grid_constant__ Geom g, const __grid_constant__ FxCoef<R, ISO> c, int zc, int images,
                unsigned *err) {
-    using Cfg = FxCfg<ZB, NSLOT, R>;
-    constexpr int NT = Cfg::NT, TXP = Cfg::TXP, S = Cfg::S, KP = Cfg::KP;
+    using Cfg = FxCfg<R>;
+    constexpr int NT = Cfg::NT, NSLOT = Cfg::NSLOT, TXP = Cfg::TXP, KP = Cfg::KP;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     // TMA destinations 128-byte aligned (128 spare bytes); an offset, so that loads stay shared loads
     u64 *ring = reinterpret_cast<u64 *>(smem_raw + ((128u - (smem_addr(smem_raw) & 127u)) & 127u));
     __shared__ __align__(8) uint64_t full[NSLOT];
-    __shared__ int scale[NSLOT];  // exponent code of each slot's plane
+    __shared__ int scale[NSLOT];     // exponent code of each slot's plane
+    __shared__ int4 window[2];       // of an output plane, by parity: {scale, planes differ, centre's shift}
     __shared__ u32 list[Cfg::LIST];
     __shared__ u32 listed;
     const int tid = threadIdx.x, lane = tid & 31, wy = tid >> 5;
@@ -215,83 +199,65 @@ heat_fx_kernel(const __grid_constant__ CUtensorMap map, const double *__restrict
     // corner, and a caller may leave it unset).  On periodic grids the z-halo planes are images of
     // interior planes and count like them.  Tiles inside the interior skip the test.
     const bool edge = x0 - Cfg::HX < 0 || x0 + Cfg::TX + Cfg::HX > nx || y0 - R < 0 || y0 + Cfg::TY + R > ny || !images;
-    auto counts = [&](int col, int row, int j) -> bool {
-        const int gx = x0 - Cfg::HX + col, gy = y0 - R + row, gz = zc0 - R + j;
-        const bool ox = gx < 0 || gx >= nx, oy = gy < 0 || gy >= ny, oz = !images && (gz < 0 || gz >= nz);
-        return gx >= -R && gx < nx + R && gy < ny + R && (int)ox + (int)oy + (int)oz <= 1;
-    };
+    u32 keep = ~0u, keep_zhalo = ~0u;  // bits 2 k, 2 k + 1: this thread's k-th pair, in a plane of the interior / beyond
+    if (edge) {
+        keep = keep_zhalo = 0u;
+#pragma unroll
+        for (int k = 0; k < KP; ++k)
+#pragma unroll
+            for (int u = 0; u < 2; ++u) {
+                const int i = tid + k * NT, row = i / (TXP / 2), gx = x0 - Cfg::HX + 2 * (i - row * (TXP / 2)) + u;
+                const int gy = y0 - R + row, outside = (gx < 0 || gx >= nx) + (gy < 0 || gy >= ny);
+                const bool near = gx >= -R && gx < nx + R && gy < ny + R;
+                if (near && outside <= 1) keep |= 1u << (2 * k + u);
+                if (near && outside + !images <= 1) keep_zhalo |= 1u << (2 * k + u);
+            }
+    }
     bool ok = true;
-    // Converts planes j .. j + ZB - 1 below `end` in place.  Two block barriers: the first also
-    // retires what every thread read before the call, so the ring is refilled there, up to plane
-    // `refill`.
-    auto convert = [&](int j, int end, int refill) -> bool {
-        double2 v[ZB][KP];
+    double2 raw[KP];  // this thread's share of the plane loaded last
+    auto load = [&](int j) {
+        const int s = j & (NSLOT - 1);
+        ok = ok && mbar_wait_bounded(&full[s], ((unsigned)j / NSLOT) & 1u);
+        const double2 *src = reinterpret_cast<const double2 *>(ring + s * Cfg::SLOT);
+        u32 hm = 0u;
 #pragma unroll
-        for (int b = 0; b < ZB; ++b) {
-            if (j + b < end) {
-                const int s = (j + b) & (NSLOT - 1);
-                ok = ok && mbar_wait_bounded(&full[s], ((unsigned)(j + b) / NSLOT) & 1u);
-                const double2 *src = reinterpret_cast<const double2 *>(ring + s * Cfg::SLOT);
-                u32 hm = 0u;
-#pragma unroll
-                for (int k = 0; k < KP; ++k) {
-                    const int i = tid + k * NT;
-                    v[b][k] = make_double2(0.0, 0.0);
-                    if (i < Cfg::PAIRS) {
-                        v[b][k] = src[i];
-                        if (edge) {
-                            const int row = i / (TXP / 2), col = 2 * (i - row * (TXP / 2));
-                            if (!counts(col, row, j + b)) v[b][k].x = 0.0;
-                            if (!counts(col + 1, row, j + b)) v[b][k].y = 0.0;
-                        }
-                    }
-                    hm = max(hm, max((u32)__double2hiint(v[b][k].x) & 0x7fffffffu,
-                                     (u32)__double2hiint(v[b][k].y) & 0x7fffffffu));
-                }
-                hm = __reduce_max_sync(0xffffffffu, hm);
-                int code = (int)(hm >> 20);
-                if (hm == 0u) {  // only zeros and the smallest denormals: tell them apart
-                    u32 any = 0u;
-#pragma unroll
-                    for (int k = 0; k < KP; ++k) any |= (u32)__double2loint(v[b][k].x) | (u32)__double2loint(v[b][k].y);
-                    code = __reduce_or_sync(0xffffffffu, any) != 0u;
-                } else if (code == 0) {
-                    code = 1;
-                }
-                if (lane == 0) atomicMax(&scale[s], code);
-            }
-        }
-        const bool bad = __syncthreads_or(!ok);
-        if (!bad && tid == 0) {
-            fence_proxy_async();  // the block's generic writes to a slot before its next TMA load
-            for (; issued < min(nplanes, refill); ++issued) {
-                scale[issued & (NSLOT - 1)] = 0;
-                issue(issued);
-            }
-        }
-#pragma unroll
-        for (int b = 0; b < ZB; ++b) {
-            if (j + b < end) {
-                const int s = (j + b) & (NSLOT - 1);
-                const int e = scale[s];
-                ulonglong2 *dst = reinterpret_cast<ulonglong2 *>(ring + s * Cfg::SLOT);
-                // outside this range nothing shows at a scale the sums use, or the outputs go to FP64
-                const bool in_range = e >= FX_EMIN && e <= FX_EMAX;
-#pragma unroll
-                for (int k = 0; k < KP; ++k) {
-                    const int i = tid + k * NT;
-                    if (i < Cfg::PAIRS)
-                        dst[i] = in_range ? make_ulonglong2(fx_from_double(v[b][k].x, e), fx_from_double(v[b][k].y, e))
-                                          : make_ulonglong2(FX_BIAS, FX_BIAS);
+        for (int k = 0; k < KP; ++k) {
+            const int i = tid + k * NT;
+            raw[k] = make_double2(0.0, 0.0);
+            if (i < Cfg::PAIRS) {
+                raw[k] = src[i];
+                if (edge) {
+                    const u32 kp = zc0 - R + j < 0 || zc0 - R + j >= nz ? keep_zhalo : keep;
+                    if (!(kp & (1u << (2 * k)))) raw[k].x = 0.0;
+                    if (!(kp & (2u << (2 * k)))) raw[k].y = 0.0;
                 }
             }
+            hm = max(hm, max((u32)__double2hiint(raw[k].x) & 0x7fffffffu, (u32)__double2hiint(raw[k].y) & 0x7fffffffu));
         }
-        __syncthreads();
-        return bad;
+        hm = __reduce_max_sync(0xffffffffu, hm);
+        int code = (int)(hm >> 20);
+        if (hm == 0u) {  // only zeros and the smallest denormals: tell them apart
+            u32 any = 0u;
+#pragma unroll
+            for (int k = 0; k < KP; ++k) any |= (u32)__double2loint(raw[k].x) | (u32)__double2loint(raw[k].y);
+            code = __reduce_or_sync(0xffffffffu, any) != 0u;
+        } else if (code == 0) {
+            code = 1;
+        }
+        if (lane == 0) atomicMax(&scale[s], code);
     };
-
-    bool bad = false;
-    for (int j = 0; j < 2 * R; j += ZB) bad = convert(j, 2 * R, 0) || bad;
+    auto convert = [&](int j) {
+        const int s = j & (NSLOT - 1);
+        // below FX_EMIN nothing shows at a scale the sums use, above FX_EMAX the outputs go to FP64
+        const int e = max(scale[s], FX_EMIN);
+        ulonglong2 *dst = reinterpret_cast<ulonglong2 *>(ring + s * Cfg::SLOT);
+#pragma unroll
+        for (int k = 0; k < KP; ++k) {
+            const int i = tid + k * NT;
+            if (i < Cfg::PAIRS)
+                dst[i] = make_ulonglong2(fx_from_double(raw[k].x, e), fx_from_double(raw[k].y, e));
+        }
+    };
 
     // Store targets.  Even extents store the images of whole pairs (a neighbour that has none lands
     // in the row padding), odd ones cell by cell.
@@ -335,49 +301,55 @@ heat_fx_kernel(const __grid_constant__ CUtensorMap map, const double *__restrict
         }
     };
 
+    const bool plain = nv == 2 && (mlo | mhi) == 0;  // both cells, no x image
     const int own = (wy + R) * TXP + Cfg::HX + 2 * lane;
-    for (int m = 0; m < count; m += ZB) {
-        bad = convert(m + 2 * R, nplanes, m + NSLOT) || bad;  // planes below m are retired
-        if (bad) break;
-        if (nv == 0) continue;
-        // the z column at one scale: the largest of the iteration's planes
-        int E[S];
-        u64 Q[S][2];
-        int top = 0;
-#pragma unroll
-        for (int k = 0; k < S; ++k) {
-            const int s = (m + k) & (NSLOT - 1);
-            E[k] = m + k < nplanes ? scale[s] : 0;
-            const ulonglong2 t = *reinterpret_cast<const ulonglong2 *>(ring + s * Cfg::SLOT + own);
-            Q[k][0] = t.x;
-            Q[k][1] = t.y;
-            top = max(top, E[k]);
-        }
-        bool mixed = false;
-#pragma unroll
-        for (int k = 0; k < S; ++k) mixed = mixed || E[k] < top;
-        if (mixed) {
-#pragma unroll
-            for (int k = 0; k < S; ++k) {
-                const int d = top - E[k];
-                Q[k][0] = fx_shift(Q[k][0], FX_BIAS, d);
-                Q[k][1] = fx_shift(Q[k][1], FX_BIAS, d);
+    load(0);
+    bool bad = __syncthreads_or(!ok);
+    for (int t = 0; !bad && t <= nplanes; ++t) {
+        // the plane's scale is complete since the barrier; its slot is read from the next one on
+        if (t < nplanes) {
+            convert(t);
+            if (tid == NT - 1 && t >= 2 * R) {  // the window of the next interval's outputs: planes t - 2R .. t
+                int top = 0, low = 4096;
+                for (int k = t - 2 * R; k <= t; ++k) {
+                    const int e = scale[k & (NSLOT - 1)];
+                    top = max(top, e);
+                    low = min(low, e);
+                }
+                window[t & 1] = make_int4(top, low < top, top - scale[(t - R) & (NSLOT - 1)], 0);
             }
+            if (t + 1 < nplanes) load(t + 1);
         }
-#pragma unroll
-        for (int b = 0; b < ZB; ++b) {
-            if (m + b >= count) break;
-            int sc = E[b];
-#pragma unroll
-            for (int k = 1; k <= 2 * R; ++k) sc = max(sc, E[b + k]);
-            const int z = zc0 + m + b;
-            const u64 *cp = ring + ((m + b + R) & (NSLOT - 1)) * Cfg::SLOT + own;
+        const int m = t - 1 - 2 * R;  // outputs of plane zc0 + m, from planes m .. t - 1
+        if (m >= 0 && nv != 0) {
+            const int4 win = window[(t - 1) & 1];
+            const int sc = win.x, dc = win.z, z = zc0 + m;
+            const u64 *cp = ring + ((m + R) & (NSLOT - 1)) * Cfg::SLOT + own;
             double res[2];
             int left = 0;  // outputs left to FP64
-            if (sc == top && sc >= FX_SMIN && sc <= FX_EMAX) {
-                left = fx_pair<R, ISO, TXP>(cp, [&](int k, int u) { return Q[b + R + k][u]; }, sc - E[b + R], sc, c.w, res);
-            } else if (sc >= FX_SMIN && sc <= FX_EMAX) {  // a finer scale than the column's: read it again
-                left = fx_pair_reread<R, ISO, TXP, Cfg::SLOT, NSLOT>(ring, scale, m + b + R, own, sc, c.w, res);
+            if (sc >= FX_SMIN && sc <= FX_EMAX) {
+                u64 Q[2 * R + 1][2];  // the z column at scale sc (its centre is read with the row)
+#pragma unroll
+                for (int k = 0; k <= 2 * R; ++k) {
+                    if (k == R) continue;
+                    const ulonglong2 q =
+                        *reinterpret_cast<const ulonglong2 *>(ring + ((m + k) & (NSLOT - 1)) * Cfg::SLOT + own);
+                    Q[k][0] = q.x;
+                    Q[k][1] = q.y;
+                }
+                auto column = [&](int k, int u) { return Q[R + k][u]; };
+                if (!win.y) {
+                    left = fx_pair<R, ISO, true, TXP>(cp, column, 0, sc, c.w, res);
+                } else {
+#pragma unroll
+                    for (int k = 0; k <= 2 * R; ++k) {
+                        if (k == R) continue;
+                        const int d = sc - scale[(m + k) & (NSLOT - 1)];
+                        Q[k][0] = fx_shift(Q[k][0], FX_BIAS, d);
+                        Q[k][1] = fx_shift(Q[k][1], FX_BIAS, d);
+                    }
+                    left = fx_pair<R, ISO, false, TXP>(cp, column, dc, sc, c.w, res);
+                }
             } else {  // zeros only, or infinities, NaN, or near the ends of the exponent range
                 res[0] = res[1] = 0.0;
                 left = sc == 0 ? 0 : 3;
@@ -388,21 +360,29 @@ heat_fx_kernel(const __grid_constant__ CUtensorMap map, const double *__restrict
                 for (int u = 0; u < 2; ++u)
                     if (left & (1 << u)) {
                         const u32 at = atomicAdd(&listed, 1u);
-                        if (at < (u32)Cfg::LIST) list[at] = (u32)(2 * lane + u) | (u32)wy << 6 | (u32)(m + b) << 10;
+                        if (at < (u32)Cfg::LIST) list[at] = (u32)(2 * lane + u) | (u32)wy << 6 | (u32)m << 10;
                         else res[u] = heat_fp64_cell<R, ISO>(in, g, c, x + u, y, z);
                     }
             }
             const int zs = images ? (z < R ? nz : (z >= nz - R ? -nz : 0)) : 0;
-            double *p = optr + b * pitch_z;
-            put(p, res);
+            if (plain) *reinterpret_cast<double2 *>(optr) = make_double2(res[0], res[1]);
+            else put(optr, res);
             if (ys | zs) {
                 const int64_t dy = (int64_t)ys * pitch_y, dz = (int64_t)zs * pitch_z;
-                if (ys) put(p + dy, res);
-                if (zs) put(p + dz, res);
-                if (ys && zs) put(p + dy + dz, res);
+                if (ys) put(optr + dy, res);
+                if (zs) put(optr + dz, res);
+                if (ys && zs) put(optr + dy + dz, res);
+            }
+            optr += pitch_z;
+        }
+        bad = __syncthreads_or(!ok);
+        if (!bad && tid == 0 && issued < nplanes && issued <= m + NSLOT) {  // planes up to m are retired
+            fence_proxy_async();  // the block's generic writes to a slot before its next TMA load
+            for (; issued < nplanes && issued <= m + NSLOT; ++issued) {
+                scale[issued & (NSLOT - 1)] = 0;
+                issue(issued);
             }
         }
-        optr += ZB * pitch_z;
     }
     if (bad) {
         if (tid == 0) {
@@ -421,34 +401,32 @@ heat_fx_kernel(const __grid_constant__ CUtensorMap map, const double *__restrict
     }
 }
 
-template <int ZB, int NSLOT, int R, bool ISO>
+template <int R, bool ISO>
 cudaError_t run(const CUtensorMap *map, const double *in, double *out, const Geom &g, const FxCoef<R, ISO> &c,
-                bool images, unsigned *err, cudaStream_t s, int zmode) {
-    using Cfg = FxCfg<ZB, NSLOT, R>;
-    auto k = heat_fx_kernel<ZB, NSLOT, R, ISO>;
-    static int occ[64] = {};  // resident CTAs per SM, per device
+                bool images, unsigned *err, cudaStream_t s, double reread, int zmode) {
+    using Cfg = FxCfg<R>;
+    auto k = heat_fx_kernel<R, ISO>;
+    static int ready[64] = {};  // per device: the shared-memory limit is raised
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
-    if (!occ[dev]) {
+    if (!ready[dev]) {
         e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
         if (e != cudaSuccess) return e;
-        int o = 0;
-        e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&o, k, Cfg::NT, Cfg::SMEM);
-        if (e != cudaSuccess) return e;
-        occ[dev] = std::max(o, 1);
+        ready[dev] = 1;
     }
     const int tx = (int)((g.n[0] + Cfg::TX - 1) / Cfg::TX), ty = (int)((g.n[1] + Cfg::TY - 1) / Cfg::TY);
     const int nz = (int)g.n[2];
-    const int chunks = choose_zchunks(tx * ty, nz, occ[dev] * device_sms(), 0.7);
+    const int chunks = choose_zchunks(tx * ty, nz, device_sms(), reread);  // one CTA per SM
     const int zc = zchunk_len((nz + chunks - 1) / chunks, nz, zmode);
     dim3 grid(tx, ty, (unsigned)((nz + zc - 1) / zc));
     return launch_pdl(k, grid, dim3(Cfg::NT), Cfg::SMEM, s, *map, in, out, g, c, zc, images ? 1 : 0, err);
 }
 
-// Launch shapes over the one 64 x 16 tile: (ZB planes per iteration, NSLOT ring depth).
-#define FX_VARIANTS(X) X(1, 16) X(2, 16) X(4, 16) X(3, 16)
+// The variants differ in how z is split into chunks: the weight that choose_zchunks gives the
+// 2R planes each chunk converts again against SMs left idle in the last wave.
+constexpr double FX_REREAD[] = {0.7, 0.35, 1.0, 0.0};
 
 template <int R, bool ISO>
 cudaError_t dispatch(int variant, const CUtensorMap *map, const double *in, double *out, const Geom &g,
@@ -466,12 +444,8 @@ cudaError_t dispatch(int variant, const CUtensorMap *map, const double *in, doub
     c.g0 = dc.g0;
     for (int a = 0; a < 3; ++a)
         for (int b = 0; b < R; ++b) c.ga[a][b] = dc.ga[a][b];
-    int i = 0;
-#define X(ZB, NS) \
-    if (i++ == variant) return run<ZB, NS, R, ISO>(map, in, out, g, c, images, err, s, zmode);
-    FX_VARIANTS(X)
-#undef X
-    return cudaErrorInvalidValue;
+    if (variant < 0 || variant >= 4) return cudaErrorInvalidValue;
+    return run<R, ISO>(map, in, out, g, c, images, err, s, FX_REREAD[variant], zmode);
 }
 
 template <int R>
@@ -503,8 +477,8 @@ bool diffusion_fx_fits(const DiffCoef &dc) {
 }
 
 void diffusion_fx_box(int r, int box[3]) {
-    box[0] = FxCfg<4, 16, 3>::TXP;
-    box[1] = FxCfg<4, 16, 3>::TY + 2 * r;
+    box[0] = FxCfg<3>::TXP;
+    box[1] = FxCfg<3>::TY + 2 * r;
     box[2] = 1;
 }
 
