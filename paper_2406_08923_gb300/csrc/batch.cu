@@ -102,7 +102,7 @@ struct Req {
     float *w = nullptr, *kc = nullptr;  // RK register and Kahan terms, 8 fields interleaved per cell
     CUtensorMap *dmaps = nullptr;  // [2][nf] descriptors in device memory
     CUtensorMap hmaps[16];         // host copy the upload reads from (lives as long as the request)
-    int tiles[3] = {1, 1, 1}, zc = 1;
+    int tiles[2] = {1, 1};  // xy tiles (xcorr: chunks, 1); z is split per iteration (split_z)
     float g0 = 0, ga[3][3] = {};
     MK<float> k{};
     float w7[7] = {};
@@ -134,6 +134,10 @@ struct stencil_server {
     unsigned *err = nullptr;
     int grid_heat = 0, grid_mhd = 0, grid_xc = 0;
     int heat_shape = 0, mhd_shape = 0;  // tile shapes of the batched heat / MHD kernels
+    // z-chunk lengths of the active heat / MHD problems, chosen again when the active set changes
+    int zc_heat = 32, zc_mhd = 32;
+    bool regroup = true;
+    int n_done = 0;
     bool own_stream = false;
     // one captured graph per pinned table buffer: table upload + every batched launch
     cudaGraph_t graph[2] = {};  // kept alive: exec node updates refer to its nodes
@@ -223,6 +227,7 @@ stencil_status admit(stencil_server_t s, Req *r) {
     }
     r->cur = 0;
     r->state = ST_ACTIVE;
+    s->regroup = true;
     s->used += (int64_t)r->bytes;
     s->peak = std::max(s->peak, s->used);
     s->active.push_back(r);
@@ -242,8 +247,31 @@ stencil_status finish(stencil_server_t s, Req *r) {
     }
     SCK(s, cudaEventRecord(r->ev, st), "completion event");
     r->state = ST_COMPLETING;
+    s->regroup = true;
     s->completing.push_back(r);
     return STENCIL_OK;
+}
+
+// z-chunk length of the active problems of one kind on `slots` resident CTAs: the one with the least
+// estimated time, full waves of CTAs that each stream zc planes, their 2 R halo planes and about
+// four planes' worth of start-up.  One 56^3 MHD problem alone fills 56 CTAs with chunks of 32
+// planes, and its substep took as long as 38 planes one after another; in chunks of 8 it fills 196.
+// Chunking never changes the results.
+int split_z(stencil_server_t s, stencil_kind kind, int slots) {
+    int best = 32;
+    int64_t least = -1;
+    for (int zc : {48, 32, 24, 16, 12, 8, 6, 4}) {
+        int64_t ctas = 0, longest = 0;
+        for (const Req *r : s->active)
+            if (r->kind == kind) {
+                const int64_t nz = r->g.n[2], len = std::min<int64_t>(zc, nz);
+                ctas += (int64_t)r->tiles[0] * r->tiles[1] * ((nz + len - 1) / len);
+                longest = std::max(longest, len);
+            }
+        const int64_t cost = (ctas + slots - 1) / slots * (longest + 2 * R + 4);
+        if (least < 0 || cost < least) { least = cost; best = zc; }
+    }
+    return best;
 }
 
 struct TableLayout {
@@ -259,10 +287,10 @@ TableLayout table_layout(int max_active) {
     return t;
 }
 
-// Capture, for each pinned table buffer, one iteration: table upload followed by the
-// persistent batched launches of every kind.  The grids are occupancy-sized and the kernels
-// read their work counts from the uploaded table, so one graph serves every batch; only the
-// upload size changes between replays.
+// Capture, for each pinned table buffer, one iteration: table upload, then one branch per kind of
+// persistent batched launches (the problems are independent, and a small batch leaves SMs to the
+// other kinds).  The grids are occupancy-sized and the kernels read their work counts from the
+// uploaded table, so one graph serves every batch; only the upload size changes between replays.
 stencil_status capture_graphs(stencil_server_t s) {
     const TableLayout t = table_layout(s->max_active);
     const BatchHeader *dhdr = reinterpret_cast<const BatchHeader *>(s->dev_tab);
@@ -270,16 +298,31 @@ stencil_status capture_graphs(stencil_server_t s) {
         cudaGraph_t graph = nullptr;
         SCK(s, cudaStreamBeginCapture(s->stream, cudaStreamCaptureModeThreadLocal), "begin capture");
         cudaError_t e = cudaMemcpyAsync(s->dev_tab, s->host_tab[i], s->table_bytes, cudaMemcpyHostToDevice, s->stream);
+        // what is captured after `branch()` depends on the upload alone
+        cudaGraphNode_t upload = nullptr;
+        if (e == cudaSuccess) {
+            cudaStreamCaptureStatus status;
+            const cudaGraphNode_t *deps = nullptr;
+            size_t ndeps = 0;
+            e = cudaStreamGetCaptureInfo(s->stream, &status, nullptr, nullptr, &deps, nullptr, &ndeps);
+            if (e == cudaSuccess && ndeps != 1) e = cudaErrorInvalidValue;
+            if (e == cudaSuccess) upload = deps[0];
+        }
+        auto branch = [&]() {
+            return cudaStreamUpdateCaptureDependencies(s->stream, &upload, nullptr, 1, cudaStreamSetCaptureDependencies);
+        };
         if (e == cudaSuccess)
             e = launch_diffusion_batch(s->heat_shape, dhdr, reinterpret_cast<const BatchHeat *>(s->dev_tab + t.off_heat),
                                        s->err, s->grid_heat, s->stream);
+        if (e == cudaSuccess) e = branch();
+        if (e == cudaSuccess)
+            e = launch_xcorr_batch(dhdr, reinterpret_cast<const BatchXcorr *>(s->dev_tab + t.off_xc), s->err,
+                                   s->grid_xc, s->stream);
+        if (e == cudaSuccess) e = branch();
         for (int sub = 0; sub < 3 && e == cudaSuccess; ++sub)
             e = launch_mhd_batch(s->mhd_shape, dhdr,
                                  reinterpret_cast<const BatchMhd *>(s->dev_tab + t.off_mhd + sub * t.mhd_stride), sub,
                                  s->err, s->grid_mhd, s->stream);
-        if (e == cudaSuccess)
-            e = launch_xcorr_batch(dhdr, reinterpret_cast<const BatchXcorr *>(s->dev_tab + t.off_xc), s->err,
-                                   s->grid_xc, s->stream);
         cudaError_t e2 = cudaStreamEndCapture(s->stream, &graph);
         if (e != cudaSuccess) {
             if (graph) cudaGraphDestroy(graph);
@@ -457,11 +500,8 @@ stencil_status stencil_server_submit(stencil_server_t s, const stencil_request *
             mhd_scaled_constants(c, &r->k);
             mhd_batch_tile(s->mhd_shape, &tx, &ty, box);
         }
-        const int nz = (int)r->g.n[2];
-        r->zc = std::min(nz, 32);
         r->tiles[0] = (int)((r->g.n[0] + tx - 1) / tx);
         r->tiles[1] = (int)((r->g.n[1] + ty - 1) / ty);
-        r->tiles[2] = (nz + r->zc - 1) / r->zc;
     }
     // device bytes held while resident
     size_t b = 2 * r->nf * up256(r->field_elems * sizeof(float));
@@ -493,6 +533,7 @@ stencil_status stencil_server_progress(stencil_server_t s, int *n_pending, int *
             r->base = nullptr;
             s->used -= (int64_t)r->bytes;
             r->state = ST_DONE;
+            ++s->n_done;
             s->cell_updates += r->ncell * (int64_t)r->nsteps;
             s->completing[i] = s->completing.back();
             s->completing.pop_back();
@@ -523,7 +564,14 @@ stencil_status stencil_server_progress(stencil_server_t s, int *n_pending, int *
         const size_t off_xc = off_mhd + 3 * mhd_stride;
         BatchHeat *hh = reinterpret_cast<BatchHeat *>(h + off_heat);
         BatchXcorr *hx = reinterpret_cast<BatchXcorr *>(h + off_xc);
+        if (s->regroup) {
+            s->zc_heat = split_z(s, STENCIL_DIFFUSION, s->grid_heat);
+            s->zc_mhd = split_z(s, STENCIL_MHD8, s->grid_mhd);
+            s->regroup = false;
+        }
         for (Req *r : s->active) {
+            const int nz = (int)r->g.n[2], zc = std::min(nz, r->kind == STENCIL_MHD8 ? s->zc_mhd : s->zc_heat);
+            const int tiles_z = (nz + zc - 1) / zc;
             if (r->kind == STENCIL_DIFFUSION) {
                 BatchHeat &it = hh[hdr->n_heat++];
                 it.map = r->dmaps + r->cur;
@@ -531,12 +579,12 @@ stencil_status stencil_server_progress(stencil_server_t s, int *n_pending, int *
                 it.g = r->g;
                 it.g0 = r->g0;
                 std::memcpy(it.ga, r->ga, sizeof(it.ga));
-                it.zc = r->zc;
+                it.zc = zc;
                 it.tiles_x = r->tiles[0];
                 it.tiles_y = r->tiles[1];
-                it.tiles_z = r->tiles[2];
+                it.tiles_z = tiles_z;
                 it.cta_begin = hdr->heat_ctas;
-                hdr->heat_ctas += r->tiles[0] * r->tiles[1] * r->tiles[2];
+                hdr->heat_ctas += r->tiles[0] * r->tiles[1] * tiles_z;
             } else if (r->kind == STENCIL_MHD8) {
                 for (int sub = 0; sub < 3; ++sub) {
                     BatchMhd &it = reinterpret_cast<BatchMhd *>(h + off_mhd + sub * mhd_stride)[hdr->n_mhd];
@@ -547,14 +595,14 @@ stencil_status stencil_server_progress(stencil_server_t s, int *n_pending, int *
                     it.kc = r->kc;
                     it.g = r->g;
                     it.k = r->k;
-                    it.zc = r->zc;
+                    it.zc = zc;
                     it.tiles_x = r->tiles[0];
                     it.tiles_y = r->tiles[1];
-                    it.tiles_z = r->tiles[2];
+                    it.tiles_z = tiles_z;
                     it.cta_begin = hdr->mhd_ctas;
                 }
                 hdr->n_mhd++;
-                hdr->mhd_ctas += r->tiles[0] * r->tiles[1] * r->tiles[2];
+                hdr->mhd_ctas += r->tiles[0] * r->tiles[1] * tiles_z;
             } else {
                 BatchXcorr &it = hx[hdr->n_xc++];
                 it.in = r->set[r->cur][0];
@@ -593,11 +641,7 @@ stencil_status stencil_server_progress(stencil_server_t s, int *n_pending, int *
     }
     if (n_pending) *n_pending = (int)s->pending.size();
     if (n_active) *n_active = (int)(s->active.size() + s->completing.size());
-    if (n_done) {
-        int d = 0;
-        for (auto &kv : s->table) d += kv.second->state == ST_DONE;
-        *n_done = d;
-    }
+    if (n_done) *n_done = s->n_done;
     return STENCIL_OK;
 }
 
@@ -633,6 +677,7 @@ stencil_status stencil_server_cancel(stencil_server_t s, int64_t ticket) {
             if (s->active[a] == r) {
                 s->active[a] = s->active.back();
                 s->active.pop_back();
+                s->regroup = true;
                 break;
             }
         // the iteration already launched may still read the block: free it in stream order
