@@ -606,8 +606,10 @@ stencil_status stencil_create(int ndim, const int64_t dims[3], int radius, const
         return st;
     }
     // the launch shape for this size; all shapes give the same bits (stencil_set_variant, stencil_autotune)
-    if (kind == STENCIL_MHD8) mhd_default(storage_code(storage), g, &p->variant, &p->zmode);
-    else if (kind == STENCIL_DIFFUSION && storage == STENCIL_F32 && ndim == 3) p->variant = diffusion_f32_default(radius, g);
+    if (kind == STENCIL_MHD8) {
+        p->mconst.fx = storage == STENCIL_F64 && mhd_fx_applies(p->mconst, g);
+        mhd_default(storage_code(storage), g, p->mconst.fx, &p->variant, &p->zmode);
+    } else if (kind == STENCIL_DIFFUSION && storage == STENCIL_F32 && ndim == 3) p->variant = diffusion_f32_default(radius, g);
     else if (kind == STENCIL_DIFFUSION && storage == STENCIL_F32 && ndim == 2) p->variant = diffusion2d_default(radius, g);
     *out = p;
     return STENCIL_OK;
@@ -726,14 +728,14 @@ static stencil_status run_pass(stencil_t p, void *const *src, void *const *dst, 
         return STENCIL_OK;
     }
     int box[3];
-    mhd_box(storage_code(p->storage), p->variant, box);
+    mhd_box(storage_code(p->storage), p->variant, p->mconst.fx, box);
     MhdMaps maps;
     for (int q = 0; q < 8; ++q) {
         stencil_status st = tma_map(p, src[q], box, &maps.m[q]);
         if (st != STENCIL_OK) return st;
     }
     Ptrs8 none{};
-    CK(p, launch_mhd(storage_code(p->storage), 0, sub, maps, ptrs(dst, 8), p->w[0], p->kc[0], none,
+    CK(p, launch_mhd(storage_code(p->storage), 0, sub, maps, ptrs(src, 8), ptrs(dst, 8), p->w[0], p->kc[0], none,
                      g, p->mconst, true, p->err, s, p->variant, p->zmode),
        "mhd launch");
     return STENCIL_OK;
@@ -907,14 +909,14 @@ stencil_status stencil_mhd_rhs(stencil_t p, void *const *fields, void *const *rh
     CK(p, launch_halo_fill(p->geom, p->radius, p->esize, ptrs(fields, 8), 8, s, p->bc == STENCIL_BC_PERIODIC),
        "halo_fill launch");
     int box[3];
-    mhd_box(storage_code(p->storage), p->variant, box);
+    mhd_box(storage_code(p->storage), p->variant, p->mconst.fx, box);
     MhdMaps maps;
     for (int q = 0; q < 8; ++q) {
         st = tma_map(p, fields[q], box, &maps.m[q]);
         if (st != STENCIL_OK) return st;
     }
     Ptrs8 none{};
-    CK(p, launch_mhd(storage_code(p->storage), 1, 0, maps, none, nullptr, nullptr, ptrs(rhs, 8), p->geom, p->mconst,
+    CK(p, launch_mhd(storage_code(p->storage), 1, 0, maps, ptrs(fields, 8), none, nullptr, nullptr, ptrs(rhs, 8), p->geom, p->mconst,
                      false, p->err, s, p->variant, p->zmode),
        "mhd rhs launch");
     return STENCIL_OK;
@@ -989,7 +991,7 @@ static const char *variant_name(stencil_t p, int v) {
     if (p->kind == STENCIL_DIFFUSION && p->ndim == 2)
         return v == 1 ? "stream2d_tb2" : v == 2 ? "stream2d_tb4" : "tile2d_32vx_by8_ry4";
     if (p->kind == STENCIL_DIFFUSION) return diffusion_variant_name(storage_code(p->storage), p->radius, v);
-    if (p->kind == STENCIL_MHD8) return mhd_variant_name(storage_code(p->storage), v);
+    if (p->kind == STENCIL_MHD8) return mhd_variant_name(storage_code(p->storage), v, p->mconst.fx);
     return f64 ? "runtime_chunk_scalar_temporal_blocking" : "chunk2184_v9_temporal_blocking";
 }
 

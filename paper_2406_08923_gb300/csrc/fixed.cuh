@@ -82,6 +82,8 @@ __device__ __forceinline__ double fx_small_to_double(long long v, int ex) {
 // Accumulators of sum W s with W = 2^28 wh + wl, s = 2^32 sh + sl (all unsigned).
 struct FxAcc {
     u64 hh = 0, m1 = 0, m2 = 1ull << 24, ll = 0;  // m2 starts at half of the last place kept
+    FxAcc() = default;
+    __device__ __forceinline__ explicit FxAcc(u64 half) : m2(half) {}
     __device__ __forceinline__ void mac(u32 wh, u32 wl, u64 s) {
         const u32 sh = (u32)(s >> 32), sl = (u32)s;
         hh += (u64)wh * sh;
@@ -92,6 +94,33 @@ struct FxAcc {
     // sum W s / 2^57, rounded, modulo 2^64, less the bias the caller folded into `corr`
     __device__ __forceinline__ long long result(u64 corr) const {
         return (long long)((hh << 3) + ((m2 + (m1 >> 4) + (ll >> 32)) >> 25) + corr);
+    }
+    __device__ __forceinline__ void add(const FxAcc &o) {
+        hh += o.hh;
+        m1 += o.m1;
+        m2 += o.m2;
+        ll += o.ll;
+    }
+    // sum W s / 2^60 as a double times 2^(ex - 1082), for weights of 60 bits whose sum is at most 2^60,
+    // up to 12 of them, and sums that may cancel (m2 started at 0): 28 bits below the last place
+    // of the integer are kept.  A negative sum is up to 2^-32 of that place short, a zero is exact.
+    __device__ __forceinline__ double wide(u64 corr, int ex) const {
+        const u64 x = m2 + (m1 >> 4) + (ll >> 32);
+        const u64 r = hh + (x >> 28) + corr;
+        const u32 s = (u32)((long long)r >> 63);
+        u32 a = (u32)(r >> 32) ^ s, b = (u32)r ^ s, c = ((u32)x << 4) ^ s;
+#pragma unroll 1
+        for (int i = 0; i < 2 && a == 0u; ++i) {  // the leading bit into a (a branch that is rarely taken)
+            a = b;
+            b = c;
+            c = 0u;
+            ex -= 32;
+        }
+        const int n = __clz((int)a);
+        const u32 hi = __funnelshift_l(b, a, n), lo = __funnelshift_l(c, b, n);  // leading bit: bit 63
+        const u64 m = (((u64)hi << 32 | lo) >> 11) + ((lo >> 10) & 1u);          // bit 52, or 53 after a carry
+        const u32 f = a == 0u ? 0u : (u32)(ex - n + 3) << 20;
+        return __hiloint2double((int)(((u32)(m >> 32) + f) | (s & 0x80000000u)), (int)(u32)m);
     }
 };
 

@@ -145,12 +145,15 @@ int diffusion2d_default(int r, const Geom &g);  // variant a 2D FP32 plan starts
 cudaError_t launch_diffusion2d_tb(int dtype, int steps, const void *in, void *out, const Geom &g, const DiffCoef &c,
                                   cudaStream_t s);
 
+template <typename C> struct MK;
+
 // MHD8 (Eqs. A1-A4 + RK3).  Constants in the compute type are built inside mhd.cu.
 struct MhdConst {
     double d1[3][3], d2c[3], d2[3][3], dm[3][3];  // scaled stencil weights
     double cs0sq, gamma, inv_cp, lnrho0, nu, eta, zeta, mu0, inv_mu0, cp_gm1;
     double K;  // heat conductivity of Eq. A3 (0: no conduction term)
     double dt;
+    bool fx;   // FP64: the plan runs the fixed-point kernel (mhd_fx_applies)
 };
 struct MhdMaps {
     CUtensorMap m[8];
@@ -161,14 +164,18 @@ struct MhdMaps {
 // The RK register w and the Kahan terms c are one array each, in the storage type, with the 8
 // fields of a cell next to each other (element 8 cell + q; `cell` the dense interior index),
 // so a cell's 8 values move as 16-byte vectors.
-cudaError_t launch_mhd(int storage, int mode, int sub, const MhdMaps &maps, const Ptrs8 &fout,
+cudaError_t launch_mhd(int storage, int mode, int sub, const MhdMaps &maps, const Ptrs8 &fin, const Ptrs8 &fout,
                        void *w, void *kc, const Ptrs8 &rhs, const Geom &g,
                        const MhdConst &k, bool images, unsigned *err, cudaStream_t s,
                        int variant, int zmode = 0);
-void mhd_box(int storage, int variant, int box[3]);
-void mhd_default(int storage, const Geom &g, int *variant, int *zmode);  // what a plan starts with
+bool mhd_fx_applies(const MhdConst &c, const Geom &g);
+cudaError_t launch_mhd_fx(int mode, int sub, const MhdMaps &maps, const Ptrs8 &fin, const Ptrs8 &fout, void *w,
+                          const Ptrs8 &rhs, const Geom &g, const MhdConst &c, const MK<double> &k, bool images,
+                          unsigned *err, cudaStream_t s, int variant, int zmode);
+void mhd_box(int storage, int variant, bool fx, int box[3]);
+void mhd_default(int storage, const Geom &g, bool fx, int *variant, int *zmode);  // what a plan starts with
 int mhd_num_variants(int storage);
-const char *mhd_variant_name(int storage, int variant);
+const char *mhd_variant_name(int storage, int variant, bool fx);
 
 // Norms: two-pass deterministic FP64 reduction.  partials holds nblocks * nfields * 4.
 int norms_blocks();

@@ -26,84 +26,9 @@
 #include <algorithm>
 #include <cstddef>
 
-#include "mhd_rhs.cuh"
+#include "mhd_win.cuh"
 
 namespace stn {
-
-// The 7-plane window of all fields around one cell: p[k] points at the cell (field 0) in
-// plane z + k - 3; field q is FE elements further, row neighbours RS elements apart.  Its
-// 6th-order central differences (weights pre-scaled by the grid spacing) are written out one
-// IEEE operation at a time (mhd_rhs.cuh says why).
-template <typename C, typename S, int FE, int RS>
-struct Win {
-    const S *p[7];
-    __device__ __forceinline__ C at(int q, int k, int dx, int dy) const {
-        return to_c<C>(p[k][q * FE + dy * RS + dx]);
-    }
-    __device__ __forceinline__ C val(int q) const { return at(q, 3, 0, 0); }
-    // value at offset s along axis (0: x, 1: y, 2: z)
-    __device__ __forceinline__ C ax(int q, int axis, int s) const {
-        return axis == 0 ? at(q, 3, s, 0) : axis == 1 ? at(q, 3, 0, s) : at(q, 3 + s, 0, 0);
-    }
-    // first derivative: c0 (f1 - f-1) + c1 (f2 - f-2) + c2 (f3 - f-3)
-    __device__ __forceinline__ C d1(int q, int axis, const C *c) const {
-        C a = mul(c[0], sub(ax(q, axis, 1), ax(q, axis, -1)));
-        a = fmad(c[1], sub(ax(q, axis, 2), ax(q, axis, -2)), a);
-        return fmad(c[2], sub(ax(q, axis, 3), ax(q, axis, -3)), a);
-    }
-    // second derivative: c0 f0 + c1 (f1 + f-1) + c2 (f2 + f-2) + c3 (f3 + f-3)
-    __device__ __forceinline__ C d2(int q, int axis, C c0, const C *c) const {
-        C a = mul(c0, ax(q, axis, 0));
-        a = fmad(c[0], add(ax(q, axis, 1), ax(q, axis, -1)), a);
-        a = fmad(c[1], add(ax(q, axis, 2), ax(q, axis, -2)), a);
-        return fmad(c[2], add(ax(q, axis, 3), ax(q, axis, -3)), a);
-    }
-    // mixed derivative of axes (a1 < a2), diagonal form:
-    // sum_a m_a [(f(+a,+a) + f(-a,-a)) - (f(+a,-a) + f(-a,+a))]
-    __device__ __forceinline__ C mx(int q, int pair, int s1, int s2) const {
-        return pair == 0 ? at(q, 3, s1, s2) : pair == 1 ? at(q, 3 + s2, s1, 0) : at(q, 3 + s2, 0, s1);
-    }
-    __device__ __forceinline__ C dmix(int q, int pair, const C *m) const {
-        C acc = mul(m[0], sub(add(mx(q, pair, 1, 1), mx(q, pair, -1, -1)), add(mx(q, pair, 1, -1), mx(q, pair, -1, 1))));
-        acc = fmad(m[1], sub(add(mx(q, pair, 2, 2), mx(q, pair, -2, -2)), add(mx(q, pair, 2, -2), mx(q, pair, -2, 2))),
-                   acc);
-        return fmad(m[2], sub(add(mx(q, pair, 3, 3), mx(q, pair, -3, -3)), add(mx(q, pair, 3, -3), mx(q, pair, -3, 3))),
-                    acc);
-    }
-};
-
-// The 8 interleaved values of one cell in the RK register / Kahan arrays (16-byte aligned):
-// loaded and stored as 16-byte vectors.
-template <typename S, typename C>
-__device__ __forceinline__ void load8(const S *p, C (&v)[8]) {
-    if constexpr (sizeof(S) == 2) {
-        const uint4 a = *reinterpret_cast<const uint4 *>(p);
-        const S *e = reinterpret_cast<const S *>(&a);
-#pragma unroll
-        for (int q = 0; q < 8; ++q) v[q] = to_c<C>(e[q]);
-    } else {
-        constexpr int PER = 16 / (int)sizeof(S);  // values per 16-byte vector
-#pragma unroll
-        for (int h = 0; h < 8 / PER; ++h) {
-            const uint4 a = reinterpret_cast<const uint4 *>(p)[h];
-            const S *e = reinterpret_cast<const S *>(&a);
-#pragma unroll
-            for (int u = 0; u < PER; ++u) v[h * PER + u] = to_c<C>(e[u]);
-        }
-    }
-}
-template <typename S>
-__device__ __forceinline__ void store8(S *p, const S (&v)[8]) {
-    constexpr int PER = 16 / (int)sizeof(S);
-#pragma unroll
-    for (int h = 0; h < 8 / PER; ++h) {
-        uint4 a;
-        S *e = reinterpret_cast<S *>(&a);
-#pragma unroll
-        for (int u = 0; u < PER; ++u) e[u] = v[h * PER + u];
-        reinterpret_cast<uint4 *>(p)[h] = a;
-    }
-}
 
 // One xy-tile of one z-chunk of one RK substep (or RHS evaluation): the whole pipeline of a
 // CTA.  `maps` points at 8 consecutive descriptors (parameter or global memory); `k` may live
@@ -313,6 +238,7 @@ static cudaError_t run(int sub, const MhdMaps &maps, const Ptrs8 &fo, void *w, v
 #define MHD_VARIANTS_BF16(X) X(32, 8, 8, 1) X(32, 8, 8, 2) X(32, 4, 8, 3) X(32, 16, 8, 1) X(64, 8, 8, 1)
 
 static const char *MHD_F64_NAMES[] = {"tx32_ty4_s8_b1", "tx16_ty8_s8_b1"};
+static const char *MHD_FX_NAMES[] = {"fx16x8", "fx16x8_more_chunks"};
 static const char *MHD_F32_NAMES[] = {"tx32_ty8_s8_b1", "tx32_ty4_s8_b2", "tx16_ty8_s8_b2", "tx32_ty16_s8_b1",
                                       "tx32_ty12_s8_b1"};
 static const char *MHD_BF16_NAMES[] = {"tx32_ty8_s8_b1", "tx32_ty8_s8_b2", "tx32_ty4_s8_b3", "tx32_ty16_s8_b1",
@@ -320,23 +246,24 @@ static const char *MHD_BF16_NAMES[] = {"tx32_ty8_s8_b1", "tx32_ty8_s8_b2", "tx32
 
 int mhd_num_variants(int storage) { return storage == 1 ? 2 : 5; }
 
-const char *mhd_variant_name(int storage, int v) {
+const char *mhd_variant_name(int storage, int v, bool fx) {
     if (v < 0 || v >= mhd_num_variants(storage)) return "?";
-    return storage == 1 ? MHD_F64_NAMES[v] : storage == 2 ? MHD_F32_NAMES[v] : MHD_BF16_NAMES[v];
+    return storage == 1 ? (fx ? MHD_FX_NAMES : MHD_F64_NAMES)[v] : storage == 2 ? MHD_F32_NAMES[v] : MHD_BF16_NAMES[v];
 }
 
 // The tile and z-chunk mode a plan starts with (one RK3 step in us, 32 x 8 with one CTA per SM
 // first).  FP32: 32 x 16 up to 5 M cells (64^3 139 -> 121, 160^3 1280 -> 1070, 200 x 230 x 70 1084 ->
 // 884), 32 x 12 beyond (256^3 4210 -> 3437, 384^3 12816 -> 10486).  BF16: 32 x 8 with two CTAs per SM
 // (64^3 153 -> 121, 200 x 150 x 171 1843 -> 1307, 256^3 4899 -> 3258).  FP64: 16 x 8 (100 x 80 x 120
-// 5028 -> 4309, 256^3 61 173 -> 60 787), except rows of up to 32 cells (32^3 178, with 16 x 8 181).
+// 5028 -> 4309), except rows of up to 32 cells (32^3 178, with 16 x 8 181); of the fixed-point kernel
+// the first.
 // Half-length chunks pay from about 2.5 M cells on (384^3 FP32 10 668 -> 10 486, 192^3 BF16 1773 ->
-// 1737; 128^3 FP32 657, with half chunks 673), in FP64 from the smallest.
-void mhd_default(int storage, const Geom &g, int *variant, int *zmode) {
+// 1737; 128^3 FP32 657, with half chunks 673), on the FP64 pipe with the 16 x 8 tile.
+void mhd_default(int storage, const Geom &g, bool fx, int *variant, int *zmode) {
     const int64_t cells = g.n[0] * g.n[1] * g.n[2];
     *zmode = cells >= 2500000 ? 1 : 0;
     if (storage == 1) {
-        *variant = g.n[0] > 32 ? 1 : 0;
+        *variant = !fx && g.n[0] > 32 ? 1 : 0;
         *zmode = *variant;
     } else if (storage == 2) {
         *variant = cells < 5000000 ? 3 : 4;
@@ -345,7 +272,8 @@ void mhd_default(int storage, const Geom &g, int *variant, int *zmode) {
     }
 }
 
-void mhd_box(int storage, int v, int box[3]) {
+void mhd_box(int storage, int v, bool fx, int box[3]) {
+    if (storage == 1 && fx) v = 1;  // the fixed-point kernel's tile is 16 x 8
     int i = 0;
     auto put = [&](int tx, int ty, int hx) {
         if (i++ == v) { box[0] = tx + 2 * hx; box[1] = ty + 2 * R6; box[2] = 1; }
@@ -357,9 +285,12 @@ void mhd_box(int storage, int v, int box[3]) {
 #undef X
 }
 
-cudaError_t launch_mhd(int storage, int mode, int sub, const MhdMaps &maps, const Ptrs8 &fo, void *w, void *kc,
+cudaError_t launch_mhd(int storage, int mode, int sub, const MhdMaps &maps, const Ptrs8 &fi, const Ptrs8 &fo, void *w, void *kc,
                        const Ptrs8 &rhs, const Geom &g, const MhdConst &c, bool images,
                        unsigned *err, cudaStream_t s, int variant, int zmode) {
+    if (storage == 1 && c.fx)
+        return launch_mhd_fx(mode, sub, maps, fi, fo, w, rhs, g, c, make_k<double>(c, RK_A[sub], RK_B[sub]), images, err, s,
+                             variant, zmode);
     int i = 0;
     cudaError_t res = cudaErrorInvalidValue;
     // the conduction term of A3 is compiled in only for launches with K != 0
