@@ -84,7 +84,10 @@ FP64_PIPE_TINSTR = 2 * 152 * 2.07e9 / 1e12  # FP64 instructions (DFMA, DADD, DMU
 # 6th-order derivatives (600 flop), the right-hand side of Eqs. A1-A4 and the 2N-storage RK
 # update, counted by tests/mhd_flops.py (checked against the oracle in test_mhd_flops.py).
 MHD_FLOPS_PER_CELL_SUBSTEP = 2465 / 3
-MHD_F64_INSTR = 600  # FP64 instructions per cell-substep the kernel executes (ncu sass counts)
+MHD_F64_INSTR = 204  # FP64 instructions per cell-substep the kernel executes (ncu sass counts)
+# 32 x 32 + 64-bit multiply-adds of the integer pipe, which the FP64 linear stencils run on: 32
+# lanes per clock and SM (28 to 30 measured with distinct operands).
+INT_PIPE_TINSTR = 32 * 152 * 2.07e9 / 1e12
 FP32_PEAK_TFLOPS = 152 * 128 * 2 * 2.07e9 / 1e12
 
 
@@ -329,12 +332,13 @@ def run_radius_sweep(L, synth, stream, hbm_peak):
                        "hbm_gbs_at_1r1w": round(gbs, 1), "frac_of_hbm": round(gbs / hbm_peak, 4),
                        "variant": p.variant()[2]}
                 if st == L.STENCIL_F64:
-                    # FP64 is bound by the FP64 pipe: 1 + 2 d r instructions per cell (2 flop each;
-                    # 1D runs 2r + 1 FMAs through the folded cross-correlation)
+                    # 1 + 2 d r multiply-adds per cell (1D: 2r + 1 of the folded cross-correlation).
+                    # 2D runs them on the FP64 pipe, 1D and 3D in fixed point on the integer
+                    # pipe, several times the FP64 peak
                     inst = (2 * r + 1) if ndim == 1 else (1 + 2 * ndim * r)
                     tf = n * inst * 2.0 / (ms / 1e3) / 1e12
                     ent["fp64_tflops"] = round(tf, 3)
-                    ent["frac_of_fp64_peak"] = round(tf / FP64_PEAK_TFLOPS, 4)
+                    ent["times_fp64_peak"] = round(tf / FP64_PEAK_TFLOPS, 4)
                 out[f"{ndim}d_{name}_r{r}"] = ent
                 p.close()
                 del a, b
@@ -372,7 +376,12 @@ def run_xcorr_radius_sweep(L, synth, stream, hbm_peak):
                 if kind == L.STENCIL_XCORR:
                     tf = n * 2.0 * (2 * r + 1) / (ms / 1e3) / 1e12
                     ent["tflops"] = round(tf, 3)
-                    ent["frac_of_fma_peak"] = round(tf / peak, 4)
+                    if st == L.STENCIL_F32:
+                        ent["frac_of_fma_peak"] = round(tf / peak, 4)
+                    else:
+                        ent["times_fp64_peak"] = round(tf / peak, 4)
+                    if st == L.STENCIL_F64 and r > 4:  # three integer multiply-adds per tap
+                        ent["frac_of_int_pipe"] = round(tf / 2 * 3 / INT_PIPE_TINSTR, 4)
                 out[f"{kname}_{name}_r{r}"] = ent
                 p.close()
                 del a, b
@@ -686,11 +695,12 @@ def run_ours(args):
                    "kernel_variant": head["variant"],
                    "l2": "inputs larger than L2 (2 x 145 MB padded FP64 fields streamed per pass)",
                    "parallelism": f"{world} independent grids (one per GPU)"},
-        "roofline": _roof("alu", achieved_tf, FP64_PEAK_TFLOPS, "TFLOP/s",
+        "roofline": _roof("hbm", achieved_gbs, hbm_peak, "GB/s",
                           traffic=_traffic("heat_f64", head["variant"]),
-                          note="FP64 nominal 1.25 TFLOP/s (recipe table: 2 FMA/clk/SM x 152 SMs x "
-                               "2.07 GHz; the wide FP64 cross-correlation reaches 99.6 % of it); 38 flop = "
-                               "19 FP64 instructions per cell-update; traffic = ncu dram bytes/launch"),
+                          note=f"{hbm_src} copy bandwidth; 16 B per cell-update; the kernel is bound by issue "
+                               "and latency of the integer pipe (64-bit fixed point), at "
+                               f"{achieved_tf / FP64_PEAK_TFLOPS:.2f} times the FP64 pipe's 1.25 TFLOP/s "
+                               "(38 flop per cell-update)"),
         "roofline_hbm": {"achieved": round(achieved_gbs, 1), "peak": hbm_peak, "unit": "GB/s",
                          "frac": round(achieved_gbs / hbm_peak, 4), "peak_source": hbm_src,
                          "bytes_per_cell": bytes_cell},
@@ -771,11 +781,13 @@ def run_extras(L, synth, stream, hbm_peak, args):
                      "mcell_updates_per_s": round(XC_N * XC_SWEEPS / (res["ms_job"] / 1e3) / 1e6, 1),
                      "launches_per_job": 1, "bound": "l2 + launch latency (4-8 MiB working set)"}
         if dt == L.STENCIL_F64:
-            # 7 FMAs (14 flop) per output and sweep on the FP64 pipe, which bounds this case
-            tf = XC_N * XC_SWEEPS * 14 / (res["ms_job"] / 1e3) / 1e12
-            out[name]["bound"] = "FP64 pipe (4 MiB working set, L2-resident)"
-            out[name]["roofline"] = _roof("alu", tf, FP64_PEAK_TFLOPS, "TFLOP/s",
-                                          note="14 flop per cell-sweep; FP64 nominal 1.25 TFLOP/s")
+            # the 10 sweeps composed into one correlation of 61 weights: three integer
+            # multiply-adds per tap, which bound this case
+            ti = XC_N * (2 * XC_SWEEPS * 3 + 1) * 3 / (res["ms_job"] / 1e3) / 1e12
+            out[name]["bound"] = "integer pipe (64-bit fixed point; 8 MiB working set, L2-resident)"
+            out[name]["roofline"] = _roof("alu", ti, INT_PIPE_TINSTR, "Tinstr/s",
+                                          note="183 multiply-adds of 32 x 32 + 64 bits per cell and job; 32 per "
+                                               "clock and SM")
     # 3D heat, 256^3, 100 steps, FP32
     res = heat_job(L, synth, L.STENCIL_F32, HEAT_N, HEAT_STEPS, w, r, stream)
     cells = HEAT_N ** 3
@@ -817,7 +829,8 @@ def run_extras(L, synth, stream, hbm_peak, args):
         "roofline": _roof("alu", tf, FP64_PEAK_TFLOPS, "TFLOP/s",
                           note=f"{MHD_FLOPS_PER_CELL_SUBSTEP:.2f} algorithmic flop per cell-substep "
                                "(tests/mhd_flops.py; an FMA is 2 flop) against the FP64 FMA peak "
-                               "2 x 2 flop/clk/SM x 152 SMs x 2.07 GHz"),
+                               "2 x 2 flop/clk/SM x 152 SMs x 2.07 GHz; the linear differences, 600 "
+                               "of the flop, run in fixed point on the integer pipe"),
         "fp64_pipe": {"instr_per_cell_substep": MHD_F64_INSTR, "achieved_tinstr_s": round(ips / 1e12, 4),
                       "peak_tinstr_s": round(FP64_PIPE_TINSTR, 4),
                       "utilisation": round(ips / 1e12 / FP64_PIPE_TINSTR, 4)},

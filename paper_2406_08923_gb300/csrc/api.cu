@@ -651,8 +651,8 @@ stencil_status stencil_halo_fill(stencil_t p, void *const *fields, void *stream)
     return STENCIL_OK;
 }
 
-// XCORR plans that run the temporally blocked, register-window kernel (csrc/xcorr.cu): radius
-// <= 4, and FP32 up to radius 32 (it beats the wide kernel there); the rest run the wide kernel.
+// XCORR plans whose sweeps of a call go several to a launch: radius <= 4, and FP32 up to radius 32
+// (csrc/xcorr.cu; it beats the wide kernels there); the rest run one sweep per launch.
 static bool xcorr_blocked(stencil_t p) {
     return p->kind == STENCIL_XCORR && (p->radius <= 4 || (p->storage == STENCIL_F32 && p->radius <= 32));
 }

@@ -3,8 +3,9 @@
 // The Euler update and the three axis Laplacians fold into one 19-point cross-correlation
 // (Eqs. 5 and 7): f' = g0 f + sum_axes sum_{a=1..3} g_{axis,a} (f(+a) + f(-a)).
 //
-// This file holds the FP64 kernel family (FP64 on GB300 is bound by the FP64 pipe, ~1/60 of
-// the FP32 rate); FP32 has its own issue-lean kernel in diffusion_f32.cu.
+// This file holds the kernel on the FP64 pipe (~1/60 of the FP32 rate), which runs where the weights
+// do not fit fixed point (diffusion_fx.cu, four times faster, runs all others), and the launch and
+// variant functions of every 3D step; FP32 has its own issue-lean kernel in diffusion_f32.cu.
 //
 // GB300 design (2.5D z-streaming):
 //   * A CTA owns a TX x TY tile of the xy-plane (TX = 32 VX, TY = BY RY) and marches along z

@@ -9,7 +9,7 @@
 // q = trunc(v 2^(1082 - E)): |q| < 2^60, and 7 bits below a double's last place at the largest
 // value.  Values are stored biased by 2^60, so that they and sums of up to 8 of them are
 // unsigned and split into 32-bit limbs for free.  A weight is an unsigned 57-bit integer
-// 2^28 wh + wl with a sign of its own.  Sums of products are exact in four 64-bit accumulators
+// 2^28 wh + wl with a sign of its own (60 bits in mhd_fx.cu, see FxAcc::wide).  Sums of products are exact in four 64-bit accumulators
 // and are rounded once, to the nearest double, at the end.
 //
 // Accuracy: truncating the values and rounding the sum costs less than 2^-58 of the scale, so an

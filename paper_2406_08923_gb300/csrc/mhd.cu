@@ -1,4 +1,5 @@
-// mhd.cu -- fused 8-field MHD step: derivatives (gamma = A B, Sec. 3.3 Eq. 8), nonlinear
+// mhd.cu -- fused 8-field MHD step (FP64 fields with tiles for more than a third of the SMs run
+// the fixed-point kernel of mhd_fx.cu): derivatives (gamma = A B, Sec. 3.3 Eq. 8), nonlinear
 // right-hand side of Eqs. A1-A4 (phi, Eq. 9) and one substep of 3-stage Runge-Kutta, all
 // in one kernel pass per substep.
 //

@@ -1,6 +1,7 @@
 // xcorr.cu -- 1D cross-correlation f'_i = sum_{j=-r..r} g_j f^_{i+j} (Sec. 3.1, Eq. 3).
 //
-// Radius 0..4 (int32, FP32, FP64) and, for FP32, 5..32.
+// FP32 of radius 0..32; int32 and FP64 of radius 0..4 where xcorr_fx.cu does not serve them: radius 0,
+// single sweeps (FP64: up to radius 2), FP64 weights that do not fit fixed point.
 //
 // GB300 design: the input (2^20 int32 = 4 MiB in the benchmark) is L2-resident and a single
 // sweep moves ~8 MB, far less than what a launch costs in latency.  So one launch performs

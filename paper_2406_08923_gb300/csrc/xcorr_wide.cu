@@ -1,6 +1,6 @@
 // xcorr_wide.cu -- 1D stencils of large radius: the cross-correlation of Eq. 3 for radius
-// 5..1024 in FP64 and 33..1024 in FP32 (the radius sweep of Sec. 5.2, Fig. 8; FP32 up to radius
-// 32 runs the temporally blocked kernel of xcorr.cu) and the max filter
+// 33..1024 in FP32 with a caller's halo (periodic: xcorr_pair.cu) and 5..1024 in FP64 where the
+// weights do not fit fixed point (xcorr_fx.cu), and the max filter
 // f'_i = max_{j=-r..r} f^_{i+j} (the nonlinear stencil of Sec. 2.1) for radius 0..1024.
 //
 // Cross-correlation.  At large radius the work is 2r+1 multiply-adds per output, so the kernel
