@@ -50,10 +50,21 @@ def _peaks():
 
 # DRAM traffic per launch of the dominant kernel from one ncu capture (profiles/), valid only
 # while the kernel source is unchanged (first 16 hex digits of sha256 of each file).
+SRC_MHD = {"mhd.cu": "7247c6ba8525b938", "mhd_win.cuh": "a8287b7e01d5801c", "mhd_rhs.cuh": "be5b445fecd5703b", "common.cuh": "3f7458d1c75ca5f9"}
+SRC_HEAT32 = {"diffusion_f32.cu": "2cacbf4617d874ff", "common.cuh": "3f7458d1c75ca5f9"}
 NCU_TRAFFIC = {
     # dram__bytes_read.sum + dram__bytes_write.sum per launch, mean of 3 launches of a 1-pass capture at
-    # the bench sizes (profiles/dram_traffic_full_size.md); MHD: the mean over the 3 RK substeps.  The
-    # records of kernels changed since their capture are left out.
+    # the bench sizes (profiles/dram_traffic_full_size.md); MHD: the mean over the 3 RK substeps
+    "heat_f64": {"variant": "fx64x16", "zmode": 0, "bytes": 150618027 + 100469845,
+                 "src": {"diffusion_fx.cu": "b8d791036485d50b", "fixed.cuh": "00ebb1ce8309c887", "common.cuh": "3f7458d1c75ca5f9"}},
+    "heat_f32": {"variant": "f32_by4_ry2_zb2_s8_m3", "zmode": 0, "bytes": 82052181 + 21760939, "src": SRC_HEAT32},
+    "heat_f32_512": {"variant": "f32_by8_ry2_zb2_s8_m2", "zmode": 0, "bytes": 586154069 + 507398315,
+                     "src": SRC_HEAT32},
+    "mhd_f32": {"variant": "tx32_ty12_s8_b1", "zmode": 1, "bytes": 5369747115 + 4896249685, "src": SRC_MHD},
+    "mhd_bf16": [
+        {"variant": "tx32_ty8_s8_b2", "zmode": 1, "bytes": 3312621312 + 2566468779, "src": SRC_MHD},
+        {"variant": "tx32_ty4_s8_b3", "zmode": 1, "bytes": 2714962944 + 2446886229, "src": SRC_MHD},
+    ],
 }
 
 
