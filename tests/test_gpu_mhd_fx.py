@@ -16,9 +16,10 @@ W2 = (-49 / 18, 3 / 2, -3 / 20, 1 / 90)
 WM = (270 / 720, -27 / 720, 2 / 720)
 
 
-def _plan(shape):
+def _plan(shape, K=0.0):
     nz, ny, nx = shape
     par = L.mhd_params(shape)
+    par.K = K
     par.dx[0], par.dx[1], par.dx[2] = 0.05, 0.06, 0.07
     par.dt = 1e-4
     p = L.Plan(3, (nx, ny, nz), 3, 8, L.STENCIL_BC_PERIODIC, L.STENCIL_MHD8, L.STENCIL_F64, L.STENCIL_F64, params=par)
@@ -72,6 +73,10 @@ def _rhs(f8, par, t):
     s2 = sum(S[a][c] ** 2 for a in range(3) for c in range(3))
     heat = t(par.eta * par.mu0) * dot(j, j) + t(2 * par.nu) * rho * s2 + t(par.zeta) * rho * div * div
     out.append(-dot(u, gs) + heat / (rho * temp))
+    if par.K:
+        gcp, gm1 = t(par.gamma) * icp, t(par.gamma - 1.0)
+        gphi = [gcp * gs[a] + gm1 * glr[a] for a in range(3)]
+        out[7] = out[7] + t(par.K) / rho * (gcp * lap(s) + gm1 * lap(lr) + dot(gphi, gphi))
     return out
 
 
@@ -100,11 +105,12 @@ def _fields(kind, shape):
 # arithmetic: its rms error may be that of a NumPy FP64 evaluation, whose order of operations
 # differs (the kernel that works in FP64 throughout reaches 1.03 of it on these fields, 1.28 where
 # cells go to FP64), plus one rounding of the result.
-@pytest.mark.parametrize("kind", ("waves", "random", "means", "tiny", "planes", "specks"))
-@pytest.mark.parametrize("shape", [(7, 59, 115)])
-def test_rhs_as_accurate_as_fp64(cuda_lib, kind, shape):
+@pytest.mark.parametrize("kind,K", [("waves", 0.0), ("random", 0.0), ("means", 0.0), ("tiny", 0.0), ("planes", 0.0),
+                                    ("specks", 0.0), ("waves", 0.7)])
+def test_rhs_as_accurate_as_fp64(cuda_lib, kind, K):
+    shape = (7, 59, 115)
     f8 = _fields(kind, shape)
-    p, par = _plan(shape)
+    p, par = _plan(shape, K)
     a = p.alloc()
     p.upload(a, f8)
     rhs = [torch.zeros(shape, dtype=torch.float64, device="cuda") for _ in range(8)]
@@ -137,6 +143,19 @@ def test_slabs_of_z_are_bit_identical(cuda_lib, kind):
     got = _step(p, f8, 2)
     twice = _step(deep, np.concatenate([f8, f8], axis=1), 2)
     assert np.array_equal(twice[:, :24], got) and np.array_equal(twice[:, 24:], got)
+
+
+@pytest.mark.parametrize("K", (0.0, 0.7))
+def test_variants_and_chunk_lengths_are_bit_identical(cuda_lib, K):
+    shape = (40, 50, 130)  # ragged tiles; chunks of 5 to 40 planes
+    f8 = 1e-3 * _fields("waves", shape)
+    p, _ = _plan(shape, K)
+    ref = _step(p, f8, 2)
+    for v in range(p.variant()[1]):
+        for zmode in range(3):
+            p.set_variant(v)
+            p.set_zmode(zmode)
+            assert np.array_equal(_step(p, f8, 2), ref), (v, zmode)
 
 
 @pytest.mark.parametrize("value", (np.inf, np.nan, 1e300, 1e-310))
