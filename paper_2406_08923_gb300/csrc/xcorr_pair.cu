@@ -27,9 +27,8 @@ constexpr int PT = 256;  // threads per CTA
 
 template <int V_> struct PairCfg {
     static constexpr int V = V_, H = PT * V, CH = 2 * H;
-    static __host__ __device__ int nwp(int r) { return (2 * r + 1 + V - 1) / V * V; }
-    static __host__ __device__ int slots(int r) { return H + nwp(r) + V; }
-    static __host__ __device__ size_t smem(int r) { return sizeof(float2) * (size_t)(slots(r) + nwp(r)); }
+    static __host__ __device__ int slots(int r) { return H + 2 * r; }
+    static __host__ __device__ size_t smem(int r) { return sizeof(float2) * (size_t)(slots(r) + 2 * r + 1); }
     static_assert(V % 2 == 1, "");
 };
 
@@ -44,7 +43,7 @@ xcorr_pair_kernel(const float *__restrict__ in, float *__restrict__ out, Geom ge
     using B = PairCfg<V>;
     constexpr int H = B::H, CH = B::CH;
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    const int tid = threadIdx.x, nw = 2 * r + 1, nwp = B::nwp(r), slots = B::slots(r);
+    const int tid = threadIdx.x, nw = 2 * r + 1, slots = B::slots(r);
     float2 *s = reinterpret_cast<float2 *>(smem_raw);
     float *sf = reinterpret_cast<float *>(smem_raw);
     float2 *ws = s + slots;
@@ -53,15 +52,13 @@ xcorr_pair_kernel(const float *__restrict__ in, float *__restrict__ out, Geom ge
     float *outx = out + geo.off[0];
     pdl_wait();
 
-    // slot i: cells c0 - r + i and c0 + H - r + i; nothing valid reads past cell c0 + CH + r - 1, the
-    // slots beyond meet zero weights and only have to be finite
+    // slot i: cells c0 - r + i and c0 + H - r + i
     if (c0 - r >= 0 && c0 + CH + r <= n) {
         const float *src = inx + (c0 - r);
-        for (int i = tid; i < H + 2 * r; i += PT) {
+        for (int i = tid; i < slots; i += PT) {
             cp_async4(&s[i].x, src + i);
             cp_async4(&s[i].y, src + H + i);
         }
-        for (int i = H + 2 * r + tid; i < slots; i += PT) s[i] = make_float2(0.f, 0.f);
     } else {
         auto cell = [&](int64_t gi) -> float {
             if (gi >= 0 && gi < n) return inx[gi];
@@ -69,13 +66,9 @@ xcorr_pair_kernel(const float *__restrict__ in, float *__restrict__ out, Geom ge
             gi %= n;
             return inx[gi < 0 ? gi + n : gi];
         };
-        for (int i = tid; i < slots; i += PT)
-            s[i] = i < H + 2 * r ? make_float2(cell(c0 - r + i), cell(c0 + H - r + i)) : make_float2(0.f, 0.f);
+        for (int i = tid; i < slots; i += PT) s[i] = make_float2(cell(c0 - r + i), cell(c0 + H - r + i));
     }
-    for (int j = tid; j < nwp; j += PT) {
-        const float w = j < nw ? wg[j] : 0.f;
-        ws[j] = make_float2(w, w);
-    }
+    for (int j = tid; j < nw; j += PT) ws[j] = make_float2(wg[j], wg[j]);
     asm volatile("cp.async.wait_all;" ::: "memory");
     __syncthreads();
 
@@ -85,8 +78,9 @@ xcorr_pair_kernel(const float *__restrict__ in, float *__restrict__ out, Geom ge
     for (int v = 0; v < V; ++v) acc[v] = make_float2(0.f, 0.f);
 #pragma unroll
     for (int q = 0; q < V - 1; ++q) x[q + V] = xp[q];
+    int j0 = 0;
 #pragma unroll 2
-    for (int j0 = 0; j0 < nwp; j0 += V) {
+    for (; j0 <= nw - V; j0 += V) {
         // the window moves by V slots a block: V - 1 of its 2V - 1 stay in registers
 #pragma unroll
         for (int q = 0; q < V - 1; ++q) x[q] = x[q + V];
@@ -98,6 +92,21 @@ xcorr_pair_kernel(const float *__restrict__ in, float *__restrict__ out, Geom ge
 #pragma unroll
             for (int v = 0; v < V; ++v) acc[v] = __ffma2_rn(w, x[v + u], acc[v]);
         }
+    }
+    // The last, partial block has its own weights only: padded with zeros it would multiply cells
+    // beyond an output's window, and 0 x infinity is NaN.
+    const int rest = nw - j0;
+    if (rest > 0) {
+#pragma unroll
+        for (int q = 0; q < V - 1; ++q) x[q] = x[q + V];
+#pragma unroll
+        for (int u = 0; u < V - 1; ++u)
+            if (u < rest) {
+                x[V - 1 + u] = xp[j0 + V - 1 + u];
+                const float2 w = ws[j0 + u];
+#pragma unroll
+                for (int v = 0; v < V; ++v) acc[v] = __ffma2_rn(w, x[v + u], acc[v]);
+            }
     }
     __syncthreads();
     const int base = tid * V;

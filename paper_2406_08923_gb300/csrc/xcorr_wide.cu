@@ -84,7 +84,7 @@ __device__ __forceinline__ void put1(T *outx, int64_t n, int r, int images, int6
 // Shared-memory layout of one staging buffer of the wide cross-correlation: the chunk's cells
 // c0 - r .. c0 + CH + r - 1 start at element `lead` = rr - r, where rr is r rounded up to whole
 // 16-byte groups, so that a bulk copy of cells c0 - rr .. c0 + CH + rr - 1 lands at element 0.
-// Past the span come zeros for the padded weight blocks.
+// Past the span come zeros that no output reads.
 template <typename T, int V_> struct WideBuf {
     static constexpr int V = V_, CH = WT * V, L = 16 / (int)sizeof(T);
     static __host__ __device__ int rr(int r) { return (r + L - 1) / L * L; }
@@ -187,7 +187,7 @@ xcorr_wide_kernel(const T *__restrict__ in, T *__restrict__ out, Geom geo, const
         bool bulk;
         ok = pp.wait(b, &bulk);
         if (ok && bulk) {
-            // cells the copy brought past the span (fewer than L) must read as 0
+            // cells the copy brought past the span (fewer than L): as in the staged chunks
             if (threadIdx.x < rr - r) buf[lead + span + threadIdx.x] = T(0);
         } else if (ok) {
             stage(pp.inx, n, c0, r, span, CH, periodic, buf + lead);
@@ -200,7 +200,8 @@ xcorr_wide_kernel(const T *__restrict__ in, T *__restrict__ out, Geom geo, const
         T acc[V];
 #pragma unroll
         for (int v = 0; v < V; ++v) acc[v] = T(0);
-        for (int j0 = 0; j0 < nwp; j0 += V) {
+        int j0 = 0;
+        for (; j0 <= nw - V; j0 += V) {
             T w[V], x[2 * V - 1];
 #pragma unroll
             for (int u = 0; u < V; ++u) w[u] = ws[j0 + u];
@@ -210,6 +211,22 @@ xcorr_wide_kernel(const T *__restrict__ in, T *__restrict__ out, Geom geo, const
             for (int u = 0; u < V; ++u)
 #pragma unroll
                 for (int v = 0; v < V; ++v) acc[v] = fma(w[u], x[v + u], acc[v]);
+        }
+        // The last, partial block has its own weights only: padded with zeros it would multiply
+        // cells beyond an output's window, and 0 x infinity is NaN.
+        const int rest = nw - j0;
+        if (rest > 0) {
+            T x[2 * V - 2];
+#pragma unroll
+            for (int q = 0; q < V - 1; ++q) x[q] = s[base + j0 + q];
+#pragma unroll
+            for (int u = 0; u < V - 1; ++u)
+                if (u < rest) {
+                    x[V - 1 + u] = s[base + j0 + V - 1 + u];
+                    const T w = ws[j0 + u];
+#pragma unroll
+                    for (int v = 0; v < V; ++v) acc[v] = fma(w, x[v + u], acc[v]);
+                }
         }
         // results through shared memory (the staged cells are no longer needed), then
         // coalesced 16-byte stores of the chunk and scalar stores of its periodic images
@@ -380,8 +397,8 @@ cudaError_t run_wide(const void *in, void *out, const Geom &g, const void *wdev,
     return cudaGetLastError();
 }
 
-// Outputs per thread V (= weights per register block): the 2r+1 weights are padded to whole
-// blocks of V, so V is chosen per radius from a few compiled sizes (all odd: lanes V cells
+// Outputs per thread V (= weights per register block): the last of the 2r+1 weights may fill a
+// block in part, so V is chosen per radius from a few compiled sizes (all odd: lanes V cells
 // apart fall on distinct banks).  A block costs V^2 multiply-adds, about 3V shared loads and
 // some address arithmetic for V outputs.  FP32 is issue-bound: the cost per output is blocks
 // x (V + 6), the 6 fitted to radius sweeps on GB300 (at r = 64 and 128, V = 15 beats V = 13
