@@ -17,11 +17,19 @@
 //     spans (S), and values of planes with a smaller one are shifted right, behind branches that
 //     are uniform per block.  S depends on nothing but those plane tiles, so results do not
 //     depend on how z is split into chunks or slabs.
-//   * With one grid spacing on all axes (ISO) the six values at distance a are summed first: four
-//     64 x 64-bit products per cell instead of ten.
-//   * Outputs whose stencil is small against S (fixed.cuh), or that meet infinities or NaN, are
-//     listed and evaluated at the end of the CTA by FP64 multiply-adds from global memory, in
-//     the order of diffusion.cu.
+//   * The pairs' sum runs in fixed point, the centre joins it in one FP64 multiply-add with its
+//     exact value: beside g0 f, which is near f when the step is small, the pairs' weights would
+//     lose their bits.
+//   * With one grid spacing on all axes (ISO) the six values at distance a are summed first: three
+//     64 x 64-bit products per cell instead of nine.
+//   * The pairs' sum is off by at most 8 units of 2^-60 of 2^ew S (2^ew: above the sum of the
+//     weights, one per distance and axis): seven of truncated and shifted values, one of rounding.
+//     The weights' own rounding costs 2^-52 of the terms they weigh at r = 3, 2^-50 at r = 4.  A
+//     chain of FP64 multiply-adds rounds each of its 1 + 6 R terms, so an output stays within the
+//     chain's bound where one of its terms is at least 2^-7 of 2^ew S: the centre's (g0 |f|), one of
+//     its four neighbours' in the plane, or the sum itself.  Outputs that show none of these, or that
+//     meet infinities or NaN, are listed and evaluated at the end of the CTA by FP64 multiply-adds
+//     from global memory, in the order of diffusion.cu.
 #include <algorithm>
 
 #include "fixed.cuh"
@@ -31,9 +39,10 @@ namespace stn {
 namespace {
 
 template <int R, bool ISO> struct FxCoef {
-    static constexpr int N = ISO ? 1 + R : 1 + 3 * R;
-    FxWeights<N> w;
-    double g0, ga[3][R];  // for the outputs evaluated in FP64
+    static constexpr int N = ISO ? R : 3 * R;
+    FxWeights<N> w;       // of the pairs
+    double g0, ga[3][R];  // the centre's; the pairs' for the outputs evaluated in FP64
+    u32 small_c, small_a[2];  // high words below which the centre and an x- or y-neighbour are small
 };
 
 template <int R> struct FxCfg {
@@ -66,12 +75,22 @@ __device__ __noinline__ double heat_fp64_cell(const double *__restrict__ in, con
     return acc;
 }
 
+// Whether two biased values' high words are below the threshold t in magnitude.
+__device__ __forceinline__ bool fx_below(u32 a, u32 b, u32 t) {
+    const u32 lo = FX_BIAS_HI - t;
+    return max(a - lo, b - lo) < 2 * t;
+}
+
 // Two neighbouring outputs: `cp` points at the first in its centre plane (scale sc - dc), z(k, u)
-// gives the value of cell u at plane offset k != 0, at scale sc; SAME: dc is 0.  Returns bit u set
-// where output u is left to FP64: the centre and its four neighbours in the plane are below 2^-6
-// of the scale.
-template <int R, bool ISO, bool SAME, int TXP, typename W, typename Z>
-__device__ __forceinline__ int fx_pair(const u64 *cp, const Z &z, int dc, int sc, const W &w, double (&res)[2]) {
+// gives the value of cell u at plane offset k != 0, at scale sc, f holds the centres' exact values;
+// SAME: dc is 0.  Returns bit u set where output u is left to FP64.
+template <int R, bool ISO, bool SAME, int TXP, typename Z>
+__device__ __forceinline__ int fx_pair(const u64 *cp, const Z &z, int dc, int sc, const FxCoef<R, ISO> &c,
+                                       const double2 f, double (&res)[2]) {
+    const FxWeights<FxCoef<R, ISO>::N> &w = c.w;
+    // the thresholds at the centre plane's scale
+    auto at_plane = [&](u32 t) { return SAME ? t : (u32)min((u64)t << min(dc, 28), (u64)FX_BIAS_HI); };
+    const u32 tc = at_plane(c.small_c), tx = at_plane(c.small_a[0]), ty = ISO ? tx : at_plane(c.small_a[1]);
     u64 X[10];  // x window: cells -4 .. 5
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
@@ -81,14 +100,11 @@ __device__ __forceinline__ int fx_pair(const u64 *cp, const Z &z, int dc, int sc
         X[2 * k + 1] = t.y;
     }
     FxAcc acc[2];
-    u32 hmx[2], hmn[2];
+    bool small[2];
 #pragma unroll
-    for (int u = 0; u < 2; ++u) {
-        const u32 a = (u32)(X[3 + u] >> 32), d = (u32)(X[5 + u] >> 32), e = (u32)(X[4 + u] >> 32);
-        hmx[u] = max(max(a, d), e);
-        hmn[u] = min(min(a, d), e);
-        acc[u].mac(w.wh[0], w.wl[0], SAME ? X[4 + u] : fx_shift(X[4 + u], FX_BIAS, dc));
-    }
+    for (int u = 0; u < 2; ++u)
+        small[u] = fx_below((u32)(X[4 + u] >> 32), (u32)(X[4 + u] >> 32), tc) &&
+                   fx_below((u32)(X[3 + u] >> 32), (u32)(X[5 + u] >> 32), tx);
     // the in-plane pairs of every distance, moved to the common scale together
     u64 sxy[2][R], sy[2][R];
 #pragma unroll
@@ -98,10 +114,7 @@ __device__ __forceinline__ int fx_pair(const u64 *cp, const Z &z, int dc, int sc
 #pragma unroll
         for (int u = 0; u < 2; ++u) {
             const u64 y1 = u ? yp.y : yp.x, y2 = u ? ym.y : ym.x;
-            if (a == 1) {
-                hmx[u] = max(hmx[u], max((u32)(y1 >> 32), (u32)(y2 >> 32)));
-                hmn[u] = min(hmn[u], min((u32)(y1 >> 32), (u32)(y2 >> 32)));
-            }
+            if (a == 1) small[u] = small[u] && fx_below((u32)(y1 >> 32), (u32)(y2 >> 32), ty);
             sxy[u][a - 1] = X[4 + u + a] + X[4 + u - a];
             sy[u][a - 1] = y1 + y2;
             if (ISO) sxy[u][a - 1] += sy[u][a - 1];
@@ -124,7 +137,7 @@ __device__ __forceinline__ int fx_pair(const u64 *cp, const Z &z, int dc, int sc
             if constexpr (ISO) {
                 u64 s = sxy[u][a - 1] + z(a, u) + z(-a, u);
                 if (neg) s = 12 * FX_BIAS - s;
-                acc[u].mac(w.wh[a], w.wl[a], s);
+                acc[u].mac(w.wh[a - 1], w.wl[a - 1], s);
             } else {
                 u64 sx = sxy[u][a - 1], s2 = sy[u][a - 1], sz = z(a, u) + z(-a, u);
                 if (neg) {
@@ -132,19 +145,19 @@ __device__ __forceinline__ int fx_pair(const u64 *cp, const Z &z, int dc, int sc
                     s2 = 4 * FX_BIAS - s2;
                     sz = 4 * FX_BIAS - sz;
                 }
-                acc[u].mac(w.wh[a], w.wl[a], sx);
-                acc[u].mac(w.wh[R + a], w.wl[R + a], s2);
-                acc[u].mac(w.wh[2 * R + a], w.wl[2 * R + a], sz);
+                acc[u].mac(w.wh[a - 1], w.wl[a - 1], sx);
+                acc[u].mac(w.wh[R + a - 1], w.wl[R + a - 1], s2);
+                acc[u].mac(w.wh[2 * R + a - 1], w.wl[2 * R + a - 1], sz);
             }
         }
     }
-    const u32 flag = SAME ? FX_FLAG_HI : (dc < 6 ? FX_FLAG_HI << dc : FX_BIAS_HI);
     int left = 0;
 #pragma unroll
     for (int u = 0; u < 2; ++u) {
         const long long v = acc[u].result(w.corr);
-        res[u] = fx_to_double(v, sc + w.ew);
-        if ((hmx[u] < FX_BIAS_HI + flag && hmn[u] >= FX_BIAS_HI - flag) || !fx_big(v)) left |= 1 << u;
+        const double sum = fx_big(v) ? fx_to_double(v, sc + w.ew) : fx_small_to_double(v, sc + w.ew);
+        res[u] = fma(c.g0, u ? f.y : f.x, sum);
+        if (small[u] && (u64)(v + (1ll << 54)) < (2ull << 54)) left |= 1 << u;
     }
     return left;
 }
@@ -306,6 +319,9 @@ heat_fx_kernel(const __grid_constant__ CUtensorMap map, const double *__restrict
     load(0);
     bool bad = __syncthreads_or(!ok);
     for (int t = 0; !bad && t <= nplanes; ++t) {
+        const int m = t - 1 - 2 * R;  // outputs of plane zc0 + m, from planes m .. t - 1
+        double2 centre = make_double2(0.0, 0.0);  // exact, for the use below
+        if (m >= 0 && nv != 0) centre = *reinterpret_cast<const double2 *>(in + (optr - out));
         // the plane's scale is complete since the barrier; its slot is read from the next one on
         if (t < nplanes) {
             convert(t);
@@ -320,7 +336,6 @@ heat_fx_kernel(const __grid_constant__ CUtensorMap map, const double *__restrict
             }
             if (t + 1 < nplanes) load(t + 1);
         }
-        const int m = t - 1 - 2 * R;  // outputs of plane zc0 + m, from planes m .. t - 1
         if (m >= 0 && nv != 0) {
             const int4 win = window[(t - 1) & 1];
             const int sc = win.x, dc = win.z, z = zc0 + m;
@@ -339,7 +354,7 @@ heat_fx_kernel(const __grid_constant__ CUtensorMap map, const double *__restrict
                 }
                 auto column = [&](int k, int u) { return Q[R + k][u]; };
                 if (!win.y) {
-                    left = fx_pair<R, ISO, true, TXP>(cp, column, 0, sc, c.w, res);
+                    left = fx_pair<R, ISO, true, TXP>(cp, column, 0, sc, c, centre, res);
                 } else {
 #pragma unroll
                     for (int k = 0; k <= 2 * R; ++k) {
@@ -348,7 +363,7 @@ heat_fx_kernel(const __grid_constant__ CUtensorMap map, const double *__restrict
                         Q[k][0] = fx_shift(Q[k][0], FX_BIAS, d);
                         Q[k][1] = fx_shift(Q[k][1], FX_BIAS, d);
                     }
-                    left = fx_pair<R, ISO, false, TXP>(cp, column, dc, sc, c.w, res);
+                    left = fx_pair<R, ISO, false, TXP>(cp, column, dc, sc, c, centre, res);
                 }
             } else {  // zeros only, or infinities, NaN, or near the ends of the exponent range
                 res[0] = res[1] = 0.0;
@@ -434,16 +449,22 @@ cudaError_t dispatch(int variant, const CUtensorMap *map, const double *in, doub
     FxCoef<R, ISO> c;
     double w[FxCoef<R, ISO>::N];
     int mult[FxCoef<R, ISO>::N];
-    w[0] = dc.g0;
-    mult[0] = 1;
-    for (int i = 1; i < FxCoef<R, ISO>::N; ++i) {
-        w[i] = dc.ga[(i - 1) / R][(i - 1) % R];
+    for (int i = 0; i < FxCoef<R, ISO>::N; ++i) {
+        w[i] = dc.ga[i / R][i % R];
         mult[i] = ISO ? 6 : 2;
     }
     if (!fx_weights<FxCoef<R, ISO>::N>(w, mult, c.w)) return cudaErrorInvalidValue;
     c.g0 = dc.g0;
     for (int a = 0; a < 3; ++a)
         for (int b = 0; b < R; ++b) c.ga[a][b] = dc.ga[a][b];
+    // A centre is small when its term is below 2^-6 of 2^ew S, a neighbour below 2^-7 of it (the first
+    // weight of equal axes is between 0.43 and 1 times 2^ew) and below 2^-6 of the scale.
+    auto threshold = [&](double weight, double share) {
+        const double t = FX_FLAG_HI * (share * std::ldexp(1.0, c.w.ew) / weight);
+        return t < FX_BIAS_HI ? (u32)t + 1 : FX_BIAS_HI;  // weight 0: every value is small
+    };
+    c.small_c = std::max(threshold(dc.g0, 1.0), 4u);
+    for (int a = 0; a < 2; ++a) c.small_a[a] = std::max(threshold(dc.ga[a][0], 0.5), FX_FLAG_HI);
     if (variant < 0 || variant >= 4) return cudaErrorInvalidValue;
     return run<R, ISO>(map, in, out, g, c, images, err, s, FX_REREAD[variant], zmode);
 }
@@ -463,17 +484,17 @@ cudaError_t dispatch_iso(int variant, const CUtensorMap *map, const double *in, 
 // range, and with the signs of a forward step that is stable or nearly so (g0 >= 0, positive at
 // odd distances, negative at even ones), which the kernel has compiled in.
 bool diffusion_fx_fits(const DiffCoef &dc) {
-    double w[13];
-    int mult[13];
-    bool signs = true;
-    for (int i = 0; i < 13; ++i) {
-        const int a = (i - 1) % 4 + 1;  // distance; weights beyond the radius are 0
-        w[i] = i == 0 ? dc.g0 : dc.ga[(i - 1) / 4][a - 1];
-        mult[i] = i == 0 ? 1 : 2;
-        signs = signs && (i == 0 || a % 2 == 1 ? w[i] >= 0.0 : w[i] <= 0.0);
+    double w[12];
+    const int mult[12] = {};
+    bool signs = std::isfinite(dc.g0) && dc.g0 >= 0.0;
+    for (int i = 0; i < 12; ++i) {
+        const int a = i % 4 + 1;  // distance; weights beyond the radius are 0
+        w[i] = dc.ga[i / 4][a - 1];
+        signs = signs && (a % 2 == 1 ? w[i] >= 0.0 : w[i] <= 0.0);
     }
-    FxWeights<13> o;
-    return signs && fx_weights<13>(w, mult, o);
+    FxWeights<12> o;
+    // 2^ew of the launch may be a quarter of this one (ISO)
+    return signs && fx_weights<12>(w, mult, o) && o.ew >= 2 - FX_EW;
 }
 
 void diffusion_fx_box(int r, int box[3]) {

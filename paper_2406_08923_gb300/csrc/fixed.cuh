@@ -8,15 +8,16 @@
 // A set of values whose largest magnitude has the (biased) exponent E is held as
 // q = trunc(v 2^(1082 - E)): |q| < 2^60, and 7 bits below a double's last place at the largest
 // value.  Values are stored biased by 2^60, so that they and sums of up to 8 of them are
-// unsigned and split into 32-bit limbs for free.  A weight is an unsigned 57-bit integer
-// 2^28 wh + wl with a sign of its own (60 bits in mhd_fx.cu, see FxAcc::wide).  Sums of products are exact in four 64-bit accumulators
-// and are rounded once, to the nearest double, at the end.
+// unsigned and split into 32-bit limbs for free.  A weight is an unsigned integer 2^28 wh + wl
+// with a sign of its own; the weights of a sum add up to at most 2^60.  Sums of products are exact in
+// four 64-bit accumulators and are rounded once, to the nearest double, at the end.
 //
-// Accuracy: truncating the values and rounding the sum costs less than 2^-58 of the scale, so an
-// output whose stencil holds a value of at least 2^-6 of the scale is no further from the exact
-// result than a chain of FP64 multiply-adds (2^-53 of its largest term).  Callers check that
-// per output and evaluate the rest in FP64; infinities, NaN and exponents near the ends of the
-// range go the same way.
+// Accuracy: what truncating the values and rounding the weights costs is a few units of 2^-60 of
+// the scale times the sum of the weights.  A chain of FP64 multiply-adds costs a few roundings,
+// 2^-53 each, of the largest TERM (weight times value): a value far below the scale, or a small
+// weight, makes the FP64 chain the more exact one.  Callers bound the terms of every output from
+// below (each kernel says how) and evaluate in FP64 where they may be small; infinities, NaN and
+// exponents near the ends of the range go the same way.
 #pragma once
 
 #include <cmath>
@@ -74,14 +75,14 @@ __device__ __forceinline__ double fx_to_double(long long v, int ex) {
 }
 // Whether fx_to_double may take v.
 __device__ __forceinline__ bool fx_big(long long v) { return (u64)(v + (1ll << 32)) >= (2ull << 32); }
-// The same for |v| <= 2^32 (exact), ex from FX_SMIN - 102 on.
+// The same for |v| <= 2^32 (exact), ex from FX_SMIN - 104 on.
 __device__ __forceinline__ double fx_small_to_double(long long v, int ex) {
     return (double)v * __hiloint2double((ex - 59) << 20, 0);  // 2^(ex - 1082)
 }
 
 // Accumulators of sum W s with W = 2^28 wh + wl, s = 2^32 sh + sl (all unsigned).
 struct FxAcc {
-    u64 hh = 0, m1 = 0, m2 = 1ull << 24, ll = 0;  // m2 starts at half of the last place kept
+    u64 hh = 0, m1 = 0, m2 = 1ull << 27, ll = 0;  // m2 starts at half of the last place kept
     FxAcc() = default;
     __device__ __forceinline__ explicit FxAcc(u64 half) : m2(half) {}
     __device__ __forceinline__ void mac(u32 wh, u32 wl, u64 s) {
@@ -91,9 +92,9 @@ struct FxAcc {
         m2 += (u64)wl * sh;
         ll += (u64)wl * sl;
     }
-    // sum W s / 2^57, rounded, modulo 2^64, less the bias the caller folded into `corr`
+    // sum W s / 2^60, rounded, modulo 2^64, less the bias the caller folded into `corr`
     __device__ __forceinline__ long long result(u64 corr) const {
-        return (long long)((hh << 3) + ((m2 + (m1 >> 4) + (ll >> 32)) >> 25) + corr);
+        return (long long)(hh + ((m2 + (m1 >> 4) + (ll >> 32)) >> 28) + corr);
     }
     __device__ __forceinline__ void add(const FxAcc &o) {
         hh += o.hh;
@@ -124,38 +125,32 @@ struct FxAcc {
     }
 };
 
-// One launch's weights: value i times 2^-ew is (2^28 wh + wl) 2^-57; `corr` takes the bias of
-// every sum off the result.  The kernels know the signs: a sum with a negative weight enters as
-// 2^61 mult - s, the biased negative.
+// One launch's weights: |value i| is (2^28 wh + wl) 2^(ew - 60); `corr` takes the bias of every sum
+// off the result.  The kernels know the signs: a sum with a negative weight enters as 2^61 mult - s,
+// the biased negative.
 template <int N> struct FxWeights {
     u32 wh[N], wl[N];
     int ew;
     u64 corr;
 };
+constexpr int FX_EW = 104;  // |ew| at most
 
-// mult[i]: how many values sum i adds.  False where fixed point does not apply (a weight is not
-// finite, all are zero, or the exponent is out of range).
+// mult[i]: how many values sum i adds (6 at most, |result| < 2^63).  False where fixed point does not
+// apply (a weight is not finite, all are zero, or the exponent is out of range).
 template <int N> inline bool fx_weights(const double *w, const int *mult, FxWeights<N> &o) {
-    double top = 0.0, sum = 0.0;
+    double sum = 0.0;
+    for (int i = 0; i < N; ++i) sum += std::fabs(w[i]);
+    if (!(sum > 0.0) || !std::isfinite(sum)) return false;
+    (void)std::frexp(sum, &o.ew);  // sum < 2^ew
+    if (o.ew < -FX_EW || o.ew > FX_EW) return false;
+    u64 bias = 0;
     for (int i = 0; i < N; ++i) {
-        if (!std::isfinite(w[i])) return false;
-        top = std::fmax(top, std::fabs(w[i]));
-        sum += mult[i] * std::fabs(w[i]);
-    }
-    if (!(top > 0.0) || !std::isfinite(sum)) return false;
-    int ew = 0;
-    (void)std::frexp(top, &ew);  // top < 2^ew
-    while (std::ldexp(sum, -ew) >= 4.0) ++ew;  // |result| < 2^62
-    if (ew < -100 || ew > 100) return false;
-    o.ew = ew;
-    u64 corr = 0;
-    for (int i = 0; i < N; ++i) {
-        const u64 W = (u64)std::llrint(std::ldexp(std::fabs(w[i]), 57 - ew));
+        const u64 W = (u64)std::llrint(std::ldexp(std::fabs(w[i]), 60 - o.ew));
         o.wh[i] = (u32)(W >> 28);
         o.wl[i] = (u32)(W & 0xfffffffu);
-        corr += W * (u64)mult[i];
+        bias += W * (u64)mult[i];
     }
-    o.corr = 0ull - 8ull * corr;  // 2^60 / 2^57 per unit
+    o.corr = 0ull - bias;
     return true;
 }
 

@@ -71,6 +71,33 @@ def test_every_output_is_as_close_as_fp64(cuda_lib, r, h, shape):
         assert worst <= 1.0, (name, worst)
 
 
+def _cold_fields(shape):
+    z, y, x = np.meshgrid(*[np.arange(n) for n in shape], indexing="ij")
+    hot = np.zeros(shape)
+    hot[4, 6, 20], hot[-3, -1, -2], hot[7, 9, 40:44] = 1.0, -0.7, 1.3
+    yield "hot cells in a cold field", hot
+    yield "hot cells in a faint field", hot + 1e-9 * np.sin(0.7 * x + 0.4 * y + 0.9 * z)
+    yield "hot spot", np.exp(-((x - 30.3) ** 2 + (y - 8.1) ** 2 + (z - 9.2) ** 2) / 18.0)
+    yield "front", np.where(x < 33, 1.0 + 0.1 * np.sin(0.5 * y), 1e-12 * np.cos(0.3 * z + y))
+    yield "large mean", 1.0 + 1e-8 * np.sin(0.3 * x + 0.2 * y + 0.25 * z)
+
+
+# small steps, and axes whose weights are far below the others': terms of small weight times a
+# large value, or of a large weight times a small value, carry the output
+@pytest.mark.parametrize("r,h", [(1, (0.5, 0.5, 0.5)), (2, (0.4, 0.5, 0.6)), (3, (0.5, 0.5, 0.5)), (3, (50.0, 0.5, 0.5)),
+                                 (3, (0.5, 0.5, 50.0)), (4, (0.5, 0.5, 0.5)), (4, (0.5, 60.0, 0.45))])
+@pytest.mark.parametrize("dt", [0.02, 1e-3, 1e-4, 1e-6, 1e-9])
+def test_every_output_is_as_close_as_fp64_at_small_steps(cuda_lib, r, h, dt):
+    shape = (21, 18, 70)
+    p = _plan(shape, r, h, dt)
+    for name, f in list(_cold_fields(shape)) + list(_fields(shape, 6)):
+        got, _ = _step(p, f)
+        ref, mag = _reference(f, r, h, dt)
+        bound = (1 + 6 * r + 2) * 2.0 ** -53 * mag + 2.0 ** -1074  # as above
+        worst = float(np.max(np.abs(got - ref) / bound))
+        assert worst <= 1.0, (name, worst)
+
+
 def test_infinities_and_nan_spread_as_in_fp64(cuda_lib):
     shape, r, h = (20, 20, 70), 3, (0.5, 0.5, 0.5)
     f = np.random.default_rng(3).standard_normal(shape)
