@@ -11,8 +11,9 @@
 //   * Between two block barriers a CTA works on three planes at once: it converts plane t in place
 //     (a thread's share, held in registers since the last interval) to biased 60-bit integers at
 //     the plane's scale, loads its share of plane t + 1 and reduces the largest exponent, and
-//     computes the outputs of plane t - R - 1.  One barrier per plane, and the warps overlap the
-//     three (two barriers with the phases one after another took 264 us per 256^3 step, this 235).
+//     computes the outputs of plane t - R - 1.  Half of the warps of each scheduler compute first and
+//     half convert first, so that they wait for different things (256^3, r = 3: 244 us per step with all
+//     in one order, 235 like this).
 //   * A thread owns 2 x-cells.  An output uses the largest scale of the 2R+1 planes its z column
 //     spans (S), and values of planes with a smaller one are shifted right, behind branches that
 //     are uniform per block.  S depends on nothing but those plane tiles, so results do not
@@ -26,10 +27,19 @@
 //     weights, one per distance and axis): seven of truncated and shifted values, one of rounding.
 //     The weights' own rounding costs 2^-52 of the terms they weigh at r = 3, 2^-50 at r = 4.  A
 //     chain of FP64 multiply-adds rounds each of its 1 + 6 R terms, so an output stays within the
-//     chain's bound where one of its terms is at least 2^-7 of 2^ew S: the centre's (g0 |f|), one of
-//     its four neighbours' in the plane, or the sum itself.  Outputs that show none of these, or that
-//     meet infinities or NaN, are listed and evaluated at the end of the CTA by FP64 multiply-adds
-//     from global memory, in the order of diffusion.cu.
+//     chain's bound where one of its terms is at least 2^-6 (r = 1), 2^-7 (r = 2), 2^-8 of 2^ew S: the
+//     centre's (g0 |f|), one of its six neighbours', or the sum itself.  Outputs that show none of
+//     these are listed and evaluated by FP64 multiply-adds from global memory, in the order of
+//     diffusion.cu, by all threads, every four planes if they are many and else at the end.
+//   * A field that falls by more than the scale holds within a tile (a hot spot, a front) has mostly
+//     such outputs.  A plane's outputs are all evaluated in FP64, with coalesced loads and without the
+//     fixed-point sums, where a row in the middle of its tile lies 2^-8 and more below the plane's
+//     largest value over half its length, and where its window meets infinities, NaN or the ends
+//     of the exponent range.
+//   * 256^3, r = 3, us per step, the FP64 pipe's kernel and this one: waves 596 and 235; a Gaussian of
+//     8, 16, 32 cells 596 and 696, 672, 290; a front of 3 cells 595 and 531; waves at r = 1, 2, 4 221
+//     and 194, 424 and 215, 821 and 261; 32^3 14.5 and 10.2.  A field of which nothing fits pays for the
+//     exponents and the conversion beside the FP64 pipe's work, at r = 1 up to 1.45 times (221, 321).
 #include <algorithm>
 
 #include "fixed.cuh"
@@ -42,7 +52,7 @@ template <int R, bool ISO> struct FxCoef {
     static constexpr int N = ISO ? R : 3 * R;
     FxWeights<N> w;       // of the pairs
     double g0, ga[3][R];  // the centre's; the pairs' for the outputs evaluated in FP64
-    u32 small_c, small_a[2];  // high words below which the centre and an x- or y-neighbour are small
+    u32 small_c, small_a[3];  // high words below which the centre and a neighbour on each axis are small
 };
 
 template <int R> struct FxCfg {
@@ -50,10 +60,12 @@ template <int R> struct FxCfg {
     static constexpr int TX = 64, TY = BY, HX = 4, TXP = TX + 2 * HX, ROWS = TY + 2 * R;
     static constexpr int PAIRS = TXP / 2 * ROWS;  // 16-byte pairs per plane tile
     static constexpr int KP = (PAIRS + NT - 1) / NT;
+    // The last warp has one pair per thread to convert, of one row, and so the time for what is done once per plane.
+    static_assert(KP == 2 && PAIRS - NT <= NT - 32, "");
     static constexpr int SLOT = ((TXP * ROWS * 8 + 127) / 128) * 128 / 8;
     static constexpr uint32_t BOX_BYTES = TXP * ROWS * 8;
     static constexpr size_t SMEM = (size_t)NSLOT * SLOT * 8 + 128;
-    static constexpr int LIST = 1024;
+    static constexpr int LIST = 2048, LIST_HIGH = 256;  // listed outputs; more are worked off before the end
     static_assert((NSLOT & (NSLOT - 1)) == 0, "ring depth is a power of two (slot = j & (NSLOT-1))");
     static_assert(NSLOT >= 2 * R + 4, "ring: an output's planes, the two being converted and loaded, one refill");
     static_assert(R >= 1 && R <= 4, "");
@@ -75,6 +87,41 @@ __device__ __noinline__ double heat_fp64_cell(const double *__restrict__ in, con
     return acc;
 }
 
+// Two neighbouring outputs in the same way; p points at the first, 16-byte aligned, w holds g0 and
+// ga[axis][distance - 1].
+template <int R>
+__device__ __noinline__ double2 heat_fp64_pair(const double *__restrict__ p, int64_t py, int64_t pz, const double *w) {
+    double x[10];  // cells -4 .. 5
+#pragma unroll
+    for (int k = 0; k < 5; ++k) {
+        if (2 * k + 1 < 4 - R || 2 * k > 5 + R) continue;
+        const double2 t = *reinterpret_cast<const double2 *>(p - 4 + 2 * k);
+        x[2 * k] = t.x;
+        x[2 * k + 1] = t.y;
+    }
+    double2 n[2][R][2];  // [y, z][distance - 1][+, -]
+#pragma unroll
+    for (int a = 1; a <= R; ++a) {
+        n[0][a - 1][0] = *reinterpret_cast<const double2 *>(p + a * py);
+        n[0][a - 1][1] = *reinterpret_cast<const double2 *>(p - a * py);
+        n[1][a - 1][0] = *reinterpret_cast<const double2 *>(p + a * pz);
+        n[1][a - 1][1] = *reinterpret_cast<const double2 *>(p - a * pz);
+    }
+    double acc[2] = {w[0] * x[4], w[0] * x[5]};
+#pragma unroll
+    for (int a = 1; a <= R; ++a) {
+#pragma unroll
+        for (int u = 0; u < 2; ++u) acc[u] = fma(w[a], x[4 + u + a] + x[4 + u - a], acc[u]);
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+            const double2 hi = n[e][a - 1][0], lo = n[e][a - 1][1];
+            acc[0] = fma(w[(e + 1) * R + a], hi.x + lo.x, acc[0]);
+            acc[1] = fma(w[(e + 1) * R + a], hi.y + lo.y, acc[1]);
+        }
+    }
+    return make_double2(acc[0], acc[1]);
+}
+
 // Whether two biased values' high words are below the threshold t in magnitude.
 __device__ __forceinline__ bool fx_below(u32 a, u32 b, u32 t) {
     const u32 lo = FX_BIAS_HI - t;
@@ -87,6 +134,7 @@ __device__ __forceinline__ bool fx_below(u32 a, u32 b, u32 t) {
 template <int R, bool ISO, bool SAME, int TXP, typename Z>
 __device__ __forceinline__ int fx_pair(const u64 *cp, const Z &z, int dc, int sc, const FxCoef<R, ISO> &c,
                                        const double2 f, double (&res)[2]) {
+    constexpr int LOW = R == 1 ? 54 : R == 2 ? 53 : 52;  // |sum| below 2^LOW: small
     const FxWeights<FxCoef<R, ISO>::N> &w = c.w;
     // the thresholds at the centre plane's scale
     auto at_plane = [&](u32 t) { return SAME ? t : (u32)min((u64)t << min(dc, 28), (u64)FX_BIAS_HI); };
@@ -106,6 +154,9 @@ __device__ __forceinline__ int fx_pair(const u64 *cp, const Z &z, int dc, int sc
         small[u] = fx_below((u32)(X[4 + u] >> 32), (u32)(X[4 + u] >> 32), tc) &&
                    fx_below((u32)(X[3 + u] >> 32), (u32)(X[5 + u] >> 32), tx);
     // the in-plane pairs of every distance, moved to the common scale together
+#pragma unroll
+    for (int u = 0; u < 2; ++u)
+        small[u] = small[u] && fx_below((u32)(z(1, u) >> 32), (u32)(z(-1, u) >> 32), c.small_a[ISO ? 0 : 2]);
     u64 sxy[2][R], sy[2][R];
 #pragma unroll
     for (int a = 1; a <= R; ++a) {
@@ -157,7 +208,7 @@ __device__ __forceinline__ int fx_pair(const u64 *cp, const Z &z, int dc, int sc
         const long long v = acc[u].result(w.corr);
         const double sum = fx_big(v) ? fx_to_double(v, sc + w.ew) : fx_small_to_double(v, sc + w.ew);
         res[u] = fma(c.g0, u ? f.y : f.x, sum);
-        if (small[u] && (u64)(v + (1ll << 54)) < (2ull << 54)) left |= 1 << u;
+        if (small[u] && (u64)(v + (1ll << LOW)) < (2ull << LOW)) left |= 1 << u;
     }
     return left;
 }
@@ -174,7 +225,11 @@ heat_fx_kernel(const __grid_constant__ CUtensorMap map, const double *__restrict
     u64 *ring = reinterpret_cast<u64 *>(smem_raw + ((128u - (smem_addr(smem_raw) & 127u)) & 127u));
     __shared__ __align__(8) uint64_t full[NSLOT];
     __shared__ int scale[NSLOT];     // exponent code of each slot's plane
-    __shared__ int4 window[2];       // of an output plane, by parity: {scale, planes differ, centre's shift}
+    __shared__ int low[NSLOT];       // how many threads of the last warp hold values far below it
+    // of an output plane, by parity: {scale (or FP64, all outputs), planes differ, centre's shift}
+    constexpr int FP64 = 4096;
+    __shared__ int4 window[2];
+    __shared__ double weights[1 + 3 * R];
     __shared__ u32 list[Cfg::LIST];
     __shared__ u32 listed;
     const int tid = threadIdx.x, lane = tid & 31, wy = tid >> 5;
@@ -193,6 +248,7 @@ heat_fx_kernel(const __grid_constant__ CUtensorMap map, const double *__restrict
         mbar_fence_init();
         listed = 0;
     }
+    if (tid < 1 + 3 * R) weights[tid] = tid == 0 ? c.g0 : c.ga[(tid - 1) / R][(tid - 1) % R];
     __syncthreads();
     pdl_launch_dependents();
     pdl_wait();
@@ -228,6 +284,7 @@ heat_fx_kernel(const __grid_constant__ CUtensorMap map, const double *__restrict
     }
     bool ok = true;
     double2 raw[KP];  // this thread's share of the plane loaded last
+    u32 raw_hm = 0u;  // its largest high word
     auto load = [&](int j) {
         const int s = j & (NSLOT - 1);
         ok = ok && mbar_wait_bounded(&full[s], ((unsigned)j / NSLOT) & 1u);
@@ -247,6 +304,7 @@ heat_fx_kernel(const __grid_constant__ CUtensorMap map, const double *__restrict
             }
             hm = max(hm, max((u32)__double2hiint(raw[k].x) & 0x7fffffffu, (u32)__double2hiint(raw[k].y) & 0x7fffffffu));
         }
+        raw_hm = hm;
         hm = __reduce_max_sync(0xffffffffu, hm);
         int code = (int)(hm >> 20);
         if (hm == 0u) {  // only zeros and the smallest denormals: tell them apart
@@ -316,33 +374,28 @@ heat_fx_kernel(const __grid_constant__ CUtensorMap map, const double *__restrict
 
     const bool plain = nv == 2 && (mlo | mhi) == 0;  // both cells, no x image
     const int own = (wy + R) * TXP + Cfg::HX + 2 * lane;
+    const bool early = (wy >> 2) & 1;  // computes before it converts
+    // the listed outputs, by all threads
+    auto work_off = [&]() {
+        for (u32 i = tid; i < min(listed, (u32)Cfg::LIST); i += NT) {
+            const int cx = x0 + (int)(list[i] & 63u), cy = y0 + (int)((list[i] >> 6) & 15u), cz = zc0 + (int)(list[i] >> 10);
+            store_with_images(out, g, R, images != 0, cx, cy, cz, heat_fp64_cell<R, ISO>(in, g, c, cx, cy, cz));
+        }
+    };
     load(0);
     bool bad = __syncthreads_or(!ok);
     for (int t = 0; !bad && t <= nplanes; ++t) {
         const int m = t - 1 - 2 * R;  // outputs of plane zc0 + m, from planes m .. t - 1
         double2 centre = make_double2(0.0, 0.0);  // exact, for the use below
         if (m >= 0 && nv != 0) centre = *reinterpret_cast<const double2 *>(in + (optr - out));
-        // the plane's scale is complete since the barrier; its slot is read from the next one on
-        if (t < nplanes) {
-            convert(t);
-            if (tid == NT - 1 && t >= 2 * R) {  // the window of the next interval's outputs: planes t - 2R .. t
-                int top = 0, low = 4096;
-                for (int k = t - 2 * R; k <= t; ++k) {
-                    const int e = scale[k & (NSLOT - 1)];
-                    top = max(top, e);
-                    low = min(low, e);
-                }
-                window[t & 1] = make_int4(top, low < top, top - scale[(t - R) & (NSLOT - 1)], 0);
-            }
-            if (t + 1 < nplanes) load(t + 1);
-        }
-        if (m >= 0 && nv != 0) {
+        auto compute = [&]() {
+            if (m < 0 || nv == 0) return;
             const int4 win = window[(t - 1) & 1];
             const int sc = win.x, dc = win.z, z = zc0 + m;
             const u64 *cp = ring + ((m + R) & (NSLOT - 1)) * Cfg::SLOT + own;
             double res[2];
             int left = 0;  // outputs left to FP64
-            if (sc >= FX_SMIN && sc <= FX_EMAX) {
+            if (sc != 0 && sc != FP64) {
                 u64 Q[2 * R + 1][2];  // the z column at scale sc (its centre is read with the row)
 #pragma unroll
                 for (int k = 0; k <= 2 * R; ++k) {
@@ -365,19 +418,28 @@ heat_fx_kernel(const __grid_constant__ CUtensorMap map, const double *__restrict
                     }
                     left = fx_pair<R, ISO, false, TXP>(cp, column, dc, sc, c, centre, res);
                 }
-            } else {  // zeros only, or infinities, NaN, or near the ends of the exponent range
+            } else if (sc == 0) {
                 res[0] = res[1] = 0.0;
-                left = sc == 0 ? 0 : 3;
+            } else {
+                const double2 v = heat_fp64_pair<R>(in + (optr - out), pitch_y, pitch_z, weights);
+                res[0] = v.x;
+                res[1] = v.y;
             }
             left &= (1 << nv) - 1;
             if (left) {
+                bool over = false;
 #pragma unroll
                 for (int u = 0; u < 2; ++u)
                     if (left & (1 << u)) {
                         const u32 at = atomicAdd(&listed, 1u);
                         if (at < (u32)Cfg::LIST) list[at] = (u32)(2 * lane + u) | (u32)wy << 6 | (u32)m << 10;
-                        else res[u] = heat_fp64_cell<R, ISO>(in, g, c, x + u, y, z);
+                        else over = true;
                     }
+                if (over) {
+                    const double2 v = heat_fp64_pair<R>(in + (optr - out), pitch_y, pitch_z, weights);
+                    if (left & 1) res[0] = v.x;
+                    if (left & 2) res[1] = v.y;
+                }
             }
             const int zs = images ? (z < R ? nz : (z >= nz - R ? -nz : 0)) : 0;
             if (plain) *reinterpret_cast<double2 *>(optr) = make_double2(res[0], res[1]);
@@ -389,8 +451,42 @@ heat_fx_kernel(const __grid_constant__ CUtensorMap map, const double *__restrict
                 if (ys && zs) put(optr + dy + dz, res);
             }
             optr += pitch_z;
+        };
+        if (early) compute();
+        // the plane's scale is complete since the barrier; its slot is read from the next one on
+        if (t < nplanes) {
+            convert(t);
+            if (wy == Cfg::BY - 1) {
+                const u32 far = __ballot_sync(0xffffffffu, keep != 0u && (int)(raw_hm >> 20) + 8 < scale[t & (NSLOT - 1)]);
+                if (lane == 31) {
+                    low[t & (NSLOT - 1)] = __popc(far);
+                    if (t >= 2 * R) {  // the window of the next interval's outputs: planes t - 2R .. t
+                        int top = 0, least = 4096;
+                        for (int k = t - 2 * R; k <= t; ++k) {
+                            const int e = scale[k & (NSLOT - 1)];
+                            top = max(top, e);
+                            least = min(least, e);
+                        }
+                        const int centre = (t - R) & (NSLOT - 1);
+                        const bool fp64 = top != 0 && (low[centre] > 16 || top < FX_SMIN || top > FX_EMAX);
+                        window[t & 1] = make_int4(fp64 ? FP64 : top, least < top, top - scale[centre], 0);
+                    }
+                }
+            }
+            if (t + 1 < nplanes) load(t + 1);
         }
+        if (!early) compute();
         bad = __syncthreads_or(!ok);
+        if (t % 4 == 3 && !bad) {
+            const bool full = listed > (u32)Cfg::LIST_HIGH;
+            __syncthreads();  // no thread lists again before all have looked
+            if (full) {
+                work_off();
+                __syncthreads();
+                if (tid == 0) listed = 0;
+                __syncthreads();
+            }
+        }
         if (!bad && tid == 0 && issued < nplanes && issued <= m + NSLOT) {  // planes up to m are retired
             fence_proxy_async();  // the block's generic writes to a slot before its next TMA load
             for (; issued < nplanes && issued <= m + NSLOT; ++issued) {
@@ -408,12 +504,7 @@ heat_fx_kernel(const __grid_constant__ CUtensorMap map, const double *__restrict
         }
         return;
     }
-    __syncthreads();  // the listed cells' first stores and the list itself
-    const u32 n = min(listed, (u32)Cfg::LIST);
-    for (u32 i = tid; i < n; i += NT) {
-        const int cx = x0 + (int)(list[i] & 63u), cy = y0 + (int)((list[i] >> 6) & 15u), cz = zc0 + (int)(list[i] >> 10);
-        store_with_images(out, g, R, images != 0, cx, cy, cz, heat_fp64_cell<R, ISO>(in, g, c, cx, cy, cz));
-    }
+    work_off();  // the loop ended with a barrier
 }
 
 template <int R, bool ISO>
@@ -457,14 +548,12 @@ cudaError_t dispatch(int variant, const CUtensorMap *map, const double *in, doub
     c.g0 = dc.g0;
     for (int a = 0; a < 3; ++a)
         for (int b = 0; b < R; ++b) c.ga[a][b] = dc.ga[a][b];
-    // A centre is small when its term is below 2^-6 of 2^ew S, a neighbour below 2^-7 of it (the first
-    // weight of equal axes is between 0.43 and 1 times 2^ew) and below 2^-6 of the scale.
-    auto threshold = [&](double weight, double share) {
-        const double t = FX_FLAG_HI * (share * std::ldexp(1.0, c.w.ew) / weight);
-        return t < FX_BIAS_HI ? (u32)t + 1 : FX_BIAS_HI;  // weight 0: every value is small
+    auto threshold = [&](double weight) {  // of a value whose term is below 2^-6, -7, -8 of 2^ew S
+        const double t = (FX_FLAG_HI >> std::min(R - 1, 2)) * std::ldexp(1.0, c.w.ew) / weight;
+        return t < FX_BIAS_HI ? std::max((u32)t + 1, 4u) : FX_BIAS_HI;  // weight 0: every value is small
     };
-    c.small_c = std::max(threshold(dc.g0, 1.0), 4u);
-    for (int a = 0; a < 2; ++a) c.small_a[a] = std::max(threshold(dc.ga[a][0], 0.5), FX_FLAG_HI);
+    c.small_c = threshold(dc.g0);
+    for (int a = 0; a < 3; ++a) c.small_a[a] = threshold(dc.ga[a][0]);
     if (variant < 0 || variant >= 4) return cudaErrorInvalidValue;
     return run<R, ISO>(map, in, out, g, c, images, err, s, FX_REREAD[variant], zmode);
 }

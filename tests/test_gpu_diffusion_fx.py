@@ -121,6 +121,28 @@ def test_launch_shapes_agree_bit_for_bit(cuda_lib, shape):
         assert np.array_equal(_step(p, f, v)[0], first), v
 
 
+# fields whose rows are evaluated in FP64 as a whole, or list up to 16 outputs each, thousands per
+# block of threads (the columns of small values), in every launch shape
+@pytest.mark.parametrize("r", [1, 3, 4])
+@pytest.mark.parametrize("kind", ["columns", "spot"])
+def test_localised_fields(cuda_lib, r, kind):
+    shape, h = (33, 200, 500), (0.5, 0.5, 0.5)
+    z, y, x = np.meshgrid(*[np.arange(n) for n in shape], indexing="ij")
+    rng = np.random.default_rng(4)
+    f = (np.where((x // 8 + y // 8) % 2, 1e-12, 1.0) * rng.uniform(0.5, 1.0, shape) if kind == "columns" else
+         np.exp(-((x - 250.3) ** 2 + (y - 99.5) ** 2 + (z - 15.7) ** 2) / 288.0))
+    p = _plan(shape, r, h)
+    ref, mag = _reference(f, r, h)
+    first = None
+    for v in range(p.variant()[1]):
+        got, whole = _step(p, f, v)
+        if first is None:
+            first = whole
+            bound = (1 + 6 * r + 2) * 2.0 ** -53 * mag + 2.0 ** -1074
+            assert float(np.max(np.abs(got - ref) / bound)) <= 1.0
+        assert np.array_equal(whole, first), v
+
+
 def test_weights_of_a_backward_step_run_on_the_fp64_pipe(cuda_lib):
     shape, r, h = (12, 18, 40), 3, (0.5, 0.5, 0.5)  # dt < 0: the signs the fixed-point kernel has not compiled in
     p = _plan(shape, r, h, dt=-0.01)
