@@ -3,7 +3,7 @@
 // Of the 600 FP64 instructions per cell and substep of the kernel in mhd.cu, which kept the FP64
 // pipe 80 % busy, 470 are the 57 linear differences of gamma = A B (Eq. 8).  Here they are sums of
 // products on the integer pipe (fixed.cuh); the right-hand side of Eqs. A1-A4, the closure and
-// the RK update stay in FP64, on the exact cell values.  One RK3 step of 256^3: 60.8 -> 33.7 ms.
+// the RK update stay in FP64, on the exact cell values.  One RK3 step of 256^3: 60.8 -> 33.4 ms.
 //
 //   * z-streaming as in mhd.cu: 16 x 8 cells per CTA, planes of all 8 fields in a ring of 8 slots.
 //     An arriving plane is converted in place to biased 60-bit integers, one binary scale per plane
@@ -14,7 +14,7 @@
 //     160^3, one substep: one thread per cell 5.1 ms, two groups 3.75, four groups 3.1 (128 registers
 //     a thread).  Bound by the latency of dependent instructions at 4 warps per scheduler (issue 34 %,
 //     FP64 pipe 43 %): the ring leaves no shared memory for a second CTA.
-//   * One body of code for all fields: unrolled it is 320 KB, and the step took 24 ms.
+//   * One body of code for all fields: unrolled it is 320 KB, and a substep took 24 ms.
 //   * A cell uses, per field, the largest scale of the 7 planes of its window.  Where those
 //     differ (11 % of the windows), values are shifted as they are read, a branch that is uniform per
 //     block and field.  The scales depend on the planes' tiles alone, so results do not depend on
@@ -24,9 +24,17 @@
 //     large values lose nothing to FP64.  Error of the right-hand side against extended precision:
 //     0.03 to 0.95 times that of the FP64 kernel (rms; waves, noise, small waves on large means,
 //     components far below their companions).
-//   * Cells where a field is small against its scale (below 2^-6, fixed.cuh says why; 0.1 % of a
-//     256^3 state of waves), or that meet infinities or NaN, are listed and evaluated by FP64
-//     from global memory at the end of the CTA, as mhd.cu does.
+//   * A field is small at a cell where it and its six neighbours are below 2^-6 of the scale
+//     (fixed.cuh says why), and where the scale is out of range, as with infinities and NaN.  A warp
+//     with more than 4 such cells of a field takes that field's derivatives in FP64 from global
+//     memory, in the operations of mhd.cu; fewer cells are listed unless the gradient shows terms of at
+//     least 2^-6 of the scale, and evaluated in FP64 throughout at the end of the CTA.
+//   * Accuracy by field, not by axis: next to larger neighbours on one axis, the difference of values
+//     far below the scale along another is exact to 2^-60 of the scale only, where FP64 keeps its digits.
+//   * One RK3 step in ms, the FP64 pipe's kernel and this one: 256^3 waves 60.8 and 33.4, a vortex of 24
+//     cells in 256^3 60.8 and 52.4.  128^3, which fills 128 tiles in 2 chunks each unevenly: waves 7.9 and
+//     5.2, a vortex of 6, 10, 16 cells 7.9 and 10.2, 10.3, 10.2, a shear layer 7.9 and 9.6 (before fields
+//     were taken in FP64 by warps 13.7, 16.9, 14.9, 17.1).
 #include <algorithm>
 
 #include "fixed.cuh"
@@ -35,7 +43,9 @@
 namespace stn {
 namespace {
 
-constexpr int TX = 16, TY = 8, GROUP = TX * TY, NGROUPS = 4, NT = NGROUPS * GROUP, NSLOT = 8, LIST = 1024;
+constexpr int TX = 16, TY = 8, GROUP = TX * TY, NGROUPS = 4, NT = NGROUPS * GROUP, NSLOT = 8;
+constexpr int LIST = 1024;
+constexpr int FP64_CELLS = 4;  // more small cells of a warp than this: the field's derivatives in FP64
 // What the groups of derivatives hand to the group of the right-hand side, per cell: u (Laplacian,
 // h, gradient) 3 x 7, A (Laplacian, h, two of the gradient) 3 x 6, lnrho and s (gradient, Laplacian) 2 x 4.
 constexpr int EX_A = 21, EX_LNRHO = 39, EX_SS = 43, NEX = 47;
@@ -99,20 +109,24 @@ template <bool MIXED> struct FxWin {
         }
         return acc.wide(w.km[pair], sc + w.em);
     }
-    // whether the field is below 2^-6 of the scale at the cell and its x and y neighbours
-    __device__ __forceinline__ bool small() const {
-        const u64 *c = p[3];
-        const u32 h[5] = {(u32)(c[0] >> 32), (u32)(c[1] >> 32), (u32)(c[-1] >> 32), (u32)(c[RS] >> 32), (u32)(c[-RS] >> 32)};
-        u32 top = 0u, low = ~0u;
-#pragma unroll
-        for (int i = 0; i < 5; ++i) {
-            top = max(top, h[i]);
-            low = min(low, h[i]);
-        }
-        const u32 flag = !MIXED ? FX_FLAG_HI : d[3] < 6 ? FX_FLAG_HI << d[3] : FX_BIAS_HI;
-        return top < FX_BIAS_HI + flag && low >= FX_BIAS_HI - flag;
-    }
 };
+
+// Whether a field is below 2^-6 of the scale at a cell and its six neighbours; p: the cell in planes
+// -1, 0, 1, whose scales lie d below it.
+__device__ __forceinline__ bool field_small(const u64 *const (&p)[3], const int (&d)[3]) {
+    bool small = true;
+#pragma unroll
+    for (int k = 0; k < 3; ++k) {
+        const u32 flag = d[k] < 6 ? FX_FLAG_HI << d[k] : FX_BIAS_HI, lo = FX_BIAS_HI - flag;
+        u32 h = (u32)(p[k][0] >> 32) - lo;
+        if (k == 1) {
+            h = max(h, max((u32)(p[k][1] >> 32) - lo, (u32)(p[k][-1] >> 32) - lo));
+            h = max(h, max((u32)(p[k][RS] >> 32) - lo, (u32)(p[k][-RS] >> 32) - lo));
+        }
+        small = small && h < 2 * flag;
+    }
+    return small;
+}
 
 // The derivatives some term uses of component c of a vector (c < 3; its own gradient component
 // only where `own`), or of lnrho and s (c = 3): gradient, Laplacian, and h[a] = d_a d_c.
@@ -144,6 +158,64 @@ __device__ __forceinline__ void field_derivs(const FxWin<MIXED> &w, const FxMhd 
             }
         }
     }
+}
+
+// Where the derivatives of field q (component c, or 3) go: Laplacian, h, gradient.
+__device__ __forceinline__ int ex_of(int q, int c) { return c == 3 ? (q == F_SS ? EX_SS : EX_LNRHO) : q < F_AX ? 7 * c : EX_A + 6 * c; }
+__device__ __forceinline__ void put_derivs(double *e, int c, bool own, bool laplacian, const double (&g)[3], double lap,
+                                           const double (&h)[3]) {
+    if (c == 3) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) e[a * GROUP] = g[a];
+        if (laplacian) e[3 * GROUP] = lap;
+        return;
+    }
+    e[0] = lap;
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+        e[(1 + a) * GROUP] = h[a];
+        if (own) e[(4 + a) * GROUP] = g[a];
+        else if (a != c) e[(a == (c + 1) % 3 ? 4 : 5) * GROUP] = g[a];
+    }
+}
+
+// The same derivatives of one field at one cell (f) by FP64 from global memory, in the operations
+// of mhd.cu, stored at e.
+struct FieldWin : WinOps<double, FieldWin> {
+    const double *f;
+    int64_t sy, sz;
+    __device__ __forceinline__ double at(int, int k, int dx, int dy) const { return f[(k - 3) * sz + dy * sy + dx]; }
+};
+template <bool CONDUCT>
+__device__ __noinline__ void field_fp64(const double *f, int64_t sy, int64_t sz, const MK<double> *k, int c, bool own, double *e) {
+    FieldWin w;
+    w.f = f;
+    w.sy = sy;
+    w.sz = sz;
+    double g[3], h[3] = {}, lap = 0.0;
+#pragma unroll
+    for (int a = 0; a < 3; ++a)
+        if (own || a != c) g[a] = w.d1(0, a, k->d1[a]);
+    if (CONDUCT || c < 3) {
+#pragma unroll
+        for (int a = 0; a < 3; ++a) {
+            const double one = w.d2(0, a, k->d2c[a], k->d2[a]);
+            if (a == c) h[a] = one;
+            lap = a == 0 ? one : add(lap, one);
+        }
+    }
+    if (c < 3) {
+#pragma unroll
+        for (int pair = 0; pair < 3; ++pair) {  // (0,1), (0,2), (1,2)
+            const int a = pair == 2 ? 1 : 0, b = pair == 0 ? 1 : 2;
+            if (c == a || c == b) {
+                const double m = w.dmix(0, pair, k->dm[pair]);
+                if (c == a) h[b] = m;
+                else h[a] = m;
+            }
+        }
+    }
+    put_derivs(e, c, own, CONDUCT, g, lap, h);
 }
 
 // What follows the right-hand side of one cell: the RK update and its stores, or the dense result.
@@ -383,18 +455,26 @@ mhd_fx_kernel(const __grid_constant__ MhdMaps maps, const __grid_constant__ FxIn
             for (int i = 0; i < n; ++i) {
                 const int q = (int)(todo >> 4 * i & 15u);
                 const int c = q == F_LNRHO || q == F_SS ? 3 : q < F_AX ? q - F_UX : q - F_AX;
+                const bool own_grad = q < F_AX;
                 double g3[3], lap, h3[3];
                 const bool some = active && m < count;
+                int sc = top[m & 1][q];
+                const bool in_range = sc >= FX_SMIN && sc <= FX_EMAX;  // all zeros count as in range
+                bool small = false;
                 if (some) {
-                    int sc = top[m & 1][q];
-                    const bool in_range = sc >= FX_SMIN && sc <= FX_EMAX;
-                    if (low[m & 1][q] == sc || !in_range) {  // all zeros count as in range
+                    const u64 *const c3[3] = {plane[2] + q * FE, plane[3] + q * FE, plane[4] + q * FE};
+                    const int d3[3] = {sc - scale[(m + 2) & (NSLOT - 1)][q], sc - scale[(m + 3) & (NSLOT - 1)][q],
+                                       sc - scale[(m + 4) & (NSLOT - 1)][q]};
+                    small = in_range ? field_small(c3, d3) : sc != 0;
+                }
+                // where many cells of a warp are small, its cells' derivatives are taken in FP64
+                const bool fp64 = __popc(__ballot_sync(0xffffffffu, small)) > FP64_CELLS;
+                if (some && !fp64) {
+                    if (low[m & 1][q] == sc || !in_range) {
                         FxWin<false> w;
 #pragma unroll
                         for (int k = 0; k < 7; ++k) w.p[k] = plane[k] + q * FE;
-                        left = left || (in_range ? w.small() : sc != 0);
-                        if (!in_range) sc = 1023;
-                        field_derivs<false, CONDUCT>(w, fw, sc, c, q < F_AX, g3, lap, h3);
+                        field_derivs<false, CONDUCT>(w, fw, in_range ? sc : 1023, c, own_grad, g3, lap, h3);
                     } else {
                         FxWin<true> w;
 #pragma unroll
@@ -402,27 +482,21 @@ mhd_fx_kernel(const __grid_constant__ MhdMaps maps, const __grid_constant__ FxIn
                             w.p[k] = plane[k] + q * FE;
                             w.d[k] = sc - scale[(m + k) & (NSLOT - 1)][q];
                         }
-                        left = left || w.small();
-                        field_derivs<true, CONDUCT>(w, fw, sc, c, q < F_AX, g3, lap, h3);
+                        field_derivs<true, CONDUCT>(w, fw, sc, c, own_grad, g3, lap, h3);
+                    }
+                    if (small) {  // and its gradient too: the cell goes to FP64
+                        int top_g = 0;
+#pragma unroll
+                        for (int a = 0; a < 3; ++a)
+                            if (own_grad || a != c) top_g = max(top_g, __double2hiint(g3[a]) & 0x7fffffff);
+                        left = left || !in_range || (top_g >> 20) < sc + fw.e1 - 5;
                     }
                 }
                 if (i == 0) asm volatile("bar.sync 2, %0;" ::"n"(NT) : "memory");
                 if (some) {
-                    if (c == 3) {
-                        double *e = ex + (q == F_SS ? EX_SS : EX_LNRHO) * GROUP + gt;
-#pragma unroll
-                        for (int a = 0; a < 3; ++a) e[a * GROUP] = g3[a];
-                        if (CONDUCT) e[3 * GROUP] = lap;
-                    } else {
-                        double *e = ex + (q < F_AX ? 7 * c : EX_A + 6 * c) * GROUP + gt;
-                        e[0] = lap;
-#pragma unroll
-                        for (int a = 0; a < 3; ++a) {
-                            e[(1 + a) * GROUP] = h3[a];
-                            if (q < F_AX) e[(4 + a) * GROUP] = g3[a];
-                            else if (a != c) e[(a == (c + 1) % 3 ? 4 : 5) * GROUP] = g3[a];
-                        }
-                    }
+                    double *e = ex + ex_of(q, c) * GROUP + gt;
+                    if (fp64) field_fp64<CONDUCT>(in.f[q] + oidx + m * pitch_z, g.pad[0], pitch_z, &ks, c, own_grad, e);
+                    else put_derivs(e, c, own_grad, CONDUCT, g3, lap, h3);
                 }
             }
             exleft[group][gt] = left;
@@ -444,8 +518,7 @@ mhd_fx_kernel(const __grid_constant__ MhdMaps maps, const __grid_constant__ FxIn
         }
         return;
     }
-    __syncthreads();
-    const u32 n = min(listed, (u32)LIST);
+    const u32 n = min(listed, (u32)LIST);  // the loop ended with a barrier
     for (u32 i = tid; i < n; i += NT) {
         const int t = (int)(list[i] & (GROUP - 1u)), z = zc0 + (int)(list[i] >> 7);
         fp64_cell<MODE, CONDUCT>(in, fout, wbuf, rbuf, g, ks, first, last, images, x0 + t % TX, y0 + t / TX, z);
@@ -501,8 +574,9 @@ bool fx_mhd_weights(const MhdConst &c, FxMhd &o) {
 }
 
 // Planes per z-chunk: the fewest periods over the waves of CTAs (one per SM), when a chunk's start costs
-// `start` of them.  At most 64, so that the list holds an eighth of a chunk's cells: where it
-// overflowed, 128^3 in chunks of 128 planes took 7590 us a step, of 64 5175.
+// `start` of them.  At most 64: localised fields make some CTAs cost twice what others do, and longer
+// chunks leave the SMs unevenly loaded (128^3 with a vortex of 16 cells 14.8 ms a step in chunks of 128
+// planes, 10.2 in chunks of 64; waves 5.05 and 5.2).
 int chunk_planes(int tiles, int nz, int start) {
     const int sms = device_sms();
     int best = 1;

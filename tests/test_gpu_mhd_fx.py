@@ -98,6 +98,15 @@ def _fields(kind, shape):
         return f
     if kind == "specks":  # cells far below the scale of their plane
         return f * np.exp2(-rng.integers(0, 60, (8,) + shape))
+    if kind == "vortex":  # localised: most cells lie far below the scale of their tile
+        d = [np.arange(n) - c for n, c in zip(shape, (3.2, 30.7, 60.4))]
+        e = np.exp(-(d[0][:, None, None] ** 2 + d[1][:, None] ** 2 + d[2] ** 2) / 50.0)
+        return np.stack([(1.0 - 0.2 * q + 0.05 * d[1][:, None] - 0.03 * q * d[2]) * e for q in range(8)])
+    if kind == "shear":  # a perturbation of a layer in y, on a flow that changes sign there
+        dy = (np.arange(shape[1]) - 29.5)[:, None]
+        f = f * np.exp(-dy ** 2 / 32.0)
+        f[1] = 0.3 * np.tanh(dy / 4.0) * np.ones(shape)
+        return f
     raise ValueError(kind)
 
 
@@ -106,7 +115,7 @@ def _fields(kind, shape):
 # differs (the kernel that works in FP64 throughout reaches 1.03 of it on these fields, 1.28 where
 # cells go to FP64), plus one rounding of the result.
 @pytest.mark.parametrize("kind,K", [("waves", 0.0), ("random", 0.0), ("means", 0.0), ("tiny", 0.0), ("planes", 0.0),
-                                    ("specks", 0.0), ("waves", 0.7)])
+                                    ("specks", 0.0), ("waves", 0.7), ("vortex", 0.0), ("vortex", 0.7), ("shear", 0.0)])
 def test_rhs_as_accurate_as_fp64(cuda_lib, kind, K):
     shape = (7, 59, 115)
     f8 = _fields(kind, shape)
@@ -122,7 +131,7 @@ def test_rhs_as_accurate_as_fp64(cuda_lib, kind, K):
         rms = lambda v: float(np.sqrt(np.mean(np.square(v))))
         err, ref = rms(got - exact[q]), rms(plain[q] - exact[q])
         print(kind, q, err, ref)
-        assert err <= (1.3 if kind in ("planes", "specks") else 1.05) * ref + 2.0 ** -53 * rms(exact[q]), (kind, q)
+        assert err <= (1.3 if kind in ("planes", "specks", "vortex", "shear") else 1.05) * ref + 2.0 ** -53 * rms(exact[q]), (kind, q)
 
 
 def _step(p, f8, steps):
@@ -133,7 +142,7 @@ def _step(p, f8, steps):
     return np.stack([np.asarray(v) for v in p.download(b)])
 
 
-@pytest.mark.parametrize("kind", ("waves", "planes", "specks"))
+@pytest.mark.parametrize("kind", ("waves", "planes", "specks", "vortex"))
 def test_slabs_of_z_are_bit_identical(cuda_lib, kind):
     # the same planes in a deeper periodic field start other z-chunks
     shape = (24, 50, 130)
@@ -156,6 +165,19 @@ def test_variants_and_chunk_lengths_are_bit_identical(cuda_lib, K):
             p.set_variant(v)
             p.set_zmode(zmode)
             assert np.array_equal(_step(p, f8, 2), ref), (v, zmode)
+
+
+def test_more_listed_cells_than_the_list_holds(cuda_lib):
+    # s at the end of the exponent range: the two columns of the last tiles list every cell, 16 per
+    # plane, in chunks of up to 128 planes; elsewhere whole warps take the field in FP64
+    shape = (140, 50, 130)
+    f8 = 1e-3 * _fields("waves", shape)
+    f8[7] *= 1e-305
+    p, _ = _plan(shape)
+    ref = _step(p, f8, 1)
+    for zmode in (1, 2):
+        p.set_zmode(zmode)
+        assert np.array_equal(_step(p, f8, 1), ref), zmode
 
 
 @pytest.mark.parametrize("value", (np.inf, np.nan, 1e300, 1e-310))
