@@ -24,9 +24,15 @@
 //     be off, 2^-53 (2r+1) sum |w f|, wherever sum |w f| is at least 2^-7 of that result.  An output
 //     of that size itself shows it; the others are listed, their sum |w f| is accumulated from
 //     the high limbs until it passes the bound (a few terms for most), and what stays below is
-//     evaluated by FP64 multiply-adds in the order j = -r .. r.
+//     evaluated by FP64 multiply-adds in the order j = -r .. r, unless its window is all zeros.
 //   * A chunk with infinities, NaN or exponents near the ends of the range is swept in FP64, one
-//     sweep after the other, in shared memory.
+//     sweep after the other, in shared memory; so is one where 8 of 32 outputs spread over it would stay
+//     below the bound (pulses and spikes far above their surroundings).  That is looked at only where a
+//     quarter of the threads load mostly small cells.  A chunk of zeros stores zeros.
+//     3 M cells, r = 100, in us on the FP64 pipe, here, and with each output by itself: noise 1063, 242,
+//     246; pulses of 100 cells 1062, 1035, 1249; a spike every 997 cells 1062, 938, 1273; zeros 1062, 11,
+//     1057. 2^20 cells, 10 sweeps of r = 3: noise 127, 33.2, 33.3; pulses 127, 134, 152; spikes 127,
+//     119, 160. Noise over 60 binary orders at r = 1000 is the slowest, 3364, 4105, 4806.
 #include <algorithm>
 #include <vector>
 
@@ -37,6 +43,10 @@ namespace stn {
 namespace {
 
 constexpr int FT = 256;  // threads per CTA
+// Weights from which on it pays to look for chunks that FP64 evaluates sooner: 11 weights, 2^20 cells,
+// 13.1 us, with the look 14.9, and 31 to 33 at worst where the FP64 pipe takes 29.5.
+constexpr int FAR_WEIGHTS = 32;
+constexpr uint16_t EMPTY = 0x8000, DONE = 0xffff;  // marks of listed outputs
 
 template <int V_> struct FxWide {
     static constexpr int V = V_, CH = FT * V;
@@ -46,7 +56,7 @@ template <int V_> struct FxWide {
     static __host__ __device__ int cells(int r) { return CH + nwp(r) + V; }
     static __host__ __device__ size_t smem(int r) { return sizeof(int2) * (size_t)(cells(r) + nwp(r)) + sizeof(uint16_t) * CH; }
     static_assert(V % 2 == 1 && SPILL >= 1, "");
-    static_assert(CH <= 65536, "list entries are 16-bit");
+    static_assert(CH < 32768, "list entries are 16-bit, one of them a mark");
 };
 
 // v as balanced limbs at scale E: v = (2^30 qh + ql) 2^(E - 1081), |2^30 qh + ql| <= 2^59, nearest.
@@ -69,7 +79,7 @@ xcorr_wide_fx_kernel(const double *__restrict__ in, double *__restrict__ out, Ge
     constexpr int CH = B::CH;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ u32 red[FT / 32];
-    __shared__ u32 listed;
+    __shared__ u32 listed, far;
     const int tid = threadIdx.x, nw = 2 * r + 1, nwp = B::nwp(r), cells = B::cells(r), len = CH + 2 * r;
     int2 *s = reinterpret_cast<int2 *>(smem_raw);
     double *sd = reinterpret_cast<double *>(smem_raw);  // the results
@@ -87,7 +97,7 @@ xcorr_wide_fx_kernel(const double *__restrict__ in, double *__restrict__ out, Ge
         }
         return (gi >= -r && gi < n + r) ? inx[gi] : 0.0;
     };
-    if (tid == 0) listed = 0u;
+    if (tid == 0) listed = far = 0u;
     pdl_wait();
 
     // The cells and their largest exponent; those past the last output's window count as 0.  A
@@ -112,7 +122,13 @@ xcorr_wide_fx_kernel(const double *__restrict__ in, double *__restrict__ out, Ge
 #pragma unroll
     for (int w = 0; w < FT / 32; ++w) hm = max(hm, red[w]);
     const int E = (int)(hm >> 20);
-    const bool fixed = E >= FX_SMIN && E <= FX_EMAX;  // uniform per block
+    bool fixed = E >= FX_SMIN && E <= FX_EMAX;  // uniform per block
+    bool zeros = false;
+    if (hm == 0u) {  // zeros only, or the smallest denormals too
+        u32 any = 0u;
+        for (int e = tid; e < used; e += FT) any |= (u32)__double2loint(load(e));
+        zeros = !__syncthreads_or(any != 0u);
+    }
 
     // FP64 multiply-adds of output p from global memory
     auto by_fp64 = [&](int p) -> double {
@@ -121,6 +137,12 @@ xcorr_wide_fx_kernel(const double *__restrict__ in, double *__restrict__ out, Ge
         return acc;
     };
 
+    // whether any cell that is not 0 lies so far below the scale that its limbs are 0
+    auto faint_cells = [&]() {
+        bool any = false;
+        for (int e = tid; e < used; e += FT) any = any || ((s[e].x | s[e].y) == 0 && load(e) != 0.0);
+        return __syncthreads_or(any) != 0;
+    };
     const int base = tid * V;
     double res[V];
     if (fixed) {
@@ -128,7 +150,32 @@ xcorr_wide_fx_kernel(const double *__restrict__ in, double *__restrict__ out, Ge
         for (int k = 0; k < KR; ++k)
             if (tid + k * FT < cells) s[tid + k * FT] = fx_limbs(kept[k], E);
         for (int e = tid + KR * FT; e < cells; e += FT) s[e] = fx_limbs(load(e), E);
-        __syncthreads();
+        int small = 0;
+        if (nw >= FAR_WEIGHTS) {
+#pragma unroll
+            for (int k = 0; k < KR; ++k) small += (int)(((u32)__double2hiint(kept[k]) & 0x7fffffffu) >> 20) + 7 < E;
+        }
+        if (__syncthreads_count(2 * small > KR) > FT / 4) {
+            // 4 outputs per warp, spread over the chunk, whose sum |w f| is taken whole
+            int below = 0;
+            const bool faint = faint_cells();
+            for (int i = 0; i < 4; ++i) {
+                const int p = ((tid >> 5) * 4 + i) * (CH / 32);
+                u64 mag = 0;
+                int any = 0;
+                for (int j = tid & 31; j < nw; j += 32) {
+                    mag += (u64)(u32)abs(ws[j].y) * (u32)abs(s[p + j].y);
+                    any |= s[p + j].x | s[p + j].y;
+                }
+                for (int d = 16; d; d >>= 1) mag += __shfl_xor_sync(0xffffffffu, mag, d);
+                below += mag < (1ull << 53) && (faint || __any_sync(0xffffffffu, any)) && c0 + p < n;
+            }
+            if ((tid & 31) == 0 && below) atomicAdd(&far, (u32)below);
+            __syncthreads();
+            fixed = far < 8u;
+        }
+    }
+    if (fixed) {
         long long hh[V], m[V];
 #pragma unroll
         for (int v = 0; v < V; ++v) hh[v] = m[v] = 0;
@@ -166,18 +213,31 @@ xcorr_wide_fx_kernel(const double *__restrict__ in, double *__restrict__ out, Ge
         // the listed outputs: `res` of most stands; the rest is replaced below
         const u32 nl = listed;
         if (nl) {
+            bool empty = false;
             for (u32 i = tid; i < nl; i += FT) {
                 const int p = list[i];
                 u64 mag = 0;  // sum |w f| in units of 2^2 of the results' last place
-                for (int j = 0; j < nw && mag < (1ull << 53); ++j)
+                int any = 0;
+                for (int j = 0; j < nw && mag < (1ull << 53); ++j) {
                     mag += (u64)(u32)abs(ws[j].y) * (u32)abs(s[p + j].y);
-                if (mag >= (1ull << 53)) list[i] = 0xffffu;
+                    any |= s[p + j].x | s[p + j].y;
+                }
+                empty = empty || !any;
+                if (mag >= (1ull << 53)) list[i] = DONE;
+                else if (!any) list[i] = (uint16_t)(p | EMPTY);
             }
-            __syncthreads();
+            if (__syncthreads_or(empty) && !faint_cells()) {  // windows of zeros
+                for (u32 i = tid; i < nl; i += FT)
+                    if (list[i] & EMPTY) list[i] = DONE;
+                __syncthreads();
+            }
         }
         // results through shared memory, then coalesced stores
 #pragma unroll
         for (int v = 0; v < V; ++v) sd[base + v] = res[v];
+    } else if (zeros) {
+#pragma unroll
+        for (int v = 0; v < V; ++v) sd[base + v] = 0.0;
     } else {
         // every sweep leaves cell e of the sum at e: it reads e .. e + 2 r1, ascending in waves of FT
         for (int e = tid; e < cells; e += FT) sd[e] = load(e);
@@ -197,7 +257,7 @@ xcorr_wide_fx_kernel(const double *__restrict__ in, double *__restrict__ out, Ge
     __syncthreads();
     if (fixed && listed) {
         for (u32 i = tid; i < listed; i += FT)
-            if (list[i] != 0xffffu) sd[list[i]] = by_fp64(list[i]);
+            if (list[i] != DONE) sd[list[i] & (EMPTY - 1)] = by_fp64(list[i] & (EMPTY - 1));
         __syncthreads();
     }
     pdl_launch_dependents();  // not earlier: the next launch's CTAs would wait on the SMs

@@ -92,6 +92,34 @@ def test_caller_halo_and_special_values(cuda_lib):
         assert np.all(np.abs(got - ref)[fine] <= (2 * r + 1) * 2.0 ** -53 * mag[fine])
 
 
+def _pulses(n, r):
+    rng = np.random.default_rng(r)
+    i = np.arange(n)
+    yield "spikes on zeros", np.where(i % 997 == 5, 1.0 + rng.random(n), 0.0)
+    yield "a spike and zeros", np.where(i == n // 2, -3.0, 0.0)
+    yield "pulses", np.exp(-((i % 4096) - 2048.0) ** 2 / 2e4)
+    yield "many orders", rng.standard_normal(n) * 2.0 ** -rng.integers(0, 60, n)
+    yield "faint half", np.where((i // 300) % 2, 1.0, 1e-30) * rng.random(n)
+    yield "signed zeros", np.where(i % 2, 0.0, -0.0)
+
+
+# chunks of which most outputs lie far below the scale, windows and chunks of zeros; radii of each block size
+@pytest.mark.parametrize("r,n,sweeps", [(5, 9001, 1), (13, 5001, 1), (100, 30011, 1), (1000, 20001, 1), (1, 20011, 16),
+                                        (3, 20011, 10), (4, 7001, 3)])
+@pytest.mark.parametrize("kind", ["average", "gauss", "orders"])
+def test_pulses_and_zeros(cuda_lib, r, n, sweeps, kind):
+    g = _weights(r, kind)
+    for name, f in _pulses(n, r):
+        got, (lo, hi) = _run(f, g, sweeps=sweeps)
+        ref, mag = f.astype(np.longdouble), np.abs(f).astype(np.longdouble)
+        for _ in range(sweeps):
+            ref, mag = _reference(np.pad(ref, r, mode="wrap"), g)[0], _reference(np.pad(mag, r, mode="wrap"), np.abs(g))[0]
+        tiny = sweeps * (2 * r + 1) * max(1.0, float(np.abs(g).sum())) ** sweeps * 2.0 ** -1074
+        worst = float(np.max(np.abs(got - ref) / (sweeps * (2 * r + 1) * 2.0 ** -53 * mag + tiny)))
+        assert worst <= 1.0, (name, worst)
+        assert np.all(got[mag == 0] == 0) and np.array_equal(lo, got[-r:]) and np.array_equal(hi, got[:r]), name
+
+
 # one launch, one launch and a remainder, and radii that fill register blocks or not; n below the
 # composed halo wraps more than once
 @pytest.mark.parametrize("r,n,sweeps", [(1, 3, 1), (1, 2305, 16), (2, 5, 16), (2, 4000, 7), (3, 4099, 10), (3, 2304, 17),
