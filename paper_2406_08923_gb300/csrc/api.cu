@@ -982,15 +982,20 @@ static int num_variants(stencil_t p) {
 
 static const char *variant_name(stencil_t p, int v) {
     if (p->kind == STENCIL_MAXFILTER) return "doubling_chunk4096";
+    // one sweep per launch, register-blocked: xcorr_pair.cu, xcorr_fx.cu (V outputs per thread) or xcorr_wide.cu
     if (p->kind == STENCIL_XCORR && !xcorr_blocked(p)) return "wide_register_blocked";
-    // FP64 sweeps one output per thread over a runtime chunk length; the other types use
-    // 2184-cell chunks and 9-output register windows
-    const bool f64 = p->storage == STENCIL_F64;
+    // Several sweeps composed into one correlation (xcorr_fx.cu).  Where they are not, FP64 sweeps one
+    // output per thread over a runtime chunk length, the other types 2184-cell chunks with 9-output
+    // register windows.
+    const bool f64 = p->storage == STENCIL_F64, fixed = p->radius > 2 ? !p->fx.empty() : p->fx.size() > 1;
     if (p->kind == STENCIL_DIFFUSION && p->ndim == 1)
-        return f64 ? "xcorr_folded_runtime_chunk_scalar_temporal_blocking" : "xcorr_folded_chunk2184_v9_temporal_blocking";
+        return fixed ? "xcorr_folded_composed_fixed_point"
+               : f64 ? "xcorr_folded_runtime_chunk_scalar_temporal_blocking" : "xcorr_folded_chunk2184_v9_temporal_blocking";
+    if (p->kind == STENCIL_XCORR && fixed) return "composed_fixed_point";
+    if (p->kind == STENCIL_XCORR && p->i32.size() > 1) return "composed_v9";
     if (p->kind == STENCIL_DIFFUSION && p->ndim == 2)
         return v == 1 ? "stream2d_tb2" : v == 2 ? "stream2d_tb4" : "tile2d_32vx_by8_ry4";
-    if (p->kind == STENCIL_DIFFUSION) return diffusion_variant_name(storage_code(p->storage), p->radius, v);
+    if (p->kind == STENCIL_DIFFUSION) return diffusion_variant_name(storage_code(p->storage), p->radius, v, p->dcoef.fx);
     if (p->kind == STENCIL_MHD8) return mhd_variant_name(storage_code(p->storage), v, p->mconst.fx);
     return f64 ? "runtime_chunk_scalar_temporal_blocking" : "chunk2184_v9_temporal_blocking";
 }

@@ -453,6 +453,8 @@ static cudaError_t run(const CUtensorMap *map, void *out, const Geom &g, const D
 // shapes the variants of radius 3 name.
 #define DIFF_VARIANT_F64(X) X(1, 8, 1, 2, 8, false)
 static const char *F64_NAMES[] = {"fx64x16", "fx64x16_more_chunks", "fx64x16_fewer_chunks", "fx64x16_even_waves"};
+static const char *F64_PIPE_NAMES[] = {"?", "f64_r1_vx2_by8_ry1_zb2_s8", "f64_r2_vx2_by8_ry1_zb2_s8", "vx2_by8_ry1_zb2_s8",
+                                       "f64_r4_vx2_by8_ry1_zb2_s8"};
 static const char *F64_NAMES_OTHER[] = {"?", "f64_r1_fx64x16", "f64_r2_fx64x16", "?", "f64_r4_fx64x16"};
 
 int diffusion_num_variants(int dtype, int r) {
@@ -460,9 +462,10 @@ int diffusion_num_variants(int dtype, int r) {
     return r == 3 ? 4 : (r >= 1 && r <= 4 ? 1 : 0);
 }
 
-const char *diffusion_variant_name(int dtype, int r, int v) {
+const char *diffusion_variant_name(int dtype, int r, int v, bool fx) {
     if (dtype != 1) return diffusion_f32_variant_name(r, v);
     if (v < 0 || v >= diffusion_num_variants(dtype, r)) return "?";
+    if (!fx) return F64_PIPE_NAMES[r];  // one shape whatever the variant
     return r == 3 ? F64_NAMES[v] : F64_NAMES_OTHER[r];
 }
 

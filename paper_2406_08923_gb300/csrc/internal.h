@@ -104,7 +104,7 @@ cudaError_t launch_diffusion(int dtype, const CUtensorMap *map_in, const void *i
                              const DiffCoef &c, bool images, unsigned *err, cudaStream_t s,
                              int variant, int zmode = 0);
 int diffusion_num_variants(int dtype, int r);
-const char *diffusion_variant_name(int dtype, int r, int variant);
+const char *diffusion_variant_name(int dtype, int r, int variant, bool fx);
 // TMA box (x, y, z) of a variant; fx: the plan's weights fit the fixed-point kernel
 void diffusion_box(int dtype, int r, int variant, bool fx, int box[3]);
 // The FP64 kernel in 64-bit fixed point (diffusion_fx.cu).

@@ -146,6 +146,7 @@ def test_localised_fields(cuda_lib, r, kind):
 def test_weights_of_a_backward_step_run_on_the_fp64_pipe(cuda_lib):
     shape, r, h = (12, 18, 40), 3, (0.5, 0.5, 0.5)  # dt < 0: the signs the fixed-point kernel has not compiled in
     p = _plan(shape, r, h, dt=-0.01)
+    assert p.variant()[2].startswith("vx2") and _plan(shape, r, h).variant()[2].startswith("fx64")
     f = np.random.default_rng(9).standard_normal(shape)
     ref, mag = _reference(f, r, h, dt=-0.01)
     assert np.all(np.abs(_step(p, f)[0] - ref) <= 21 * 2.0 ** -53 * mag)

@@ -173,3 +173,18 @@ def test_composed_int32_sweeps_are_exact(cuda_lib, r, n, sweeps):
     whole = p.view3(b[0])[0, 0].cpu().numpy().astype(np.uint32)
     o = p.origin[0]
     assert np.array_equal(whole[o - r:o + n + r], np.pad(ref, r, mode="wrap"))
+
+
+@pytest.mark.parametrize("r,storage,g,bc,name", [
+    (3, L.STENCIL_F64, [0.1] * 7, L.STENCIL_BC_PERIODIC, "composed_fixed_point"),
+    (1, L.STENCIL_F64, [0.3] * 3, L.STENCIL_BC_PERIODIC, "composed_fixed_point"),
+    (3, L.STENCIL_F64, [0.1] * 7, L.STENCIL_BC_CALLER, "composed_fixed_point"),
+    (1, L.STENCIL_F64, [0.3] * 3, L.STENCIL_BC_CALLER, "runtime_chunk_scalar_temporal_blocking"),
+    (3, L.STENCIL_F64, [2.0 ** -120] * 7, L.STENCIL_BC_PERIODIC, "runtime_chunk_scalar_temporal_blocking"),
+    (3, L.STENCIL_F64, [np.nan] * 7, L.STENCIL_BC_PERIODIC, "runtime_chunk_scalar_temporal_blocking"),
+    (2, L.STENCIL_I32, [1, -2, 3, 1, 1], L.STENCIL_BC_PERIODIC, "composed_v9"),
+    (2, L.STENCIL_I32, [1, -2, 3, 1, 1], L.STENCIL_BC_CALLER, "chunk2184_v9_temporal_blocking"),
+    (3, L.STENCIL_F32, [0.1] * 7, L.STENCIL_BC_PERIODIC, "chunk2184_v9_temporal_blocking")])
+def test_variant_name_tells_the_kernel(cuda_lib, r, storage, g, bc, name):
+    g = np.array(g, dtype=np.int32 if storage == L.STENCIL_I32 else np.float64)
+    assert L.Plan(1, (5000,), r, 1, bc, L.STENCIL_XCORR, storage, storage, coeffs=g).variant()[2] == name
