@@ -324,8 +324,9 @@ const char *stencil_last_error_detail(stencil_t p) {
 }
 
 // The fixed-point tables of a plan's 2r+1 weights w1 for 1 .. kmax sweeps per launch, in one
-// allocation: per k the composed weights (doubles), then the limb pairs.  Leaves p->fx empty where
-// some k's weights do not fit.  False after a CUDA error (reported in the creation detail).
+// allocation: per k the composed weights (doubles), then the limb pairs.  Ends before the first k
+// whose weights do not fit (composed weights grow or shrink with k).  False after a CUDA error
+// (reported in the creation detail).
 static bool make_fx(stencil_t p, const double *w1, int kmax) {
     std::vector<unsigned char> host;
     std::vector<FxSweep> fx;
@@ -335,7 +336,7 @@ static bool make_fx(stencil_t p, const double *w1, int kmax) {
     for (int k = 1; k <= kmax; ++k) {
         FxSweep f{};
         if (k > 1) fx_convolve(w1, p->radius, hi, lo);
-        if (!fx_wide_weights(hi.data(), lo.data(), (int)hi.size(), limbs, &f.ew)) return true;
+        if (!fx_wide_weights(hi.data(), lo.data(), (int)hi.size(), limbs, &f.ew)) break;
         f.r = k * p->radius;
         f.r1 = p->radius;
         f.sweeps = k;
@@ -346,6 +347,7 @@ static bool make_fx(stencil_t p, const double *w1, int kmax) {
         at.emplace_back(a, b);
         fx.push_back(f);
     }
+    if (fx.empty()) return true;
     cudaError_t e = cudaMalloc(&p->fxmem, host.size());
     if (e == cudaSuccess) e = cudaMemcpy(p->fxmem, host.data(), host.size(), cudaMemcpyHostToDevice);
     if (e != cudaSuccess) {
@@ -819,7 +821,8 @@ stencil_status stencil_step(stencil_t p, void *const *fin, void *const *fout, in
     if (xcorr_like) {
         // temporal blocking for the radius <= 4 kernel; one sweep per launch otherwise
         const bool single = !periodic || p->kind == STENCIL_MAXFILTER || (p->kind == STENCIL_XCORR && !xcorr_blocked(p));
-        const int maxs = single ? 1 : xcorr_max_sweeps_per_launch(p->radius);
+        // as many sweeps per launch as the fixed-point tables hold, if they hold several
+        const int maxs = single ? 1 : p->fx.size() > 1 ? (int)p->fx.size() : xcorr_max_sweeps_per_launch(p->radius);
         for (int left = nsteps; left > 0;) {
             int k = std::min(left, maxs);
             sweeps.push_back(k);

@@ -175,6 +175,23 @@ def test_composed_int32_sweeps_are_exact(cuda_lib, r, n, sweeps):
     assert np.array_equal(whole[o - r:o + n + r], np.pad(ref, r, mode="wrap"))
 
 
+# weights whose sum is far from 1 leave the range of fixed point after some sweeps (11, 16 and 15 at
+# r = 3): fewer sweeps still compose, and calls of more take several launches
+@pytest.mark.parametrize("total", [1000.0, 100.0, 0.01])
+@pytest.mark.parametrize("r,sweeps", [(3, 1), (3, 10), (3, 16), (3, 25), (4, 16)])
+def test_weights_that_compose_for_some_sweeps(cuda_lib, total, r, sweeps):
+    n, g = 4099, np.full(2 * r + 1, total / (2 * r + 1))
+    p = L.Plan(1, (n,), r, 1, L.STENCIL_BC_PERIODIC, L.STENCIL_XCORR, L.STENCIL_F64, L.STENCIL_F64, coeffs=g)
+    assert p.variant()[2] == "composed_fixed_point"
+    f = np.random.default_rng(8).standard_normal(n)
+    got, (lo, hi) = _run(f, g, sweeps=sweeps)
+    ref, mag = f.astype(np.longdouble), np.abs(f).astype(np.longdouble)
+    for _ in range(sweeps):
+        ref, mag = _reference(np.pad(ref, r, mode="wrap"), g)[0], _reference(np.pad(mag, r, mode="wrap"), np.abs(g))[0]
+    assert float(np.max(np.abs(got - ref) / (sweeps * (2 * r + 1) * 2.0 ** -53 * mag))) <= 1.0
+    assert np.array_equal(lo, got[-r:]) and np.array_equal(hi, got[:r])
+
+
 @pytest.mark.parametrize("r,storage,g,bc,name", [
     (3, L.STENCIL_F64, [0.1] * 7, L.STENCIL_BC_PERIODIC, "composed_fixed_point"),
     (1, L.STENCIL_F64, [0.3] * 3, L.STENCIL_BC_PERIODIC, "composed_fixed_point"),
