@@ -10,6 +10,7 @@
 #include <fstream>
 #include <map>
 #include <mutex>
+#include <new>
 #include <sstream>
 #include <string>
 #include <vector>
@@ -590,19 +591,26 @@ stencil_status stencil_create(int ndim, const int64_t dims[3], int radius, const
             if (e != cudaSuccess) { cuda_fail(nullptr, e, "cudaMemcpy(weights)"); okay = false; }
         }
     }
-    if (okay && storage == STENCIL_F64 && radius > 0 &&
-        (kind == STENCIL_XCORR || (kind == STENCIL_DIFFUSION && ndim == 1))) {
-        const double *w1 = kind == STENCIL_XCORR && radius > 4 ? wide_w.data() : p->gd;
-        okay = make_fx(p, w1, bc == STENCIL_BC_PERIODIC && radius <= 4 ? xcorr_max_sweeps_per_launch(radius) : 1);
+    bool host_memory = true;
+    try {
+        if (okay && storage == STENCIL_F64 && radius > 0 &&
+            (kind == STENCIL_XCORR || (kind == STENCIL_DIFFUSION && ndim == 1))) {
+            const double *w1 = kind == STENCIL_XCORR && radius > 4 ? wide_w.data() : p->gd;
+            okay = make_fx(p, w1, bc == STENCIL_BC_PERIODIC && radius <= 4 ? xcorr_max_sweeps_per_launch(radius) : 1);
+        }
+        if (storage == STENCIL_I32 && kind == STENCIL_XCORR && radius > 0 && bc == STENCIL_BC_PERIODIC)
+            i32_compose(p->gi, radius, xcorr_max_sweeps_per_launch(radius), p->i32);
+    } catch (const std::bad_alloc &) {  // nothing is thrown across the C ABI
+        g_create_detail = "host allocation of the weight tables failed";
+        okay = host_memory = false;
     }
-    if (storage == STENCIL_I32 && kind == STENCIL_XCORR && radius > 0 && bc == STENCIL_BC_PERIODIC)
-        i32_compose(p->gi, radius, xcorr_max_sweeps_per_launch(radius), p->i32);
     if (okay) {
         e = cudaMemset(p->err, 0, sizeof(unsigned));
         if (e != cudaSuccess) { cuda_fail(nullptr, e, "cudaMemset(error word)"); okay = false; }
     }
     if (!okay) {
-        stencil_status st = g_create_detail.find("cudaErrorMemoryAllocation") != std::string::npos ? STENCIL_ENOMEM : STENCIL_ECUDA;
+        stencil_status st = !host_memory || g_create_detail.find("cudaErrorMemoryAllocation") != std::string::npos
+                                ? STENCIL_ENOMEM : STENCIL_ECUDA;
         free_scratch(p);
         delete p;
         return st;
