@@ -4,8 +4,9 @@
 // (Eqs. 5 and 7): f' = g0 f + sum_axes sum_{a=1..3} g_{axis,a} (f(+a) + f(-a)).
 //
 // This file holds the kernel on the FP64 pipe (~1/60 of the FP32 rate), which runs where the weights
-// do not fit fixed point (diffusion_fx.cu, four times faster, runs all others), and the launch and
-// variant functions of every 3D step; FP32 has its own issue-lean kernel in diffusion_f32.cu.
+// do not fit fixed point (diffusion_fx.cu runs all others: 256^3, r = 3, a smooth field 235 us per step,
+// here 596), and the launch and variant functions of every 3D step; FP32 has its own issue-lean kernel
+// in diffusion_f32.cu.
 //
 // GB300 design (2.5D z-streaming):
 //   * A CTA owns a TX x TY tile of the xy-plane (TX = 32 VX, TY = BY RY) and marches along z
@@ -13,8 +14,7 @@
 //     (TX + 8) x (TY + 6) arrives by one TMA load (cp.async.bulk.tensor.3d) in a ring of
 //     NSLOT shared-memory slots, completion on one mbarrier per slot; loads run NSLOT - 3
 //     planes ahead of the compute.
-//   * A thread owns VX = 2 VP consecutive x cells in RY rows and computes them as VP pairs
-//     (the pair template also admits FP32 with Blackwell's packed FP32x2 FMA/ADD).  Shared
+//   * A thread owns VX = 2 VP consecutive x cells in RY rows and computes them as VP pairs.  Shared
 //     memory is read with 16-byte vector loads.
 //   * Each iteration computes ZB consecutive z planes (register blocking in z).  The
 //     z-columns (planes z-3..z+ZB+2) live in a register queue that shifts by ZB once per
@@ -35,26 +35,8 @@ namespace stn {
 template <int N> __device__ __forceinline__ int slot_of(int j) { return (int)((unsigned)j & (N - 1)); }
 template <int N> __device__ __forceinline__ uint32_t parity_of(int j) { return ((unsigned)j / (unsigned)N) & 1u; }
 
-// Pair arithmetic: PK selects Blackwell's packed FP32x2 instructions for float; otherwise
-// the two lanes are computed with scalar instructions.
-template <typename T, bool PK> struct PairOps;
-template <> struct PairOps<float, true> {
-    using P = float2;
-    static __device__ __forceinline__ P add(P a, P b) { return __fadd2_rn(a, b); }
-    static __device__ __forceinline__ P mul(P a, P b) { return __fmul2_rn(a, b); }
-    static __device__ __forceinline__ P fma2(P a, P b, P c) { return __ffma2_rn(a, b, c); }
-    static __device__ __forceinline__ P make(float a, float b) { return make_float2(a, b); }
-};
-template <> struct PairOps<float, false> {
-    using P = float2;
-    static __device__ __forceinline__ P add(P a, P b) { return make_float2(a.x + b.x, a.y + b.y); }
-    static __device__ __forceinline__ P mul(P a, P b) { return make_float2(a.x * b.x, a.y * b.y); }
-    static __device__ __forceinline__ P fma2(P a, P b, P c) {
-        return make_float2(fmaf(a.x, b.x, c.x), fmaf(a.y, b.y, c.y));
-    }
-    static __device__ __forceinline__ P make(float a, float b) { return make_float2(a, b); }
-};
-template <bool PK> struct PairOps<double, PK> {
+// Pair arithmetic.
+struct PairOps {
     using P = double2;
     static __device__ __forceinline__ P add(P a, P b) { return make_double2(a.x + b.x, a.y + b.y); }
     static __device__ __forceinline__ P mul(P a, P b) { return make_double2(a.x * b.x, a.y * b.y); }
@@ -115,13 +97,13 @@ __device__ __forceinline__ void ld_vec(const T *p, T (&dst)[N]) {
 // One xy-tile of one z-chunk: the whole 2.5D pipeline of a CTA.  `map` may point at a
 // __grid_constant__ parameter or at a descriptor in global memory (batched launches).
 // Returns false if a bounded wait expired (ERR_TIMEOUT recorded, loads drained).
-template <typename T, int VP, int BY, int RY, int ZB, int NSLOT, bool PK, bool PDL, int R>
+template <typename T, int VP, int BY, int RY, int ZB, int NSLOT, bool PDL, int R>
 __device__ __forceinline__ bool diffusion_tile(const CUtensorMap *map, T *__restrict__ out, const Geom &g,
                                                const DC<T> &c, int tile_x, int tile_y, int tile_z, int zc,
                                                int images, unsigned *err, T *ring, uint64_t *full) {
     using Cfg = DiffCfg<T, VP, BY, RY, ZB, NSLOT, R>;
-    using O = PairOps<T, PK>;
-    using P = typename O::P;
+    using O = PairOps;
+    using P = O::P;
     constexpr int VX = Cfg::VX, LV = Cfg::LV;
     const int lane = threadIdx.x & 31, wy = threadIdx.x >> 5;
     const int x0 = tile_x * Cfg::TX, y0 = tile_y * Cfg::TY;
@@ -306,13 +288,8 @@ __device__ __forceinline__ bool diffusion_tile(const CUtensorMap *map, T *__rest
                                     for (int xi = 0; xi < 2; ++xi) {
                                         if (xi == 1 && (!xvec || xshift == 0)) break;
                                         T *xp = rp + (xi ? xshift : 0);
-                                        if constexpr (VP == 2 && sizeof(T) == 4) {  // one 16-byte store
-                                            *reinterpret_cast<float4 *>(xp) =
-                                                make_float4(res[r][0].x, res[r][0].y, res[r][1].x, res[r][1].y);
-                                        } else {
 #pragma unroll
-                                            for (int p = 0; p < VP; ++p) *reinterpret_cast<P *>(xp + 2 * p) = res[r][p];
-                                        }
+                                        for (int p = 0; p < VP; ++p) *reinterpret_cast<P *>(xp + 2 * p) = res[r][p];
                                     }
                                     if (xmask) {
 #pragma unroll
@@ -364,7 +341,7 @@ __device__ __forceinline__ bool diffusion_tile(const CUtensorMap *map, T *__rest
     return !bad;
 }
 
-template <typename T, int VP, int BY, int RY, int ZB, int NSLOT, bool PK, int R>
+template <typename T, int VP, int BY, int RY, int ZB, int NSLOT, int R>
 __global__ void __launch_bounds__(32 * BY)
 diffusion_kernel(const __grid_constant__ CUtensorMap map_in, T *__restrict__ out, Geom g, DC<T> c,
                  int zc, int images, unsigned *err) {
@@ -372,7 +349,7 @@ diffusion_kernel(const __grid_constant__ CUtensorMap map_in, T *__restrict__ out
     // TMA destinations are kept 128-byte aligned (dynamic smem has 128 spare bytes)
     T *ring = reinterpret_cast<T *>((reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~uintptr_t(127));
     __shared__ __align__(8) uint64_t full[NSLOT];
-    diffusion_tile<T, VP, BY, RY, ZB, NSLOT, PK, true, R>(&map_in, out, g, c, blockIdx.x, blockIdx.y, blockIdx.z,
+    diffusion_tile<T, VP, BY, RY, ZB, NSLOT, true, R>(&map_in, out, g, c, blockIdx.x, blockIdx.y, blockIdx.z,
                                                           zc, images, err, ring, full);
 }
 
@@ -413,7 +390,7 @@ int device_sms() {
     return sms[dev];
 }
 
-template <typename T, int VP, int BY, int RY, int ZB, int NSLOT, bool PK, int R>
+template <typename T, int VP, int BY, int RY, int ZB, int NSLOT, int R>
 static cudaError_t run(const CUtensorMap *map, void *out, const Geom &g, const DiffCoef &dc, bool images,
                        unsigned *err, cudaStream_t s, int zmode) {
     using Cfg = DiffCfg<T, VP, BY, RY, ZB, NSLOT, R>;
@@ -421,7 +398,7 @@ static cudaError_t run(const CUtensorMap *map, void *out, const Geom &g, const D
     c.g0 = (T)dc.g0;
     for (int a = 0; a < 3; ++a)
         for (int b = 0; b < 4; ++b) c.ga[a][b] = (T)dc.ga[a][b];
-    auto k = diffusion_kernel<T, VP, BY, RY, ZB, NSLOT, PK, R>;
+    auto k = diffusion_kernel<T, VP, BY, RY, ZB, NSLOT, R>;
     static int occ[64] = {};  // resident CTAs per SM, per device
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -447,11 +424,11 @@ static cudaError_t run(const CUtensorMap *map, void *out, const Geom &g, const D
                       err);
 }
 
-// The shape of the FP64-pipe kernel: (VP pairs per row, BY warps, RY rows, ZB planes, NSLOT, packed
-// FP32x2).  It serves plans whose weights do not fit the fixed-point kernel of diffusion_fx.cu
-// (not finite, or the signs of a backward or far from stable step); every other FP64 plan runs that one, whose launch
+// The shape of the FP64-pipe kernel: (VP pairs per row, BY warps, RY rows, ZB planes, NSLOT).  It serves
+// plans whose weights do not fit the fixed-point kernel of diffusion_fx.cu (not finite, all zero, or the
+// signs of a backward or far from stable step); every other FP64 plan runs that one, whose launch
 // shapes the variants of radius 3 name.
-#define DIFF_VARIANT_F64(X) X(1, 8, 1, 2, 8, false)
+#define DIFF_VARIANT_F64(X) X(1, 8, 1, 2, 8)
 static const char *F64_NAMES[] = {"fx64x16", "fx64x16_more_chunks", "fx64x16_fewer_chunks", "fx64x16_even_waves"};
 static const char *F64_PIPE_NAMES[] = {"?", "f64_r1_vx2_by8_ry1_zb2_s8", "f64_r2_vx2_by8_ry1_zb2_s8", "vx2_by8_ry1_zb2_s8",
                                        "f64_r4_vx2_by8_ry1_zb2_s8"};
@@ -472,7 +449,7 @@ const char *diffusion_variant_name(int dtype, int r, int v, bool fx) {
 void diffusion_box(int dtype, int r, int v, bool fx, int box[3]) {
     if (dtype != 1) return diffusion_f32_box(r, v, box);
     if (fx) return diffusion_fx_box(r, box);
-#define X(VP, BY, RY, ZB, NS, PK) box[0] = 64 * VP + 8, box[1] = BY * RY + 2 * r, box[2] = 1;
+#define X(VP, BY, RY, ZB, NS) box[0] = 64 * VP + 8, box[1] = BY * RY + 2 * r, box[2] = 1;
     DIFF_VARIANT_F64(X)
 #undef X
 }
@@ -480,7 +457,7 @@ void diffusion_box(int dtype, int r, int v, bool fx, int box[3]) {
 template <int R>
 static cudaError_t dispatch_f64(const CUtensorMap *map, void *out, const Geom &g, const DiffCoef &c, bool images,
                                 unsigned *err, cudaStream_t s, int zmode) {
-#define X(VP, BY, RY, ZB, NS, PK) return run<double, VP, BY, RY, ZB, NS, PK, R>(map, out, g, c, images, err, s, zmode);
+#define X(VP, BY, RY, ZB, NS) return run<double, VP, BY, RY, ZB, NS, R>(map, out, g, c, images, err, s, zmode);
     DIFF_VARIANT_F64(X)
 #undef X
 }

@@ -49,6 +49,10 @@ cudaError_t launch_xcorr(int dtype, int r, const void *in, void *out, const Geom
 int xcorr_wide_max_radius();
 cudaError_t launch_xcorr_wide(int dtype, int r, const void *in, void *out, const Geom &g, const void *wdev,
                               bool periodic, bool images, unsigned *err, cudaStream_t s);
+// One asynchronous 4-byte copy into shared memory (cp.async.wait_all ends them).
+__device__ __forceinline__ void cp_async4(void *dst, const void *src) {
+    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
+}
 // FP64 cross-correlation in fixed point, and sweeps composed into one (xcorr_fx.cu).
 // `limbs` receives the limb pairs of weights hi + lo (lo may be null) and `ew` their scale; false
 // where fixed point does not apply (a weight is not finite, all are zero, exponents out of range).

@@ -276,9 +276,6 @@ xcorr_wide_fx_kernel(const double *__restrict__ in, double *__restrict__ out, Ge
         }
 }
 
-__device__ __forceinline__ void cp_async4(void *dst, const void *src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
-}
 __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wait_all;" ::: "memory"); }
 
 // int32 sweeps composed into one correlation of radius r <= 64 modulo 2^32.  Shared loads as above;

@@ -32,10 +32,6 @@ template <int V_> struct PairCfg {
     static_assert(V % 2 == 1, "");
 };
 
-__device__ __forceinline__ void cp_async4(void *dst, const void *src) {
-    asm volatile("cp.async.ca.shared.global [%0], [%1], 4;" ::"r"(smem_addr(dst)), "l"(src) : "memory");
-}
-
 template <int V, int MINB>
 __global__ void __launch_bounds__(PT, MINB)
 xcorr_pair_kernel(const float *__restrict__ in, float *__restrict__ out, Geom geo, const float *__restrict__ wg, int r,
