@@ -30,9 +30,9 @@
 //     below the bound (pulses and spikes far above their surroundings).  That is looked at only where a
 //     quarter of the threads load mostly small cells.  A chunk of zeros stores zeros.
 //     3 M cells, r = 100, in us on the FP64 pipe, here, and with each output by itself: noise 1063, 242,
-//     246; pulses of 100 cells 1062, 1035, 1249; a spike every 997 cells 1062, 938, 1273; zeros 1062, 11,
+//     246; pulses of 100 cells 1062, 1035, 1249; a spike every 997 cells 1062, 1066, 1273; zeros 1062, 11,
 //     1057. 2^20 cells, 10 sweeps of r = 3: noise 127, 33.2, 33.3; pulses 127, 134, 152; spikes 127,
-//     119, 160. Noise over 60 binary orders at r = 1000 is the slowest, 3364, 4105, 4806.
+//     136, 160. Noise over 60 binary orders at r = 1000 is the slowest, 3364, 4063, 4806.
 #include <algorithm>
 #include <vector>
 
@@ -153,7 +153,8 @@ xcorr_wide_fx_kernel(const double *__restrict__ in, double *__restrict__ out, Ge
         int small = 0;
         if (nw >= FAR_WEIGHTS) {
 #pragma unroll
-            for (int k = 0; k < KR; ++k) small += (int)(((u32)__double2hiint(kept[k]) & 0x7fffffffu) >> 20) + 7 < E;
+            for (int k = 0; k < KR; ++k)
+                small += (int)(((u32)__double2hiint(kept[k]) & 0x7fffffffu) >> 20) + 7 < E && tid + k * FT < used;
         }
         if (__syncthreads_count(2 * small > KR) > FT / 4) {
             // 4 outputs per warp, spread over the chunk, whose sum |w f| is taken whole
@@ -217,14 +218,18 @@ xcorr_wide_fx_kernel(const double *__restrict__ in, double *__restrict__ out, Ge
             for (u32 i = tid; i < nl; i += FT) {
                 const int p = list[i];
                 u64 mag = 0;  // sum |w f| in units of 2^2 of the results' last place
-                int any = 0;
-                for (int j = 0; j < nw && mag < (1ull << 53); ++j) {
+                for (int j = 0; j < nw && mag < (1ull << 53); ++j)
                     mag += (u64)(u32)abs(ws[j].y) * (u32)abs(s[p + j].y);
-                    any |= s[p + j].x | s[p + j].y;
+                if (mag >= (1ull << 53)) {
+                    list[i] = DONE;
+                } else {
+                    int any = 0;
+                    for (int j = 0; j < nw && !any; ++j) any = s[p + j].x | s[p + j].y;
+                    if (!any) {
+                        list[i] = (uint16_t)(p | EMPTY);
+                        empty = true;
+                    }
                 }
-                empty = empty || !any;
-                if (mag >= (1ull << 53)) list[i] = DONE;
-                else if (!any) list[i] = (uint16_t)(p | EMPTY);
             }
             if (__syncthreads_or(empty) && !faint_cells()) {  // windows of zeros
                 for (u32 i = tid; i < nl; i += FT)
