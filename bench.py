@@ -55,8 +55,8 @@ SRC_HEAT32 = {"diffusion_f32.cu": "2cacbf4617d874ff", "common.cuh": "3f7458d1c75
 NCU_TRAFFIC = {
     # dram__bytes_read.sum + dram__bytes_write.sum per launch, mean of 3 launches of a 1-pass capture at
     # the bench sizes (profiles/dram_traffic_full_size.md); MHD: the mean over the 3 RK substeps
-    "heat_f64": {"variant": "fx64x16", "zmode": 0, "bytes": 150618027 + 100469845,
-                 "src": {"diffusion_fx.cu": "b8d791036485d50b", "fixed.cuh": "00ebb1ce8309c887", "common.cuh": "3f7458d1c75ca5f9"}},
+    "heat_f64": {"variant": "fx64x16", "zmode": 0, "bytes": 147689301 + 102447019,
+                 "src": {"diffusion_fx.cu": "f11a4d341b8b66a9", "fixed.cuh": "84e7b11e6dde86ee", "common.cuh": "3f7458d1c75ca5f9"}},
     "heat_f32": {"variant": "f32_by4_ry2_zb2_s8_m3", "zmode": 0, "bytes": 82052181 + 21760939, "src": SRC_HEAT32},
     "heat_f32_512": {"variant": "f32_by8_ry2_zb2_s8_m2", "zmode": 0, "bytes": 586154069 + 507398315,
                      "src": SRC_HEAT32},
@@ -95,7 +95,7 @@ FP64_PIPE_TINSTR = 2 * 152 * 2.07e9 / 1e12  # FP64 instructions (DFMA, DADD, DMU
 # 6th-order derivatives (600 flop), the right-hand side of Eqs. A1-A4 and the 2N-storage RK
 # update, counted by tests/mhd_flops.py (checked against the oracle in test_mhd_flops.py).
 MHD_FLOPS_PER_CELL_SUBSTEP = 2465 / 3
-MHD_F64_INSTR = 204  # FP64 instructions per cell-substep the kernel executes (ncu sass counts)
+MHD_F64_INSTR = 198  # FP64 instructions per cell-substep the kernel executes (ncu sass counts)
 # 32 x 32 + 64-bit multiply-adds of the integer pipe, which the FP64 linear stencils run on: 32
 # lanes per clock and SM (28 to 30 measured with distinct operands).
 INT_PIPE_TINSTR = 32 * 152 * 2.07e9 / 1e12

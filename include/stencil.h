@@ -130,8 +130,9 @@ enum { STENCIL_MHD_LNRHO = 0, STENCIL_MHD_UX, STENCIL_MHD_UY, STENCIL_MHD_UZ,
  *   out      receives the plan.
  *
  * The only call that allocates device memory: library-owned scratch (one extra field set for
- * ping-pong, the RK register and Kahan compensation arrays for MHD8, reduction buffers, and
- * for XCORR of radius > 4 a device copy of the weights).
+ * ping-pong, the RK register and Kahan compensation arrays for MHD8, reduction buffers, for
+ * XCORR of radius > 4 a device copy of the weights, and for F64 XCORR and 1D DIFFUSION tables of
+ * the weights of up to 16 sweeps).
  * Returns EINVAL on invalid arguments, EUNSUPPORTED on valid but unimplemented
  * combinations, ENOMEM/ECUDA if the scratch allocation fails (nothing is leaked).
  */
@@ -159,7 +160,10 @@ stencil_status stencil_layout(stencil_t plan, int64_t padded[3], int64_t pitch[3
 /*
  * stencil_step -- advance `nsteps` iterations (Sec. 2.4: f'_i = zeta(f^, i) for all i).
  *
- *   XCORR      nsteps sweeps of Eq. 3 (each sweep feeds the next).
+ *   XCORR      nsteps sweeps of Eq. 3 (each sweep feeds the next).  Sweeps of one call may be
+ *              evaluated as one correlation with the composed weights: the same result modulo
+ *              2^32, and in F64 (and 1D DIFFUSION) one with fewer roundings, whose last bits
+ *              differ from those of as many calls of one sweep.
  *   MAXFILTER  nsteps max-filter sweeps (each sweep feeds the next).
  *   DIFFUSION  nsteps forward-Euler steps of Eqs. 4-7.
  *   MHD8       nsteps RK3 steps (3 substeps each) of Eqs. A1-A4.

@@ -7,13 +7,13 @@
 // two are equal bit for bit.  In FP64 the composed sum has fewer roundings than the sweeps; its
 // weights are convolved in double-double arithmetic, so that the fixed-point weights are
 // as exact as those of a single sweep.  2^20 cells, 10 sweeps, r = 3: int32 12.6 -> 6.6 us on the
-// device, FP64 129 -> 35 us.
+// device, FP64 129 -> 33 us.
 //
 // FP64.  2r+1 FP64 multiply-adds per output ran at 99 % of the FP64 pipe (2 per clock and SM).
 // Here a CTA converts its chunk of cells, halo included, to signed 59-bit integers of one binary
 // scale, split into two 30-bit limbs, and the weights come as limbs too.  A product is then three
 // 32 x 32 + 64-bit multiply-adds (the product of the two low limbs, below 2^-60 of the scale, is
-// left out), at 32 per clock and SM: 5.3 times the FP64 rate.  3 M cells, r = 100: 1063 -> 238 us.
+// left out), at 32 per clock and SM: 5.3 times the FP64 rate.  3 M cells, r = 100: 1063 -> 234 us.
 //
 //   * As in xcorr_wide.cu each thread computes V consecutive outputs (V odd: conflict-free shared
 //     loads) and keeps V weights and 2V-1 cells in registers per block of V weights.

@@ -15,7 +15,7 @@
 //     other's staging and stores.  (Persistent CTAs with the next chunk's copies in flight
 //     measured no faster: 98 against 97 us at r = 64 before the window was kept.)
 //   * Bound by the FP32 pipe and the shared loads together (58 % and about 50 % busy at r = 64).
-//     2^24 cells: r = 64 101.7 -> 92.5 us, r = 256 346 -> 295; 2^20 cells, r = 64 15.6 -> 10.5.
+//     2^24 cells: r = 64 101.7 -> 91.4 us, r = 256 346 -> 298; 2^20 cells, r = 64 15.6 -> 10.5.
 #include <algorithm>
 
 #include "internal.h"

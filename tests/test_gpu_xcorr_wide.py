@@ -35,8 +35,9 @@ def _weights(r, signed):
 
 
 @pytest.mark.parametrize("storage", [L.STENCIL_F64, L.STENCIL_F32])
-# radii cover every compiled register-block size V (FP32 9/11/13/15, FP64 5/7/9), and the
-# sizes both the bulk-copied interior chunks and the staged edge chunks
+# radii and sizes of every block size of the kernels that serve periodic arrays (csrc/xcorr_pair.cu, V = 3 to 13;
+# csrc/xcorr_fx.cu, V = 3, 7, 9), interior and edge chunks.  csrc/xcorr_wide.cu serves a caller's halo in FP32
+# and FP64 weights out of range: below, test_gpu_xcorr_pair.py and test_gpu_fp64_pipe.py.
 @pytest.mark.parametrize("r,n,sweeps", [(5, 3001, 1), (8, 20001, 2), (16, 70001, 3), (32, 50003, 1), (100, 4097, 2),
                                         (128, 300007, 1), (1024, 5000, 1), (1024, (1 << 20) + 3, 2)])
 def test_wide_xcorr_matches_oracle(cuda_lib, storage, r, n, sweeps):
@@ -47,7 +48,7 @@ def test_wide_xcorr_matches_oracle(cuda_lib, storage, r, n, sweeps):
         data = data.astype(np.float32).astype(np.float64)
         g = g.astype(np.float32).astype(np.float64)
     p, a, b = _run(L.STENCIL_XCORR, storage, n, r, data, coeffs=g, sweeps=sweeps)
-    # FP32 up to radius 32 runs the temporally blocked kernel, the rest the wide one
+    # FP32 up to radius 32 runs the temporally blocked kernel, the rest the wide ones
     blocked = storage == L.STENCIL_F32 and r <= 32
     assert (p.variant()[2] == "wide_register_blocked") != blocked, p.variant()[2]
     got = p.download(b)[0]
