@@ -32,9 +32,8 @@
 //   * Accuracy by field, not by axis: next to larger neighbours on one axis, the difference of values
 //     far below the scale along another is exact to 2^-60 of the scale only, where FP64 keeps its digits.
 //   * One RK3 step in ms, the FP64 pipe's kernel and this one: 256^3 waves 60.8 and 33.4, a vortex of 24
-//     cells in 256^3 60.8 and 52.4.  128^3, which fills 128 tiles in 2 chunks each unevenly: waves 7.9 and
-//     5.2, a vortex of 6, 10, 16 cells 7.9 and 10.2, 10.3, 10.2, a shear layer 7.9 and 9.6 (before fields
-//     were taken in FP64 by warps 13.7, 16.9, 14.9, 17.1).
+//     cells in 256^3 60.8 and 52.4; 128^3 waves 7.9 and 5.1, a vortex of 6, 10, 16 cells 7.9 and 9.1, 9.0,
+//     7.8, a shear layer 7.9 and 8.2 (before fields were taken in FP64 by warps 13.7, 16.9, 14.9, 17.1).
 #include <algorithm>
 
 #include "fixed.cuh"
@@ -574,14 +573,17 @@ bool fx_mhd_weights(const MhdConst &c, FxMhd &o) {
 }
 
 // Planes per z-chunk: the fewest periods over the waves of CTAs (one per SM), when a chunk's start costs
-// `start` of them.  At most 64: localised fields make some CTAs cost twice what others do, and longer
-// chunks leave the SMs unevenly loaded (128^3 with a vortex of 16 cells 14.8 ms a step in chunks of 128
-// planes, 10.2 in chunks of 64; waves 5.05 and 5.2).
+// `start` of them.  Localised fields make some CTAs cost twice what others do, and few long chunks
+// leave the SMs unevenly loaded, so chunks have at most 32 planes where the tiles are fewer than two per SM,
+// else 64 (128^3, 128 tiles, ms a step in chunks of 128, 64, 32 planes: a vortex of 16 cells 14.8, 10.2,
+// 7.8, a shear layer 13.7, 9.6, 8.2, waves 5.05, 5.2, 5.1; 256^3, 512 tiles, in chunks of 64 and 32: waves
+// 33.7 and 34.3, a vortex of 24 cells 52.8 and 52.6).
 int chunk_planes(int tiles, int nz, int start) {
     const int sms = device_sms();
     int best = 1;
     int64_t least = INT64_MAX;
-    for (int c = (nz + 63) / 64; c <= nz; ++c) {
+    const int most = tiles < 2 * sms ? 32 : 64;
+    for (int c = (nz + most - 1) / most; c <= nz; ++c) {
         const int zc = (nz + c - 1) / c;
         const int64_t ctas = (int64_t)tiles * ((nz + zc - 1) / zc), cost = (ctas + sms - 1) / sms * (zc + start);
         if (cost < least) {

@@ -169,8 +169,8 @@ def test_variants_and_chunk_lengths_are_bit_identical(cuda_lib, K):
 
 def test_more_listed_cells_than_the_list_holds(cuda_lib):
     # s at the end of the exponent range: the two columns of the last tiles list every cell, 16 per
-    # plane, in chunks of up to 128 planes; elsewhere whole warps take the field in FP64
-    shape = (140, 50, 130)
+    # plane, in chunks of up to 128 planes (tiles for two per SM); elsewhere whole warps take the field in FP64
+    shape = (132, 272, 130)
     f8 = 1e-3 * _fields("waves", shape)
     f8[7] *= 1e-305
     p, _ = _plan(shape)
