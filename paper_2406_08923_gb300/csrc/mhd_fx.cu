@@ -3,7 +3,7 @@
 // Of the 600 FP64 instructions per cell and substep of the kernel in mhd.cu, which kept the FP64
 // pipe 80 % busy, 470 are the 57 linear differences of gamma = A B (Eq. 8).  Here they are sums of
 // products on the integer pipe (fixed.cuh); the right-hand side of Eqs. A1-A4, the closure and
-// the RK update stay in FP64, on the exact cell values.  One RK3 step of 256^3: 60.8 -> 33.4 ms.
+// the RK update stay in FP64, on the exact cell values.  One RK3 step of 256^3: 60.8 -> 32.6 ms.
 //
 //   * z-streaming as in mhd.cu: 16 x 8 cells per CTA, planes of all 8 fields in a ring of 8 slots.
 //     An arriving plane is converted in place to biased 60-bit integers, one binary scale per plane
@@ -27,12 +27,12 @@
 //   * A field is small at a cell where it and its six neighbours are below 2^-6 of the scale
 //     (fixed.cuh says why), and where the scale is out of range, as with infinities and NaN.  A warp
 //     with more than 4 such cells of a field takes that field's derivatives in FP64 from global
-//     memory, in the operations of mhd.cu; fewer cells are listed unless the gradient shows terms of at
+//     memory, in the operations of mhd.cu; fewer cells are marked unless the gradient shows terms of at
 //     least 2^-6 of the scale, and evaluated in FP64 throughout at the end of the CTA.
 //   * Accuracy by field, not by axis: next to larger neighbours on one axis, the difference of values
 //     far below the scale along another is exact to 2^-60 of the scale only, where FP64 keeps its digits.
-//   * One RK3 step in ms, the FP64 pipe's kernel and this one: 256^3 waves 60.8 and 33.4, a vortex of 24
-//     cells in 256^3 60.8 and 52.4; 128^3 waves 7.9 and 5.1, a vortex of 6, 10, 16 cells 7.9 and 9.1, 9.0,
+//   * One RK3 step in ms, the FP64 pipe's kernel and this one: 256^3 waves 60.8 and 32.6, a vortex of 24
+//     cells in 256^3 60.8 and 51.9; 128^3 waves 7.9 and 5.0, a vortex of 6, 10, 16 cells 7.9 and 9.1, 9.0,
 //     7.8, a shear layer 7.9 and 8.2 (before fields were taken in FP64 by warps 13.7, 16.9, 14.9, 17.1).
 #include <algorithm>
 
@@ -43,7 +43,9 @@ namespace stn {
 namespace {
 
 constexpr int TX = 16, TY = 8, GROUP = TX * TY, NGROUPS = 4, NT = NGROUPS * GROUP, NSLOT = 8;
-constexpr int LIST = 1024;
+// Cells left to FP64: a bit each until the end of the chunk, then in lists of up to LIST cells (7 bits of
+// the cell, 7 of the plane).
+constexpr int LIST = 1024, MAX_PLANES = 128;
 constexpr int FP64_CELLS = 4;  // more small cells of a warp than this: the field's derivatives in FP64
 // What the groups of derivatives hand to the group of the right-hand side, per cell: u (Laplacian,
 // h, gradient) 3 x 7, A (Laplacian, h, two of the gradient) 3 x 6, lnrho and s (gradient, Laplacian) 2 x 4.
@@ -272,8 +274,9 @@ mhd_fx_kernel(const __grid_constant__ MhdMaps maps, const __grid_constant__ FxIn
     __shared__ int scale[NSLOT][8];  // exponent codes of each slot's plane, per field
     __shared__ int top[2][8], low[2][8];  // the largest and smallest of a window, by parity
     __shared__ MK<double> ks;  // FP64 operands from registers rather than the constant bank (mhd.cu)
-    __shared__ u32 list[LIST];
-    __shared__ u32 listed;
+    __shared__ u32 marks[MAX_PLANES][GROUP / 32];
+    __shared__ uint16_t list[LIST];
+    __shared__ u32 listed, unlisted;
     double *ex = reinterpret_cast<double *>(ring + NSLOT * Cfg::SLOT_ELEMS);
     __shared__ unsigned char exleft[NGROUPS][GROUP];
     const int tid = threadIdx.x, lane = tid & 31, group = tid / GROUP, gt = tid % GROUP, tx = gt % TX, ty = gt / TX;
@@ -292,7 +295,6 @@ mhd_fx_kernel(const __grid_constant__ MhdMaps maps, const __grid_constant__ FxIn
             for (int q = 0; q < 8; ++q) scale[s][q] = 0;
         }
         mbar_fence_init();
-        listed = 0;
     }
     __syncthreads();
     const int bx = (int)g.off[0] + x0 - Cfg::HX;
@@ -422,20 +424,16 @@ mhd_fx_kernel(const __grid_constant__ MhdMaps maps, const __grid_constant__ FxIn
                 left = exleft[1][gt] | exleft[2][gt] | exleft[3][gt];
             }
             asm volatile("bar.arrive 2, %0;" ::"n"(NT) : "memory");  // ex has been read
-            if (some) {
+            const u32 mark = __ballot_sync(0xffffffffu, left);
+            if (m > 0 && lane == 0) marks[m - 1][gt / 32] = mark;
+            if (some && !left) {
                 const int z = zc0 + m - 1;
-                if (left) {
-                    const u32 at = atomicAdd(&listed, 1u);
-                    if (at < (u32)LIST) list[at] = (u32)gt | (u32)(m - 1) << 7;
-                    else fp64_cell<MODE, CONDUCT>(in, fout, wbuf, rbuf, g, ks, first, last, images, x, y, z);
-                } else {
 #pragma unroll
-                    for (int q = 0; q < 8; ++q) d.val[q] = val[q];
-                    double rhs[8];
-                    mhd_rhs_assemble<CONDUCT>(d, ks, rhs);
-                    finish_cell<MODE>(ks, rhs, val, wcur, first != 0, last != 0, wbuf, fout, rbuf, g, images != 0,
-                                      edge_xy || z < R6 || z >= nz - R6, cell, oidx, x, y, z);
-                }
+                for (int q = 0; q < 8; ++q) d.val[q] = val[q];
+                double rhs[8];
+                mhd_rhs_assemble<CONDUCT>(d, ks, rhs);
+                finish_cell<MODE>(ks, rhs, val, wcur, first != 0, last != 0, wbuf, fout, rbuf, g, images != 0,
+                                  edge_xy || z < R6 || z >= nz - R6, cell, oidx, x, y, z);
             }
             if (m > 0) {
                 cell += nxy;
@@ -517,10 +515,41 @@ mhd_fx_kernel(const __grid_constant__ MhdMaps maps, const __grid_constant__ FxIn
         }
         return;
     }
-    const u32 n = min(listed, (u32)LIST);  // the loop ended with a barrier
-    for (u32 i = tid; i < n; i += NT) {
-        const int t = (int)(list[i] & (GROUP - 1u)), z = zc0 + (int)(list[i] >> 7);
-        fp64_cell<MODE, CONDUCT>(in, fout, wbuf, rbuf, g, ks, first, last, images, x0 + t % TX, y0 + t / TX, z);
+    // The marked cells by all threads, in lists that the first warp fills (the loop ended with a barrier).
+    const u32 *mark = &marks[0][0];
+    const int words = count * (GROUP / 32);
+    for (int at = 0;;) {
+        if (tid < 32) {
+            u32 n = 0;
+            while (at < words) {  // 32 words at most fill a list
+                u32 bits = at + lane < words ? mark[at + lane] : 0u;
+                const u32 own_n = __popc(bits);
+                u32 upto = own_n;
+#pragma unroll
+                for (int d = 1; d < 32; d *= 2) {
+                    const u32 other = __shfl_up_sync(0xffffffffu, upto, d);
+                    if (lane >= d) upto += other;
+                }
+                const u32 total = __shfl_sync(0xffffffffu, upto, 31);
+                if (n + total > (u32)LIST) break;
+                for (u32 i = n + upto - own_n; bits; bits &= bits - 1, ++i)
+                    list[i] = (uint16_t)((at + lane) * 32 + __ffs((int)bits) - 1);
+                n += total;
+                at += 32;
+            }
+            if (lane == 0) {
+                listed = n;
+                unlisted = at < words;
+            }
+        }
+        __syncthreads();
+        const bool again = unlisted;
+        for (u32 i = tid; i < listed; i += NT) {
+            const int t = (int)(list[i] & (GROUP - 1u)), z = zc0 + (int)(list[i] / GROUP);
+            fp64_cell<MODE, CONDUCT>(in, fout, wbuf, rbuf, g, ks, first, last, images, x0 + t % TX, y0 + t / TX, z);
+        }
+        if (!again) break;
+        __syncthreads();
     }
 }
 
@@ -611,7 +640,7 @@ cudaError_t run(int sub, const MhdMaps &maps, const FxIn &in, const Ptrs8 &fo, d
         ready[dev] = 1;
     }
     const int tx = (int)((g.n[0] + TX - 1) / TX), ty = (int)((g.n[1] + TY - 1) / TY), nz = (int)g.n[2];
-    const int zc = zchunk_len(chunk_planes(tx * ty, nz, start), nz, zmode);
+    const int zc = std::min(zchunk_len(chunk_planes(tx * ty, nz, start), nz, zmode), MAX_PLANES);
     const dim3 grid(tx, ty, (unsigned)((nz + zc - 1) / zc));
     kern<<<grid, NT, SMEM, s>>>(maps, in, fo, w, rhs, g, k, fw, zc, sub == 0 ? 1 : 0, sub == 2 ? 1 : 0, images ? 1 : 0,
                                 err);
