@@ -13,7 +13,7 @@
 //     results in shared memory, so that the FP64 pipe and the integer pipe work at the same time.
 //     160^3, one substep: one thread per cell 5.1 ms, two groups 3.75, four groups 3.1 (128 registers
 //     a thread).  Bound by the latency of dependent instructions at 4 warps per scheduler (128^3: issue
-//     32 %, FP64 pipe 38 %): the ring leaves no shared memory for a second CTA.
+//     34 %, FP64 pipe 39 %): the ring leaves no shared memory for a second CTA.
 //   * One body of code for all fields: unrolled it is 320 KB, and a substep took 24 ms.
 //   * A cell uses, per field, the largest scale of the 7 planes of its window.  Where those
 //     differ (11 % of the windows), values are shifted as they are read, a branch that is uniform per
