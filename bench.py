@@ -55,8 +55,8 @@ SRC_HEAT32 = {"diffusion_f32.cu": "2cacbf4617d874ff", "common.cuh": "3f7458d1c75
 NCU_TRAFFIC = {
     # dram__bytes_read.sum + dram__bytes_write.sum per launch, mean of 3 launches of a 1-pass capture at
     # the bench sizes (profiles/dram_traffic_full_size.md); MHD: the mean over the 3 RK substeps
-    "heat_f64": {"variant": "fx64x16", "zmode": 0, "bytes": 147689301 + 102447019,
-                 "src": {"diffusion_fx.cu": "f11a4d341b8b66a9", "fixed.cuh": "84e7b11e6dde86ee", "common.cuh": "3f7458d1c75ca5f9"}},
+    "heat_f64": {"variant": "fx64x16", "zmode": 0, "bytes": 147750229 + 102371072,
+                 "src": {"diffusion_fx.cu": "2b4f7cb8238067a7", "fixed.cuh": "84e7b11e6dde86ee", "common.cuh": "3f7458d1c75ca5f9"}},
     "heat_f32": {"variant": "f32_by4_ry2_zb2_s8_m3", "zmode": 0, "bytes": 82052181 + 21760939, "src": SRC_HEAT32},
     "heat_f32_512": {"variant": "f32_by8_ry2_zb2_s8_m2", "zmode": 0, "bytes": 586154069 + 507398315,
                      "src": SRC_HEAT32},

@@ -38,7 +38,7 @@
 //     of the exponent range.
 //   * 256^3, r = 3, us per step, the FP64 pipe's kernel and this one: waves 596 and 235; a Gaussian of
 //     8, 16, 32 cells 596 and 696, 672, 290; a front of 3 cells 595 and 531; waves at r = 1, 2, 4 221
-//     and 194, 424 and 215, 821 and 261; 32^3 14.5 and 10.2.  A field of which nothing fits pays for the
+//     and 194, 424 and 215, 821 and 261; 32^3 14.5 and 9.8.  A field of which nothing fits pays for the
 //     exponents and the conversion beside the FP64 pipe's work, at r = 1 up to 1.45 times (221, 321).
 #include <algorithm>
 
@@ -213,7 +213,7 @@ __device__ __forceinline__ int fx_pair(const u64 *cp, const Z &z, int dc, int sc
     return left;
 }
 
-template <int R, bool ISO>
+template <int R, bool ISO, bool LONG>
 __global__ void __launch_bounds__(FxCfg<R>::NT, 1)
 heat_fx_kernel(const __grid_constant__ CUtensorMap map, const double *__restrict__ in, double *__restrict__ out,
                const __grid_constant__ Geom g, const __grid_constant__ FxCoef<R, ISO> c, int zc, int images,
@@ -374,7 +374,7 @@ heat_fx_kernel(const __grid_constant__ CUtensorMap map, const double *__restrict
 
     const bool plain = nv == 2 && (mlo | mhi) == 0;  // both cells, no x image
     const int own = (wy + R) * TXP + Cfg::HX + 2 * lane;
-    const bool early = (wy >> 2) & 1;  // computes before it converts
+    const bool early = LONG && ((wy >> 2) & 1);  // computes before it converts
     // the listed outputs, by all threads
     auto work_off = [&]() {
         for (u32 i = tid; i < min(listed, (u32)Cfg::LIST); i += NT) {
@@ -452,7 +452,9 @@ heat_fx_kernel(const __grid_constant__ CUtensorMap map, const double *__restrict
             }
             optr += pitch_z;
         };
-        if (early) compute();
+        if constexpr (LONG) {
+            if (early) compute();
+        }
         // the plane's scale is complete since the barrier; its slot is read from the next one on
         if (t < nplanes) {
             convert(t);
@@ -477,7 +479,7 @@ heat_fx_kernel(const __grid_constant__ CUtensorMap map, const double *__restrict
         }
         if (!early) compute();
         bad = __syncthreads_or(!ok);
-        if (t % 4 == 3 && !bad) {
+        if (LONG && t % 4 == 3 && !bad) {
             const bool full = listed > (u32)Cfg::LIST_HIGH;
             __syncthreads();  // no thread lists again before all have looked
             if (full) {
@@ -507,18 +509,24 @@ heat_fx_kernel(const __grid_constant__ CUtensorMap map, const double *__restrict
     work_off();  // the loop ended with a barrier
 }
 
+// Chunks of this many planes and more run the LONG body: half of the warps compute first, and the list is
+// worked off before the end.  Its two copies of the computation cost a short kernel their fetching: 32^3
+// (chunks of one plane) 10.2 us a step, without 9.8; 128^3 (15 planes) 39.5 and 39.4; 200 x 150 x 171 (40)
+// 113.6 and 118.9, a Gaussian of 16 cells in 256^3 (37) 672 and 756.
+constexpr int FX_LONG = 12;
 template <int R, bool ISO>
 cudaError_t run(const CUtensorMap *map, const double *in, double *out, const Geom &g, const FxCoef<R, ISO> &c,
                 bool images, unsigned *err, cudaStream_t s, double reread, int zmode) {
     using Cfg = FxCfg<R>;
-    auto k = heat_fx_kernel<R, ISO>;
     static int ready[64] = {};  // per device: the shared-memory limit is raised
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
     if (dev < 0 || dev >= 64) return cudaErrorInvalidDevice;
     if (!ready[dev]) {
-        e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
+        e = cudaFuncSetAttribute(heat_fx_kernel<R, ISO, true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
+        if (e == cudaSuccess)
+            e = cudaFuncSetAttribute(heat_fx_kernel<R, ISO, false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)Cfg::SMEM);
         if (e != cudaSuccess) return e;
         ready[dev] = 1;
     }
@@ -527,6 +535,7 @@ cudaError_t run(const CUtensorMap *map, const double *in, double *out, const Geo
     const int chunks = choose_zchunks(tx * ty, nz, device_sms(), reread);  // one CTA per SM
     const int zc = zchunk_len((nz + chunks - 1) / chunks, nz, zmode);
     dim3 grid(tx, ty, (unsigned)((nz + zc - 1) / zc));
+    const auto k = zc >= FX_LONG ? heat_fx_kernel<R, ISO, true> : heat_fx_kernel<R, ISO, false>;
     return launch_pdl(k, grid, dim3(Cfg::NT), Cfg::SMEM, s, *map, in, out, g, c, zc, images ? 1 : 0, err);
 }
 
